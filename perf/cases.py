@@ -252,10 +252,12 @@ def work(case):
 
 
 def tolerance(case):
-    """Codes, scales and bases are the same bits for every correct implementation, bf16 weights too;
-    fp32 weights may take the quotient of the update to an ulp or two instead of to half an ulp."""
-    if case["call"].startswith("dequant"):
-        return {"rel": 1e-7, "max": 1e-6}
-    if case["params"] != "fp32":
-        return {"rel": 1e-7, "max": 1e-6, "differ": 0.0}
-    return {"rel": 4e-7, "max": 1e-5, "differ": 0.0}
+    """Codes, scales and bases are the same bits for every correct implementation, bf16 weights too.
+    fp32 weights may take the quotient of the update to an ulp or two instead of to half an ulp: two such
+    implementations differed by 1.1e-8 (2-norm) and 2.8e-7 (largest) after three steps.  With the L2 term the
+    weights feed back into the moments: one code in 4e7 then differed, and with it one weight by 2.3e-4."""
+    if case["params"] == "fp32" and case["variant"] == "adam_l2":
+        return {"rel": 1e-6, "max": 0.02, "differ": 1e-6}
+    if case["params"] == "fp32" and not case["call"].startswith("dequant"):
+        return {"rel": 1e-7, "max": 2e-6, "differ": 0.0}
+    return {"rel": 1e-8, "max": 1e-7, "differ": 0.0}
