@@ -787,7 +787,9 @@ int solo_dequant(const solo_state_t* s, int which, float* out_dev, void* stream)
         a.which = 0;
     }
     const int bits = which == 0 ? s->bits_m : s->bits_v;
-    int64_t grid = std::min<int64_t>(s->tiles_total, (int64_t)sm_count(s->device) * 8);
+    // sixteen CTAs of 128 threads fill an SM; shares of at most eight tiles let the SMs end together
+    const int64_t grid = std::min<int64_t>(std::min<int64_t>(s->tiles_total, (int64_t)1 << 30),
+                                           std::max<int64_t>((int64_t)sm_count(s->device) * 16, s->tiles_total / 8));
     cudaError_t e = solo::launch_dequant(bits, a, (unsigned)grid, (cudaStream_t)stream);
     if (e != cudaSuccess) {
         cudaGetLastError();

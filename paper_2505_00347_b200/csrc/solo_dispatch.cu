@@ -79,10 +79,10 @@ int kernel_occupancy(StepKernel k, size_t dyn_smem, int threads) {
 
 cudaError_t launch_dequant(int bits, const DequantArgs& a, unsigned grid, cudaStream_t stream) {
     switch (bits) {
-        case 2: solo_dequant_kernel<2><<<grid, CTA, 0, stream>>>(a); break;
-        case 3: solo_dequant_kernel<3><<<grid, CTA, 0, stream>>>(a); break;
-        case 4: solo_dequant_kernel<4><<<grid, CTA, 0, stream>>>(a); break;
-        case 8: solo_dequant_kernel<8><<<grid, CTA, 0, stream>>>(a); break;
+        case 2: solo_dequant_kernel<2><<<grid, DQ_CTA, 0, stream>>>(a); break;
+        case 3: solo_dequant_kernel<3><<<grid, DQ_CTA, 0, stream>>>(a); break;
+        case 4: solo_dequant_kernel<4><<<grid, DQ_CTA, 0, stream>>>(a); break;
+        case 8: solo_dequant_kernel<8><<<grid, DQ_CTA, 0, stream>>>(a); break;
         default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
