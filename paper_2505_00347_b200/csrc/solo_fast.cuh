@@ -116,6 +116,48 @@ __device__ __forceinline__ float rcp_approx(float x) {
     return y;
 }
 
+// Two binary32 values in a register pair.  The operations round each half like their scalar
+// counterparts (round to nearest, no flush to zero) and take one issue slot for two results: in kernels that
+// are bound by instruction issue with the FMA pipe a quarter busy they halve the cost of the arithmetic.
+struct F2 {
+    unsigned long long v;
+    static __device__ __forceinline__ F2 pack(float l, float h) {
+        F2 r;
+        asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(l), "f"(h));
+        return r;
+    }
+    static __device__ __forceinline__ F2 dup(float x) { return pack(x, x); }
+    static __device__ __forceinline__ F2 load(const char* p) {           // 8-byte aligned shared memory
+        const float2 t = *reinterpret_cast<const float2*>(p);
+        return pack(t.x, t.y);
+    }
+    __device__ __forceinline__ float lo() const {
+        float l, h;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(l), "=f"(h) : "l"(v));
+        return l;
+    }
+    __device__ __forceinline__ float hi() const {
+        float l, h;
+        asm("mov.b64 {%0, %1}, %2;" : "=f"(l), "=f"(h) : "l"(v));
+        return h;
+    }
+};
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+    F2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+    return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+    F2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+    F2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+    return r;
+}
+
 // max(acc, |x|) that returns NaN when x is NaN: a NaN among the block's values makes the block's
 // scale NaN, as the maximum over bit patterns of the general kernel does.
 __device__ __forceinline__ float max_abs_nan(float acc, float x) {

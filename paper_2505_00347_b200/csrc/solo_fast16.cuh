@@ -6,8 +6,10 @@
 // logarithmic levels: no quantile, no draws, nearest level).  (One instantiation for all of them
 // measured 11 % slower on the modes of MODES = 1 than the one that leaves Eq. 5 and the tables out.)
 //
-// Same arithmetic, element for element, as solo_step_fast_kernel (solo_fast.cuh); what changes
-// is the work split.  A CTA of 128 threads owns a tile of 2048 consecutive elements, a thread
+// Same arithmetic, element for element, as solo_step_fast_kernel (solo_fast.cuh), in packed pairs of
+// binary32 (F2): the kernel is bound by instruction issue and a packed operation gives two results per issue
+// slot.  2^27 elements, block 128: 2/3 bit 436 -> 416 us, 4/4 bit 491 -> 455 us, 2/2 bit 429 -> 395 us, with the
+// L2 term 596 -> 508 us.  What changes is the work split.  A CTA of 128 threads owns a tile of 2048 consecutive elements, a thread
 // sixteen of them, a block of 64 / 128 / 256 elements G = 4 / 8 / 16 consecutive lanes, a warp eight,
 // four or two blocks.  The per-thread work that does not depend on the element count (waiting for the
 // staged inputs, addressing, the level tables, the exchange with the first warp, the rounds of the
@@ -41,15 +43,6 @@ namespace solo {
 constexpr int EPT16 = 16;               // elements per thread
 static_assert(CTA16 * EPT16 == TILE, "same tile as the other kernels");
 
-#ifndef SOLO_F16_MIX
-#define SOLO_F16_MIX 1                  // 1: the first moment's codes are computed between the exchanges of the sort
-#endif
-#ifndef SOLO_F16_M3FMA
-#define SOLO_F16_M3FMA 1                // 3-bit first moments: seven saturated multiply-adds instead of a 3-step table search
-#endif
-#ifndef SOLO_F16_M4FMA
-#define SOLO_F16_M4FMA 1                // 4-bit first moments: two levels of three saturated multiply-adds
-#endif
 #ifndef SOLO_F16_CTAS
 #define SOLO_F16_CTAS 7                 // resident CTAs per SM every instantiation is compiled for (72 registers)
 #endif
@@ -65,9 +58,13 @@ struct Fast16Shared {
     // keys, and row 15 holds a sentinel above every key.
     uint32_t sort[ROWS][CTA16];
     // per block: K_v second-moment levels alpha^k Delta_v and K_m first-moment levels y_k Delta_m.
-    // Two arrays, so that the four blocks of a warp occupy distinct banks (up to eight levels).
-    float tab_v[NG][1 << BV];
-    float tab_m[NG][1 << BM];
+    // Two arrays, so that the four blocks of a warp occupy distinct banks (up to eight levels).  2-bit
+    // moments: the sixteen pairs of levels instead, so that one look-up serves two elements; four lanes
+    // per block spend more on building sixteen pairs than they save (2/2 bit at block 64 on 2^27 elements:
+    // 346 us with single levels, 380 us with pairs).
+    static constexpr bool PAIRS = G >= 8;
+    alignas(8) float tab_v[NG][BV == 2 && PAIRS ? 32 : 1 << BV];
+    alignas(8) float tab_m[NG][BM == 2 && PAIRS ? 32 : 1 << BM];
     // Exchange with the first warp.  One copy is enough: xin is written before the tile's first
     // barrier and read between its two barriers, xout is written between the barriers and read
     // after the second, and nobody writes either again before passing those barriers.
@@ -91,15 +88,16 @@ __device__ __forceinline__ void bar_sync16(int id) {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(CTA16) : "memory");
 }
 
-// Byte offsets (4 * code) of sixteen 2-bit codes in one word; see CodeOffsets.
-struct CodeOffsets16x2 {
+// Byte offsets (8 * pair of codes) of the eight pairs among sixteen 2-bit codes in one word, for a table of
+// float pairs; see CodeOffsets.
+struct PairOffsets2 {
     uint32_t even, odd;
-    __device__ __forceinline__ explicit CodeOffsets16x2(uint32_t c) : even(c & 0x33333333u), odd(c & 0xCCCCCCCCu) {}
-    __device__ __forceinline__ uint32_t operator()(int i) const {
-        const uint32_t w = (i & 1) ? odd : even;
+    __device__ __forceinline__ explicit PairOffsets2(uint32_t c) : even(c & 0x0F0F0F0Fu), odd(c & 0xF0F0F0F0u) {}
+    __device__ __forceinline__ uint32_t operator()(int j) const {
+        const uint32_t w = (j & 1) ? odd : even;
         uint32_t top;
-        asm("mul.lo.u32 %0, %1, %2;" : "=r"(top) : "r"(w), "r"(1u << (30 - 2 * i)));
-        return top >> 28;
+        asm("mul.lo.u32 %0, %1, %2;" : "=r"(top) : "r"(w), "r"(1u << (28 - 4 * j)));
+        return top >> 25;
     }
 };
 
@@ -357,7 +355,9 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     }
 
     const typename Shared::Stage& st = s.stage;
-    float mh[EPT16], vh[EPT16];
+    F2 mh[EPT16 / 2], vh[EPT16 / 2];                              // elements 2j, 2j + 1 (in the thread's order)
+    auto mh_at = [&](int i) { return (i & 1) ? mh[i >> 1].hi() : mh[i >> 1].lo(); };
+    auto vh_at = [&](int i) { return (i & 1) ? vh[i >> 1].hi() : vh[i >> 1].lo(); };
     uint32_t mx_v = 0;
     float mx_m_f = 0.0f;
     {
@@ -368,7 +368,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
         const int so = (int)(jb_tile & 3) + grp;
         const float dm = st.sc[0][so], dv = st.sc[1][so], al = st.sc[2][so];
 
-        // per-block level tables (Eq. 2), built by the block's eight lanes
+        // per-block level tables (Eq. 2), built by the block's G lanes
         float* const tab_vf = s.tab_v[grp];
         float* const tab_mf = s.tab_m[grp];
         {
@@ -376,66 +376,81 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
             a2[0] = al;
 #pragma unroll
             for (int i = 1; i < BV; ++i) a2[i] = a2[i - 1] * a2[i - 1];
+            auto level_v = [&](uint32_t k) { return (vtab ? s_yv[k] : pow_sm<BV>(a2, k)) * dv; };
+            if constexpr (BV == 2 && Shared::PAIRS) {
 #pragma unroll
-            for (int r0 = 0; r0 < KV; r0 += G)
-                if (r0 + gl < KV) tab_vf[r0 + gl] = (vtab ? s_yv[r0 + gl] : pow_sm<BV>(a2, (uint32_t)(r0 + gl))) * dv;
+                for (int r0 = 0; r0 < 16; r0 += G)
+                    *reinterpret_cast<float2*>(tab_vf + 2 * (r0 + gl)) = make_float2(level_v((r0 + gl) & 3), level_v((r0 + gl) >> 2));
+            } else {
 #pragma unroll
-            for (int r0 = 0; r0 < KM; r0 += G)
-                if (r0 + gl < KM) tab_mf[r0 + gl] = s_y[r0 + gl] * dm;
+                for (int r0 = 0; r0 < KV; r0 += G)
+                    if (r0 + gl < KV) tab_vf[r0 + gl] = level_v(r0 + gl);
+            }
+            if constexpr (BM == 2 && Shared::PAIRS) {
+#pragma unroll
+                for (int r0 = 0; r0 < 16; r0 += G)
+                    *reinterpret_cast<float2*>(tab_mf + 2 * (r0 + gl)) = make_float2(s_y[(r0 + gl) & 3] * dm, s_y[(r0 + gl) >> 2] * dm);
+            } else {
+#pragma unroll
+                for (int r0 = 0; r0 < KM; r0 += G)
+                    if (r0 + gl < KM) tab_mf[r0 + gl] = s_y[r0 + gl] * dm;
+            }
         }
         __syncwarp();
 
         // Eq. 2, Eq. 3
         const char* const tab_v = reinterpret_cast<const char*>(tab_vf);
         const char* const tab_m = reinterpret_cast<const char*>(tab_mf);
-        const CodeOffsets16x2 om16(cm[0] | (cm[1] << 16));        // used for 2-bit codes only
+        const PairOffsets2 om16(cm[0] | (cm[1] << 16)), ov16(cv[0] | (cv[1] << 16));   // used for 2-bit codes only
         const CodeOffsets<BM> om4a(cm[0], 0u), om4b(cm[1], 0u);
         const CodeOffsets<BV> ov4a(cv[0], 0u), ov4b(cv[1], 0u);
         const unsigned char* const sgb = st.g + 32 * tid;
         const uint4* const sg[2] = {reinterpret_cast<const uint4*>(sgb + 16u * sw),
                                     reinterpret_cast<const uint4*>(sgb + 16u - 16u * sw)};
+        const F2 beta1 = F2::dup(a.beta1), omb1 = F2::dup(a.omb1), beta2 = F2::dup(a.beta2), omb2 = F2::dup(a.omb2);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const uint4 gw = *sg[h];
             const uint32_t gg[4] = {gw.x, gw.y, gw.z, gw.w};
-            float g8[8];
+            F2 g2[4];
 #pragma unroll
-            for (int k = 0; k < 8; ++k)
-                g8[k] = __uint_as_float((k & 1) ? (gg[k >> 1] & 0xffff0000u) : (gg[k >> 1] << 16));
+            for (int k = 0; k < 4; ++k) g2[k] = F2::pack(__uint_as_float(gg[k] << 16), __uint_as_float(gg[k] & 0xffff0000u));
             if (l2) {                                             // Adam: the decay term joins the gradient
-                float p8[8];
+                F2 p2[4];
                 if constexpr (PBF) {
                     const uint4 pw = reinterpret_cast<const uint4*>(st.p)[2 * tid + ((uint32_t)h ^ sw)];
                     const uint32_t pin[4] = {pw.x, pw.y, pw.z, pw.w};
 #pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        p8[2 * k] = __uint_as_float(pin[k] << 16);
-                        p8[2 * k + 1] = __uint_as_float(pin[k] & 0xffff0000u);
-                    }
+                    for (int k = 0; k < 4; ++k) p2[k] = F2::pack(__uint_as_float(pin[k] << 16), __uint_as_float(pin[k] & 0xffff0000u));
                 } else {
                     const float4* const ph = reinterpret_cast<const float4*>(st.p + 64 * tid + 32u * ((uint32_t)h ^ sw));
                     const float4 pa = ph[0], pb = ph[1];
-                    p8[0] = pa.x; p8[1] = pa.y; p8[2] = pa.z; p8[3] = pa.w;
-                    p8[4] = pb.x; p8[5] = pb.y; p8[6] = pb.z; p8[7] = pb.w;
+                    p2[0] = F2::pack(pa.x, pa.y); p2[1] = F2::pack(pa.z, pa.w);
+                    p2[2] = F2::pack(pb.x, pb.y); p2[3] = F2::pack(pb.z, pb.w);
                 }
+                const F2 wd = F2::dup(a.weight_decay);
 #pragma unroll
-                for (int k = 0; k < 8; ++k) g8[k] = __fmaf_rn(a.weight_decay, p8[k], g8[k]);
+                for (int k = 0; k < 4; ++k) g2[k] = fma2(wd, p2[k], g2[k]);
             }
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int i = 8 * h + k;
-                const float gi = g8[k];
-                const float mt = *reinterpret_cast<const float*>(tab_m + (BM == 2 ? om16(i) : i < 8 ? om4a(i) : om4b(i - 8)));
-                const float vt = *reinterpret_cast<const float*>(tab_v + (i < 8 ? ov4a(i) : ov4b(i - 8)));
-                mh[i] = __fmaf_rn(a.beta1, mt, a.omb1 * gi);
+            for (int k = 0; k < 4; ++k) {
+                const int j = 4 * h + k;                          // pair of elements 2j, 2j + 1
+                auto code_m = [&](int i) { return *reinterpret_cast<const float*>(tab_m + (i < 8 ? om4a(i) : om4b(i - 8))); };
+                auto code_v = [&](int i) { return *reinterpret_cast<const float*>(tab_v + (i < 8 ? ov4a(i) : ov4b(i - 8))); };
+                F2 mt, vt;
+                if constexpr (BM == 2 && Shared::PAIRS) mt = F2::load(tab_m + om16(j));
+                else mt = F2::pack(code_m(2 * j), code_m(2 * j + 1));
+                if constexpr (BV == 2 && Shared::PAIRS) vt = F2::load(tab_v + ov16(j));
+                else vt = F2::pack(code_v(2 * j), code_v(2 * j + 1));
+                mh[j] = fma2(beta1, mt, mul2(omb1, g2[k]));
                 if (belief) {                                     // AdaBelief: (g - m^)^2, plus eps
-                    const float sig = gi - mh[i];
-                    vh[i] = __fmaf_rn(a.beta2, vt, a.omb2 * (sig * sig)) + a.eps;
+                    const F2 sig = fma2(mh[j], F2::dup(-1.0f), g2[k]);      // g - m^, one rounding
+                    vh[j] = add2(fma2(beta2, vt, mul2(omb2, mul2(sig, sig))), F2::dup(a.eps));
                 } else {
-                    vh[i] = __fmaf_rn(a.beta2, vt, a.omb2 * (gi * gi));
+                    vh[j] = fma2(beta2, vt, mul2(omb2, mul2(g2[k], g2[k])));
                 }
-                mx_m_f = max_abs_nan(mx_m_f, mh[i]);
-                mx_v = max(mx_v, __float_as_uint(vh[i]));
+                mx_m_f = max_abs_nan(max_abs_nan(mx_m_f, mh[j].lo()), mh[j].hi());
+                mx_v = max(max(mx_v, __float_as_uint(vh[j].lo())), __float_as_uint(vh[j].hi()));
             }
         }
     }
@@ -459,20 +474,23 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
         const float4* const sp[2] = {reinterpret_cast<const float4*>(spb + 32u * sw),
                                      reinterpret_cast<const float4*>(spb + 32u - 32u * sw)};
         float4* const gp[2] = {reinterpret_cast<float4*>(gpb + 32u * sw), reinterpret_cast<float4*>(gpb + 32u - 32u * sw)};
+        const F2 isb = F2::dup(a.inv_sqrt_bc2), eps = F2::dup(a.eps), lr = F2::dup(a.step_size), decay = F2::dup(a.decay);
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             const float4 pv = sp[q >> 1][q & 1];
-            float p[4] = {pv.x, pv.y, pv.z, pv.w};
+            F2 p[2] = {F2::pack(pv.x, pv.y), F2::pack(pv.z, pv.w)};
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const int i = 4 * q + k;
-                const float den = __fmaf_rn(sqrt_approx(vh[i]), a.inv_sqrt_bc2, a.eps);
-                const float rc = rcp_approx(den);
-                const float q0 = mh[i] * rc;
-                const float q1 = __fmaf_rn(__fmaf_rn(-den, q0, mh[i]), rc, q0);
-                p[k] = __fmaf_rn(-a.step_size, q1, DECAY ? p[k] * a.decay : p[k]);
+            for (int k = 0; k < 2; ++k) {
+                const F2 m = mh[2 * q + k], v = vh[2 * q + k];
+                const F2 den = fma2(F2::pack(sqrt_approx(v.lo()), sqrt_approx(v.hi())), isb, eps);
+                // with the negated reciprocal every product has its sign turned, so that the quotient comes
+                // out negated and no operand needs a negation: -q0 = m (-1/den), -q1 = (m - den q0)(-1/den) - q0
+                const F2 nrc = F2::pack(rcp_approx(-den.lo()), rcp_approx(-den.hi()));
+                const F2 nq0 = mul2(m, nrc);
+                const F2 nq1 = fma2(fma2(den, nq0, m), nrc, nq0);
+                p[k] = fma2(lr, nq1, DECAY ? mul2(p[k], decay) : p[k]);
             }
-            __stcs(gp[q >> 1] + (q & 1), make_float4(p[0], p[1], p[2], p[3]));
+            __stcs(gp[q >> 1] + (q & 1), make_float4(p[0].lo(), p[0].hi(), p[1].lo(), p[1].hi()));
         }
     } else {
         const uint4* const sp = reinterpret_cast<const uint4*>(st.p) + 2 * tid;
@@ -490,8 +508,8 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
 #pragma unroll
             for (int k = 0; k < 8; ++k) {
                 const int i = 8 * h + k;
-                const float den = __fmaf_rn(__fsqrt_rn(vh[i]), a.inv_sqrt_bc2, a.eps);
-                p[k] = __fmaf_rn(-a.step_size, __fdiv_rn(mh[i], den), DECAY ? p[k] * a.decay : p[k]);
+                const float den = __fmaf_rn(__fsqrt_rn(vh_at(i)), a.inv_sqrt_bc2, a.eps);
+                p[k] = __fmaf_rn(-a.step_size, __fdiv_rn(mh_at(i), den), DECAY ? p[k] * a.decay : p[k]);
             }
             uint32_t pp[4];
             if (a.param_sr) {
@@ -517,78 +535,73 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     uint32_t om[2] = {0u, 0u};                                    // eight codes per word
     const float dm_new = __uint_as_float(mx_m);
     const float inv_m = __frcp_rn(dm_new);
-    // BM == 2: code = number of midpoints below r, each comparison as the saturation of
-    // (r - mid) * 2^100 on the FMA pipe (exactly 0 or 1, see fast_tile), accumulated in binary32
+    // code = number of midpoints below r, each comparison as the saturation of (r - mid) * 2^100 on the FMA
+    // pipe (exactly 0 or 1, see fast_tile).  The codes of elements 2j and 2j + 1 are accumulated side by side
+    // in one pair of binary32 (eight 2- or 3-bit codes per pair, at most 21 bits each: exact).
     constexpr float BIG = 0x1p100f;
-    const float n0 = -s_mid[0] * BIG, n1 = -s_mid[1] * BIG, n2 = -s_mid[BM == 2 ? 2 : 1] * BIG;
-    constexpr bool M3_FMA = BM == 3 && SOLO_F16_M3FMA;           // 3-bit: all seven comparisons that way (24 bits per word: exact)
+    const float n0 = -s_mid[0] * BIG, n1 = -s_mid[1] * BIG, n2 = -s_mid[2] * BIG;
     float n3[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    if constexpr (M3_FMA) {
+    if constexpr (BM == 3) {
 #pragma unroll
         for (int k = 0; k < 4; ++k) n3[k] = -s_mid[3 + k] * BIG;
     }
     // 4-bit: the same comparisons in two levels of three: mid[3], mid[7], mid[11] give the quarter s of
     // the codebook, the three midpoints inside it come from a table row addressed by s (s_mid4, scaled
-    // like n0..n2); code = 4 s + their count.  Four codes (16 bits) per binary32 accumulator.
-    constexpr bool M4_FMA = BM == 4 && SOLO_F16_M4FMA;
+    // like n0..n2); code = 4 s + their count.  Four codes (12 bits each half) per accumulator.
     float nq[3] = {0.0f, 0.0f, 0.0f};
-    if constexpr (M4_FMA) {
+    if constexpr (BM == 4) {
         nq[0] = -s_mid[3] * BIG; nq[1] = -s_mid[7] * BIG; nq[2] = -s_mid[11] * BIG;
     }
-    float omf4[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    float omf[2] = {0.0f, 0.0f};
-    auto quant_m = [&](int i) {                                   // call with i = 15, 14, ..., 0
-        const float r = mh[i] * inv_m;
-        if constexpr (BM == 2) {
-            float& acc = omf[i >> 3];
-            acc = __fmaf_rn(acc, 4.0f, __saturatef(__fmaf_rn(r, BIG, n0)));
-            acc += __saturatef(__fmaf_rn(r, BIG, n1));
-            acc += __saturatef(__fmaf_rn(r, BIG, n2));
-        } else if constexpr (M3_FMA) {
-            float& acc = omf[i >> 3];
-            acc = __fmaf_rn(acc, 8.0f, __saturatef(__fmaf_rn(r, BIG, n0)));
-            acc += __saturatef(__fmaf_rn(r, BIG, n1));
-            acc += __saturatef(__fmaf_rn(r, BIG, -s_mid[2] * BIG));
+    constexpr int CPA = BM == 4 ? 4 : 8;                          // codes per accumulator
+    F2 omf[EPT16 / CPA];
 #pragma unroll
-            for (int k = 0; k < 4; ++k) acc += __saturatef(__fmaf_rn(r, BIG, n3[k]));
-        } else if constexpr (M4_FMA) {
-            const float c0 = __saturatef(__fmaf_rn(r, BIG, nq[0]));
-            const float c1 = __saturatef(__fmaf_rn(r, BIG, nq[1]));
-            const float c2 = __saturatef(__fmaf_rn(r, BIG, nq[2]));
-            // 2^23 + 16 s: the low bits of the pattern are the byte offset of row s
-            const float t = __fmaf_rn(c2, 16.0f, __fmaf_rn(c1, 16.0f, __fmaf_rn(c0, 16.0f, 8388608.0f)));
-            const float4 row = *reinterpret_cast<const float4*>(reinterpret_cast<const char*>(s_mid4) + (__float_as_uint(t) & 0x30u));
-            const float sq = (c0 + c1) + c2;
-            float code = __fmaf_rn(sq, 4.0f, __saturatef(__fmaf_rn(r, BIG, row.x)));
-            code += __saturatef(__fmaf_rn(r, BIG, row.y));
-            code += __saturatef(__fmaf_rn(r, BIG, row.z));
-            omf4[i >> 2] = __fmaf_rn(omf4[i >> 2], 16.0f, code);
+    for (int k = 0; k < EPT16 / CPA; ++k) omf[k] = F2::dup(0.0f);
+    const F2 inv_m2 = F2::dup(inv_m);
+    auto quant_m = [&](int j) {                                   // call with j = 7, 6, ..., 0
+        const F2 r = mul2(mh[j], inv_m2);
+        F2& acc = omf[2 * j / CPA];
+        const F2 up = F2::dup((float)(KM * KM));
+        auto step = [&](float n) {
+            return F2::pack(__saturatef(__fmaf_rn(r.lo(), BIG, n)), __saturatef(__fmaf_rn(r.hi(), BIG, n)));
+        };
+        if constexpr (BM <= 3) {
+            acc = fma2(acc, up, step(n0));
+            acc = add2(acc, step(n1));
+            acc = add2(acc, step(n2));
+            if constexpr (BM == 3) {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) acc = add2(acc, step(n3[k]));
+            }
         } else {
-            uint32_t q = 0;
-#pragma unroll
-            for (int st2 = KM / 2; st2 >= 1; st2 >>= 1)
-                if (r > s_mid[q + st2 - 1]) q += st2;
-            om[i >> 3] = (om[i >> 3] << BM) + q;
+            const F2 c0 = step(nq[0]), c1 = step(nq[1]), c2 = step(nq[2]);
+            // 2^23 + 16 s: the low bits of the pattern are the byte offset of row s
+            const F2 sq = add2(add2(c0, c1), c2);
+            const F2 t = fma2(sq, F2::dup(16.0f), F2::dup(8388608.0f));
+            auto row_at = [&](float o) {
+                return *reinterpret_cast<const float4*>(reinterpret_cast<const char*>(s_mid4) + (__float_as_uint(o) & 0x30u));
+            };
+            const float4 ra = row_at(t.lo()), rb = row_at(t.hi());
+            auto inner = [&](float na, float nb) {
+                return F2::pack(__saturatef(__fmaf_rn(r.lo(), BIG, na)), __saturatef(__fmaf_rn(r.hi(), BIG, nb)));
+            };
+            acc = fma2(acc, up, fma2(sq, F2::dup(4.0f), inner(ra.x, rb.x)));
+            acc = add2(acc, inner(ra.y, rb.y));
+            acc = add2(acc, inner(ra.z, rb.z));
         }
     };
     auto quant_m_done = [&]() {
-        if constexpr (BM == 2 || M3_FMA) {
-            om[0] = (uint32_t)omf[0];
-            om[1] = (uint32_t)omf[1];
-        }
-        if constexpr (M4_FMA) {
-            om[0] = (uint32_t)omf4[0] | ((uint32_t)omf4[1] << 16);
-            om[1] = (uint32_t)omf4[2] | ((uint32_t)omf4[3] << 16);
+        uint32_t half[EPT16 / CPA];
+#pragma unroll
+        for (int k = 0; k < EPT16 / CPA; ++k) half[k] = (uint32_t)__fmaf_rn(omf[k].hi(), (float)KM, omf[k].lo());
+        if constexpr (BM <= 3) {
+            om[0] = half[0];
+            om[1] = half[1];
+        } else {
+            om[0] = half[0] | (half[1] << 16);
+            om[1] = half[2] | (half[3] << 16);
         }
         if (dm_new < TINY) { om[0] = 0; om[1] = 0; }             // vanishing block: all codes 0
     };
-    if constexpr (!SOLO_F16_MIX) {
-        if (!round_m) {
-#pragma unroll
-            for (int i = EPT16 - 1; i >= 0; --i) quant_m(i);
-            quant_m_done();
-        }
-    }
     if (round_m) {
         // Eq. 5: q = number of levels y_1 .. y_{K-2} that r reaches (the lower end of its bracket), plus
         // one when the element's draw u (Philox purpose 1) falls below (r - y_q) / (y_{q+1} - y_q).
@@ -629,7 +642,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
 #pragma unroll
             for (int e = 1; e >= 0; --e) {
                 const int i = 2 * j + e;
-                const float r = mh[i] * inv_m;
+                const float r = mh_at(i) * inv_m;
                 const float t = r * BIG;
                 float qf;
                 if constexpr (BM == 4) {
@@ -695,12 +708,10 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
         };
         if (fixed_base) {
             // every block keeps the given base: no quantile to find
-            if constexpr (SOLO_F16_MIX) {
-                if (!round_m) {
+            if (!round_m) {
 #pragma unroll
-                    for (int i = EPT16 - 1; i >= 0; --i) quant_m(i);
-                    quant_m_done();
-                }
+                for (int j = EPT16 / 2 - 1; j >= 0; --j) quant_m(j);
+                quant_m_done();
             }
             if (round_v) {
 #pragma unroll
@@ -710,12 +721,12 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
         } else {
             uint32_t key[EPT16];
 #pragma unroll
-            for (int i = 0; i < EPT16; ++i) key[i] = __float_as_uint(vh[i]);
-            if (SOLO_F16_MIX && !round_m) {
+            for (int i = 0; i < EPT16; ++i) key[i] = __float_as_uint(vh_at(i));
+            if (!round_m) {
 #pragma unroll
                 for (int k = 0; k < 62; ++k) {
                     cswap(key[SORT16_PAIRS[k][0]], key[SORT16_PAIRS[k][1]]);
-                    if ((k & 3) == 3 || k == 61) quant_m(15 - (k >> 2));
+                    if ((k & 7) == 7 || k == 61) quant_m(7 - (k >> 3));
                 }
                 quant_m_done();
             } else {
@@ -772,7 +783,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
             float acc[2] = {0.0f, 0.0f};                         // eight codes, at most 24 bits: exact
 #pragma unroll
             for (int i = EPT16 - 1; i >= 0; --i) {
-                const float r = vh[i] * inv;
+                const float r = vh_at(i) * inv;
                 float& c = acc[i >> 3];
                 c = __fmaf_rn(c, (float)KV, __saturatef(__fmaf_rn(r, BIG, na.x)));
                 c += __saturatef(__fmaf_rn(r, BIG, na.y));
@@ -793,7 +804,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
             float acc[4] = {0.0f, 0.0f, 0.0f, 0.0f};            // four codes each
 #pragma unroll
             for (int i = EPT16 - 1; i >= 0; --i) {
-                const float r = vh[i] * inv;
+                const float r = vh_at(i) * inv;
                 const float c0 = __saturatef(__fmaf_rn(r, BIG, nq4.x));
                 const float c1 = __saturatef(__fmaf_rn(r, BIG, nq4.y));
                 const float c2 = __saturatef(__fmaf_rn(r, BIG, nq4.z));
@@ -812,32 +823,35 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
         const float inv = sc.y, il = sc.z, lim = sc.w;
         constexpr float KM1 = (float)(KV - 1);
         constexpr float MAGIC = 12582912.0f;
-        constexpr uint32_t MAGIC_BITS = 0x4B400000u;
         const float ils = il * (1.0f / KM1);
         // xi = (d + 1/2) / 2^16 - 1/2 (exact), scaled like t; zero without the dither
-        const float xs1 = round_v ? (float)(0x1p-16 / (KV - 1)) : 0.0f;
-        const float xs0 = round_v ? (float)((-0.5 + 0x1p-17) / (KV - 1)) : 0.0f;
+        const F2 xs1 = F2::dup(round_v ? (float)(0x1p-16 / (KV - 1)) : 0.0f);
+        const F2 xs0 = F2::dup(round_v ? (float)((-0.5 + 0x1p-17) / (KV - 1)) : 0.0f);
+        const F2 inv2 = F2::dup(inv);
+        // codes of elements 2j and 2j + 1 side by side in one pair of binary32, as for the first moment
+        constexpr int CPA = BV == 4 ? 4 : 8;
         float worst = 0.0f;
-        uint32_t acc[2] = {0u, 0u};
+        F2 acc[EPT16 / CPA];
+#pragma unroll
+        for (int k = 0; k < EPT16 / CPA; ++k) acc[k] = F2::dup(0.0f);
 #pragma unroll
         for (int j = EPT16 / 2 - 1; j >= 0; --j) {
-            float d[2];                                           // the 16-bit draws of elements 2j, 2j + 1 as binary32
-            halves_to_float(w[j], d[0], d[1]);
-#pragma unroll
-            for (int e = 1; e >= 0; --e) {
-                const int i = 2 * j + e;
-                const float r = vh[i] * inv;
-                const float ts = __saturatef(__fmaf_rn(lg2_approx(r), ils, __fmaf_rn(d[e], xs1, xs0)));
-                const float u = __fmaf_rn(ts, KM1, MAGIC);
-                worst = fmaxf(worst, fabsf(__fmaf_rn(ts, KM1, MAGIC - u)));
-                acc[i >> 3] = acc[i >> 3] * (1u << BV) + __float_as_uint(u);
-            }
+            float d0, d1;                                         // the 16-bit draws of elements 2j, 2j + 1 as binary32
+            halves_to_float(w[j], d0, d1);
+            const F2 x = fma2(F2::pack(d0, d1), xs1, xs0);
+            const F2 r = mul2(vh[j], inv2);
+            const F2 ts = F2::pack(__saturatef(__fmaf_rn(lg2_approx(r.lo()), ils, x.lo())),
+                                   __saturatef(__fmaf_rn(lg2_approx(r.hi()), ils, x.hi())));
+            const F2 q = add2(fma2(ts, F2::dup(KM1), F2::dup(MAGIC)), F2::dup(-MAGIC));      // the codes, rounded
+            const F2 off = fma2(ts, F2::dup(-KM1), q);            // their distance from what was rounded
+            worst = fmaxf(fmaxf(worst, fabsf(off.lo())), fabsf(off.hi()));
+            acc[2 * j / CPA] = fma2(acc[2 * j / CPA], F2::dup((float)(KV * KV)), q);
         }
-        uint32_t magic_sum = 0;
+        uint32_t half[EPT16 / CPA];
 #pragma unroll
-        for (int i = 0; i < 8; ++i) magic_sum = (magic_sum << BV) + MAGIC_BITS;
-        ov[0] = acc[0] - magic_sum;
-        ov[1] = acc[1] - magic_sum;
+        for (int k = 0; k < EPT16 / CPA; ++k) half[k] = (uint32_t)__fmaf_rn(acc[k].hi(), (float)KV, acc[k].lo());
+        ov[0] = BV <= 3 ? half[0] : half[0] | (half[1] << 16);
+        ov[1] = BV <= 3 ? half[1] : half[EPT16 / CPA - 2] | (half[EPT16 / CPA - 1] << 16);
         if (__any_sync(0xffffffffu, worst > lim)) {
             // too close to a rounding boundary for the approximate logarithm somewhere in the warp:
             // the exact sequence for all sixteen
@@ -851,7 +865,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
 #pragma unroll
                 for (int e = 1; e >= 0; --e) {
                     const int i = 2 * j + e;
-                    const float r = vh[i] * inv;
+                    const float r = vh_at(i) * inv;
                     uint32_t q = KV - 1;
                     if (!(r < TINY)) {
                         float t = __fmaf_rn(log2_sp(r), il, __fmaf_rn(d[e], x1, x0));
