@@ -293,8 +293,7 @@ float solo_default_beta1(int bits_m, int from_scratch);
  * their full tiles in a kernel with sixteen elements per thread and the remaining tiles in the
  * streamlined kernel, or in the general one where the streamlined kernel does not apply (two
  * launches).  That kernel covers every mode of solo_hyper_t (Eq. 5 rounding and the baseline
- * second-moment codebooks included) as long as the quantile is the p = 0.1 one or none is taken
- * (fixed base, baseline codebook).  1: always the general kernel.  2: like 0 without the
+ * second-moment codebooks included) and every p.  1: always the general kernel.  2: like 0 without the
  * sixteen-per-thread kernel.  3: like 0 with the sixteen-per-thread kernel whatever the tensor
  * sizes.  All produce the same packed state and the same bf16 parameters; the fp32 parameters
  * of the two faster kernels are identical to each other and differ from the IEEE sequence of

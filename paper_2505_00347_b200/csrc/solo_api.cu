@@ -232,11 +232,7 @@ int launch_step(solo_state* s, StepArgs& a, cudaStream_t stream) {
     // worth its second launch only when there is work for many tiles per CTA (measured faster on the
     // 7B-shaped, the GPT-125M-shaped and the ragged set; a 1 Mi-element tensor is launch-bound)
     const bool large = s->tiles_total >= 8192;
-    // p = 0.1: rank 7, 13, 26 of a block of 64, 128, 256
-    const bool rank16 = (s->block == 64 && a.k_full == 7) || (s->block == 128 && a.k_full == 13) ||
-                        (s->block == 256 && a.k_full == 26);
-    // (a fixed base or a baseline codebook needs no quantile, so any p goes with them)
-    if (fast_ok && ((policy == 0 && large) || policy == 3) && (rank16 || a.fixed_alpha > 0.0f || a.tables_v))
+    if (fast_ok && ((policy == 0 && large) || policy == 3))
         k16 = solo::fast16_kernel(s->bits_m, s->bits_v, s->block, a.param_bf16 != 0,
                                   plain ? 0 : (a.tables_v || a.round_m) ? 2 : 1);
     if (k16) {

@@ -38,8 +38,7 @@ StepKernel fast_kernel_bm3(int bv_index, int block, bool param_bf16, bool plain)
 StepKernel fast_kernel_bm4(int bv_index, int block, bool param_bf16, bool plain);
 StepKernel fast_kernel_bm8(int bv_index, int block, bool param_bf16, bool plain);
 StepKernel fast_kernel(int bits_m, int bits_v, int block, bool param_bf16, bool plain);
-// Sixteen elements per thread: 2/3/4-bit states, blocks of 64, 128 or 256, fp32 or bf16 parameters, the
-// quantile rank of p = 0.1 or no quantile (fixed base, baseline codebook); `modes`: 0 as `plain` for
+// Sixteen elements per thread: 2/3/4-bit states, blocks of 64, 128 or 256, fp32 or bf16 parameters; `modes`: 0 as `plain` for
 // fast_kernel, 1 the modes fast_kernel reads at run time, 2 those plus Eq. 5 rounding and the baseline
 // second-moment codebooks; full tiles
 // of aligned tensors only (the rest is left to a launch of the streamlined or of the general kernel with

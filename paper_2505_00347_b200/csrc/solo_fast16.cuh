@@ -1,6 +1,6 @@
 // Sixteen elements per thread: the streamlined step for the plain step (2/3/4-bit states, blocks of
 // 64, 128 or 256, fp32 or bf16 parameters; no L2 term in the gradient, no AdaBelief, base from the
-// p = 0.1 quantile, xi drawn: MODES = 0).  Two more instantiations read other modes from the arguments:
+// p-quantile, xi drawn: MODES = 0).  Two more instantiations read other modes from the arguments:
 // MODES = 1 the L2 term, AdaBelief, a fixed base, no dither; MODES = 2 also stochastic rounding of the
 // first moment (Eq. 5) and the baseline second-moment codebooks (a fixed level table instead of the
 // logarithmic levels: no quantile, no draws, nearest level).  (One instantiation for all of them
@@ -15,8 +15,8 @@
 // staged inputs, addressing, the level tables, the exchange with the first warp, the rounds of the
 // selection) is spent once per sixteen elements instead of once per eight.
 //
-// Resources are cut for seven resident CTAs per SM (28 warps): at most 72 registers per thread
-// and one input stage of 13.6 KB (21.5 KB of shared memory in all).  The stage is read only
+// Resources are cut for seven or eight resident CTAs per SM (ctas16): at most 72 or 64 registers per thread
+// and one input stage of 13.6 KB (15 KB of shared memory in all; 23 KB for blocks of 64).  The stage is read only
 // before the tile's first CTA barrier, so the copies of the CTA's next tile are issued right after
 // that barrier and land while the tile's second half (per-block scalars, random draws,
 // quantization) runs.  Parameters stay in the stage until the update of their four elements needs
@@ -43,20 +43,19 @@ namespace solo {
 constexpr int EPT16 = 16;               // elements per thread
 static_assert(CTA16 * EPT16 == TILE, "same tile as the other kernels");
 
-#ifndef SOLO_F16_CTAS
-#define SOLO_F16_CTAS 7                 // resident CTAs per SM every instantiation is compiled for (72 registers)
-#endif
+// Resident CTAs per SM an instantiation is compiled for: eight (64 registers), seven (72) for 4-bit first moments
+// and for blocks of 256, which spill more at 64 (2^27 elements: 2/3 bit at block 128 380 us at seven, 367 us at
+// eight; 4/4 bit 422 and 421 us; 4/4 bit at block 256 432 and 434 us).
+template <int BM, int G>
+constexpr int ctas16() { return BM == 4 || G == 16 ? 7 : 8; }
 
 // G: lanes per block (4, 8 or 16 for blocks of 64, 128 or 256 elements); NG = 128 / G blocks per tile.
 template <int BM, int BV, bool PBF, int G>
 struct Fast16Shared {
     static constexpr int NG = CTA16 / G;
-    static constexpr int ROUNDS = G == 4 ? 6 : G == 8 ? 12 : 25;   // rank of the p = 0.1 quantile minus one: 7, 13, 26
-    static constexpr int ROWS = ROUNDS < 15 ? ROUNDS : 16;         // G = 16: all fifteen further keys and a sentinel row
-    // Sorted keys of the threads, one column per thread: row j holds the (j+2)-th smallest key.
-    // The rounds of popping read rows 0..ROUNDS-1 at most; with 25 rounds a thread can run out of
-    // keys, and row 15 holds a sentinel above every key.
-    uint32_t sort[ROWS][CTA16];
+    // G = 4: sorted keys of the threads, one column per thread: row j holds the (j+2)-th smallest key, row 15 a
+    // sentinel above every key
+    uint32_t sort[G == 4 ? 16 : 1][G == 4 ? CTA16 : 1];
     // per block: K_v second-moment levels alpha^k Delta_v and K_m first-moment levels y_k Delta_m.
     // Two arrays, so that the four blocks of a warp occupy distinct banks (up to eight levels).  2-bit
     // moments: the sixteen pairs of levels instead, so that one look-up serves two elements; four lanes
@@ -150,27 +149,8 @@ __device__ __forceinline__ void store_codes16(uint8_t* tile_codes, uint32_t* sta
     }
 }
 
-// Sorts sixteen keys so that key[0..12] are the thirteen smallest in ascending order (Batcher's
-// odd-even merge sort without the one exchange that only orders key[13], key[14]).
-__device__ __forceinline__ void sort16_low13(uint32_t (&k)[EPT16]) {
-#define SOLO_CS(a, b) cswap(k[a], k[b])
-    SOLO_CS(0, 1); SOLO_CS(2, 3); SOLO_CS(0, 2); SOLO_CS(1, 3); SOLO_CS(1, 2);
-    SOLO_CS(4, 5); SOLO_CS(6, 7); SOLO_CS(4, 6); SOLO_CS(5, 7); SOLO_CS(5, 6);
-    SOLO_CS(0, 4); SOLO_CS(2, 6); SOLO_CS(2, 4); SOLO_CS(1, 5); SOLO_CS(3, 7); SOLO_CS(3, 5);
-    SOLO_CS(1, 2); SOLO_CS(3, 4); SOLO_CS(5, 6);
-    SOLO_CS(8, 9); SOLO_CS(10, 11); SOLO_CS(8, 10); SOLO_CS(9, 11); SOLO_CS(9, 10);
-    SOLO_CS(12, 13); SOLO_CS(14, 15); SOLO_CS(12, 14); SOLO_CS(13, 15); SOLO_CS(13, 14);
-    SOLO_CS(8, 12); SOLO_CS(10, 14); SOLO_CS(10, 12); SOLO_CS(9, 13); SOLO_CS(11, 15); SOLO_CS(11, 13);
-    SOLO_CS(9, 10); SOLO_CS(11, 12); SOLO_CS(13, 14);
-    SOLO_CS(0, 8); SOLO_CS(4, 12); SOLO_CS(4, 8); SOLO_CS(2, 10); SOLO_CS(6, 14); SOLO_CS(6, 10);
-    SOLO_CS(2, 4); SOLO_CS(6, 8); SOLO_CS(10, 12);
-    SOLO_CS(1, 9); SOLO_CS(5, 13); SOLO_CS(5, 9); SOLO_CS(3, 11); SOLO_CS(7, 15); SOLO_CS(7, 11);
-    SOLO_CS(3, 5); SOLO_CS(7, 9); SOLO_CS(11, 13);
-    SOLO_CS(1, 2); SOLO_CS(3, 4); SOLO_CS(5, 6); SOLO_CS(7, 8); SOLO_CS(9, 10); SOLO_CS(11, 12);
-#undef SOLO_CS
-}
-
-// The same network as a list, for callers that issue other work between its exchanges.
+// Batcher's odd-even merge sort of sixteen keys without the one exchange that only orders key[13], key[14], as a
+// list, so that other work can be issued between its exchanges.
 __device__ constexpr unsigned char SORT16_PAIRS[62][2] = {
     {0, 1}, {2, 3}, {0, 2}, {1, 3}, {1, 2}, {4, 5}, {6, 7}, {4, 6}, {5, 7}, {5, 6},
     {0, 4}, {2, 6}, {2, 4}, {1, 5}, {3, 7}, {3, 5}, {1, 2}, {3, 4}, {5, 6},
@@ -197,36 +177,142 @@ __device__ __forceinline__ uint32_t group_max16(uint32_t x) {
     return x;
 }
 
-// Minimum of the group's keys as each lane holds them.  Groups of sixteen: the two groups of a warp are
-// served by one full-mask minimum and one maximum, the upper group (`hi`) holding its keys complemented
-// (its minimum is the complement of the warp's maximum; keys are 31-bit, so the lower group's keys stay
-// below and the upper group's above 2^31); a lane holds the minimum iff its own value equals the result.
+// Minimum of 31-bit keys over the calling lane's group.  Groups of sixteen: one full-mask minimum and one
+// maximum serve both groups of the warp, the upper group's keys going in complemented (vx = ~0 there, else 0).
 template <int G>
-__device__ __forceinline__ uint32_t group_min16k(uint32_t x, bool hi) {
+__device__ __forceinline__ uint32_t group_min31(uint32_t x, uint32_t vx) {
     if constexpr (G == 16) {
-        const uint32_t lo = __reduce_min_sync(0xffffffffu, x);
-        const uint32_t up = __reduce_max_sync(0xffffffffu, x);
-        return hi ? up : lo;
+        const uint32_t lo = __reduce_min_sync(0xffffffffu, x ^ vx);
+        const uint32_t up = __reduce_max_sync(0xffffffffu, x ^ vx);
+        return (vx ? up : lo) ^ vx;
     } else {
         return group_min16<G>(x);
     }
 }
 
-// One selection round over groups of G lanes, as pop_round in solo_fast.cuh (columns of CTA16 words;
-// keys as they are, or complemented in the upper group of sixteen).  CLAMP: the offset stops at the
-// sentinel row (needed when a thread can be asked for more keys than it has).
-template <int G, bool LAST, bool CLAMP>
-__device__ __forceinline__ uint32_t pop_round16(uint32_t& head, int& off, const uint32_t* col, uint32_t le,
-                                                uint32_t self, bool hi) {
-    const uint32_t tgt = group_min16k<G>(head, hi);
-    if constexpr (LAST) return tgt;
-    const uint32_t nxt = col[off];
-    const uint32_t upto = __ballot_sync(0xffffffffu, head == tgt) & le;
-    // if (upto == self) { head = nxt; off += CTA16; }
-    asm("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, %2, %3;\n\t@p mov.u32 %0, %4;\n\t@p add.s32 %1, %1, %5;\n\t}"
-        : "+r"(head), "+r"(off) : "r"(upto), "r"(self), "r"(nxt), "n"(CTA16));
-    if constexpr (CLAMP) off = min(off, 15 * CTA16);
-    return tgt;
+// How many of the four predicates of each of the group's lanes hold.
+template <int G>
+__device__ __forceinline__ int group_count4(bool p0, bool p1, bool p2, bool p3, int lane) {
+    const uint32_t b0 = __ballot_sync(0xffffffffu, p0), b1 = __ballot_sync(0xffffffffu, p1);
+    const uint32_t b2 = __ballot_sync(0xffffffffu, p2), b3 = __ballot_sync(0xffffffffu, p3);
+    if constexpr (G == 16) {
+        const uint32_t sel = (lane & 16) ? 0x7632u : 0x5410u;
+        return __popc(__byte_perm(b0, b1, sel)) + __popc(__byte_perm(b2, b3, sel));
+    } else {
+        // the byte of each ballot that holds the group (two groups of four)
+        const uint32_t sel = 0x40u + 0x11u * ((uint32_t)lane >> 3);
+        uint32_t b = __byte_perm(__byte_perm(b0, b1, sel), __byte_perm(b2, b3, sel), 0x5410u);
+        if constexpr (G == 4) b &= (lane & 4) ? 0xF0F0F0F0u : 0x0F0F0F0Fu;
+        return __popc(b);
+    }
+}
+
+// The rank-th smallest (1-based) of the values that the G lanes of a group hold, one each: the lanes sort
+// them among themselves (bitonic network over shuffles) and read the lane of that rank.
+template <int G>
+__device__ __forceinline__ uint32_t lanes_rank(uint32_t x, int rank, int lane) {
+#pragma unroll
+    for (int size = 2; size <= G; size <<= 1) {
+#pragma unroll
+        for (int d = size >> 1; d >= 1; d >>= 1) {
+            const uint32_t y = __shfl_xor_sync(0xffffffffu, x, d);
+            const bool upper = ((lane & d) != 0) != (size < G && (lane & size) != 0);      // this lane keeps the larger one
+            x = (y < x) != upper ? y : x;
+        }
+    }
+    return __shfl_sync(0xffffffffu, x, (lane & ~(G - 1)) + rank - 1);
+}
+
+// k-th smallest (1-based, duplicates counted) of the 16 * G keys of a group of G lanes; each lane holds its
+// sixteen as four sorted lists l[q][0..3].  A round: T = the smallest second key among the group's 4 * G
+// lists; every list whose head is at most T drops it.  The n keys dropped are at most every key that stays, so
+// the rank sought becomes k - n.  Of uniformly spread keys a round drops as many as one draws until
+// two fall into the same list (about 7.6 of 32 lists), so rank 13 takes two or three rounds, each serving
+// all groups of the warp, where popping one minimum per round took twelve and needed all sixteen keys
+// of a lane in order (62 exchanges; four lists of four: 20).  When n reaches the rank, the key sought is
+// among the heads: the same rounds follow over the lanes' sorted heads, then the lanes sort one value each.
+// ROUNDS rounds are laid out in line with `side(r)`, independent work of the caller, between them.  Every loop
+// ends: a round drops at least one key (the loops are bounded by k all the same).
+template <int G, int ROUNDS, class Side>
+__device__ __forceinline__ uint32_t select_rank16(uint32_t (&l)[4][4], const int k, const int lane, Side&& side) {
+    const uint32_t vx = G == 16 && (lane & 16) ? 0xFFFFFFFFu : 0u;
+    int rem = k;
+    auto round = [&]() {
+        const uint32_t t = group_min31<G>(min(min(l[0][1], l[1][1]), min(l[2][1], l[3][1])), vx);
+        bool p[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) p[q] = l[q][0] <= t;
+        const int n = group_count4<G>(p[0], p[1], p[2], p[3], lane);
+        const bool go = n < rem;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (p[q] && go) { l[q][0] = l[q][1]; l[q][1] = l[q][2]; l[q][2] = l[q][3]; l[q][3] = KEY_MAX; }
+        if (go) rem -= n;
+        return go;
+    };
+    bool go = true;
+#pragma unroll
+    for (int r = 0; r < ROUNDS; ++r) {
+        go = round();
+        side(r);
+    }
+#pragma unroll 1
+    for (int it = 0; it < k && __any_sync(0xffffffffu, go); ++it) go = round();
+    uint32_t h[4] = {l[0][0], l[1][0], l[2][0], l[3][0]};
+    cswap(h[0], h[1]); cswap(h[2], h[3]); cswap(h[0], h[2]); cswap(h[1], h[3]); cswap(h[1], h[2]);
+    const uint32_t gmask = ((1u << G) - 1u) << (lane & ~(G - 1));
+    auto head_round = [&]() {
+        const uint32_t t = group_min31<G>(h[1], vx);
+        const bool p = h[0] <= t;
+        const int n = __popc(__ballot_sync(0xffffffffu, p) & gmask);
+        go = n < rem;
+        if (p && go) { h[0] = h[1]; h[1] = h[2]; h[2] = h[3]; h[3] = KEY_MAX; }
+        if (go) rem -= n;
+    };
+    head_round();
+    head_round();
+#pragma unroll 1
+    for (int it = 0; it < k && __any_sync(0xffffffffu, go); ++it) head_round();
+    return lanes_rank<G>(h[0], rem, lane);
+}
+
+// Four lanes per block: k-th smallest of the 64 keys, each lane's sixteen sorted, by popping one minimum per round
+// from exactly one lane (the lowest whose head equals it), k - 1 times.  With rank 7 (p = 0.1) six rounds over
+// two-step minima beat the batch rounds of select_rank16, whose lists collide sooner with fewer lanes (2/2 bit,
+// 2^27 elements: 328 us against 370 us).  `col`: the lane's column of Fast16Shared::sort; `side(r)` as above.
+template <class Side>
+__device__ __forceinline__ uint32_t select_pops4(const uint32_t (&key)[EPT16], const int k, uint32_t* const col, const int lane,
+                                                 Side&& side) {
+#pragma unroll
+    for (int j = 1; j < EPT16; ++j) col[(j - 1) * CTA16] = key[j];
+    const uint32_t self = 1u << lane;
+    const uint32_t le = (self | (self - 1u)) & (15u << (lane & ~3));
+    uint32_t head = key[0];
+    int off = 0;
+    auto pop = [&]() {
+        const uint32_t tgt = group_min16<4>(head);
+        const uint32_t nxt = col[off];
+        const uint32_t upto = __ballot_sync(0xffffffffu, head == tgt) & le;
+        // if (upto == self) { head = nxt; off += CTA16; }
+        asm("{\n\t.reg .pred p;\n\tsetp.eq.u32 p, %2, %3;\n\t@p mov.u32 %0, %4;\n\t@p add.s32 %1, %1, %5;\n\t}"
+            : "+r"(head), "+r"(off) : "r"(upto), "r"(self), "r"(nxt), "n"(CTA16));
+    };
+    if (k == 7) {                                                 // p = 0.1
+#pragma unroll
+        for (int r = 0; r < 6; ++r) {
+            pop();
+            side(r);
+        }
+    } else {
+#pragma unroll
+        for (int r = 0; r < 6; ++r) side(r);
+#pragma unroll 1
+        for (int r = 1; r < k; ++r) {
+            pop();
+            off = min(off, 15 * CTA16);                           // (row 15: the sentinel)
+        }
+    }
+    return group_min16<4>(head);
 }
 
 // Bulk copies of one full tile's inputs into the stage (one thread; a bulk copy is a warp-wide
@@ -306,7 +392,6 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
                                             const int tensor, Ahead16& ah, const bool next_full, const int64_t tile_no) {
     using Shared = Fast16Shared<BM, BV, PBF, G>;
     constexpr int KM = 1 << BM, KV = 1 << BV, NG = Shared::NG;    // G lanes per block, NG blocks per tile
-    constexpr int ROUNDS = Shared::ROUNDS;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int gl = tid & (G - 1), grp = tid / G;
     const uint32_t sw = ((uint32_t)tid >> 2) & 1u;               // 1: this thread takes elements 8..15 first (see the top of the file)
@@ -719,42 +804,45 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
             }
             x_p = 0u;
         } else {
-            uint32_t key[EPT16];
+            // the keys are sorted with the first moment's FMA-pipe work issued between the ALU-pipe exchanges
+            if constexpr (G == 4) {
+                uint32_t key[EPT16];
 #pragma unroll
-            for (int i = 0; i < EPT16; ++i) key[i] = __float_as_uint(vh_at(i));
-            if (!round_m) {
+                for (int i = 0; i < EPT16; ++i) key[i] = __float_as_uint(vh_at(i));
 #pragma unroll
                 for (int k = 0; k < 62; ++k) {
                     cswap(key[SORT16_PAIRS[k][0]], key[SORT16_PAIRS[k][1]]);
-                    if ((k & 7) == 7 || k == 61) quant_m(7 - (k >> 3));
+                    if (!round_m && ((k & 7) == 7 || k == 61)) quant_m(7 - (k >> 3));
                 }
-                quant_m_done();
+                cswap(key[13], key[14]);
+                if (!round_m) quant_m_done();
+                x_p = select_pops4(key, a.k_full, &s.sort[0][tid], lane, [&](int r) {
+                    if (round_v) {
+#pragma unroll
+                        for (int q = r * 10 / 6; q < (r + 1) * 10 / 6; ++q) philox_round(q);
+                    }
+                });
             } else {
-                sort16_low13(key);
-            }
-            if constexpr (ROUNDS > 12) cswap(key[13], key[14]); // all sixteen in order
-            uint32_t* const col = &s.sort[0][tid];
-            constexpr int KEPT = ROUNDS < 15 ? ROUNDS : 15;       // keys after the smallest that can be asked for
-            // (upper group of sixteen lanes: complemented, see group_min16k)
-            const bool hi = G == 16 && (lane & 16);
-            const uint32_t vx = hi ? 0xFFFFFFFFu : 0u;
+                uint32_t l[4][4];
 #pragma unroll
-            for (int j = 1; j <= KEPT; ++j) col[(j - 1) * CTA16] = key[j] ^ vx;
-            // ROUNDS rounds pop the ROUNDS smallest keys of the block, the next minimum is x_p
-            const uint32_t self = 1u << lane;
-            const uint32_t le = (self | (self - 1u)) & ((G == 32 ? 0xFFFFFFFFu : ((1u << G) - 1u)) << (lane & ~(G - 1)));
-            uint32_t head = key[0] ^ vx;
-            int off = 0;
+                for (int i = 0; i < EPT16; ++i) l[i >> 2][i & 3] = __float_as_uint(vh_at(i));
 #pragma unroll
-            for (int r = 0; r < ROUNDS; ++r) {
-                pop_round16<G, false, (ROUNDS > 15)>(head, off, col, le, self, hi);
-                if (r < 10 && round_v) philox_round(r);
-            }
-            if (round_v) {
+                for (int q = 0; q < 4; ++q) {
+                    cswap(l[q][0], l[q][1]); cswap(l[q][2], l[q][3]);
+                    if (!round_m) quant_m(7 - 2 * q);
+                    cswap(l[q][0], l[q][2]); cswap(l[q][1], l[q][3]);
+                    if (!round_m) quant_m(6 - 2 * q);
+                    cswap(l[q][1], l[q][2]);
+                }
+                if (!round_m) quant_m_done();
+                constexpr int ROUNDS = G == 16 ? 3 : 2;
+                x_p = select_rank16<G, ROUNDS>(l, a.k_full, lane, [&](int r) {
+                    if (round_v) {
 #pragma unroll
-                for (int r = ROUNDS; r < 10; ++r) philox_round(r);
+                        for (int q = r * 10 / ROUNDS; q < (r + 1) * 10 / ROUNDS; ++q) philox_round(q);
+                    }
+                });
             }
-            x_p = pop_round16<G, true, false>(head, off, col, le, self, hi) ^ vx;
         }
 #pragma unroll
         for (int i = 0; i < 4; ++i) { w[i] = ca[i]; w[4 + i] = cb[i]; }
@@ -887,7 +975,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
 }
 
 template <int BM, int BV, bool PBF, int G, int MODES>
-__global__ void __launch_bounds__(CTA16, SOLO_F16_CTAS) solo_step_fast16_kernel(const StepArgs a) {
+__global__ void __launch_bounds__(CTA16, ctas16<BM, G>()) solo_step_fast16_kernel(const StepArgs a) {
     constexpr int KM = 1 << BM;
     constexpr bool EXT = MODES == 2;
     using Shared = Fast16Shared<BM, BV, PBF, G>;
@@ -955,8 +1043,7 @@ __global__ void __launch_bounds__(CTA16, SOLO_F16_CTAS) solo_step_fast16_kernel(
                                         -midv[4 * (tid - 4) + 2] * 0x1p100f, 0.0f);
         }
     }
-    // (never overwritten: rows 0..14 hold keys; complemented for the upper group of sixteen lanes)
-    if constexpr (Shared::ROWS == 16) s.sort[15][tid] = (G == 16 && (tid & 16)) ? ~KEY_MAX : KEY_MAX;
+    if constexpr (G == 4) s.sort[15][tid] = KEY_MAX;              // never overwritten
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s.mbar)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
