@@ -40,6 +40,7 @@ struct StepArgs {
     int32_t num_tensors;
     int64_t total_tiles;               // the launch covers tiles [tile_first, total_tiles)
     int64_t tile_first;
+    int32_t share;                     // sixteen-per-thread kernel: tiles of one CTA
     int32_t only_partial;              // streamlined and general kernel: skip full tiles of aligned tensors (another launch did them)
     int64_t debug_stall_tile_p1;       // test hook of the staged kernels: 1 + the number of the tile whose input copy
                                        // announces 16 bytes more than it brings (the wait for it runs out); 0: none

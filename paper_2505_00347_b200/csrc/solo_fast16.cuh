@@ -80,7 +80,25 @@ struct Fast16Shared {
         float sc[3][NG + 4];             // Delta_m, Delta_v, alpha of the tile's blocks, from a 16-byte boundary
     };
     alignas(16) Stage stage;
-    alignas(8) unsigned long long mbar;
+    alignas(8) unsigned long long mbar;      // the stage's copies
+    // The CTA's walk over the tiles (see produce_tile16): kept here and not in registers, because one thread uses it
+    alignas(8) unsigned long long mbar_steal;
+    alignas(16) uint4 steal;                 // answer of the last request for another CTA's tiles
+    struct Walk {
+        char* p;                             // tensor: its parameters, gradients, first block
+        const char* g;
+        int64_t jb0;
+        int tensor, t_lo, t_hi, full_tiles;  // tensor: tiles [t_lo, t_hi), the first full_tiles of them full
+        int tile, tile_end;                  // last tile handed out; end of the tiles taken
+        uint32_t phase;                      // parity of mbar_steal's next phase
+    } walk;
+    struct Desc {
+        char* p;                             // the tile's parameters, gradients, first block
+        const char* g;
+        int64_t jb;
+        int tensor, tin, tile, valid;        // valid 0: no tile left
+    };
+    alignas(8) Desc desc[2];                 // written for the next tile between the two barriers of this one
 };
 
 __device__ __forceinline__ void bar_sync16(int id) {
@@ -231,10 +249,10 @@ __device__ __forceinline__ uint32_t lanes_rank(uint32_t x, int rank, int lane) {
 // all groups of the warp, where popping one minimum per round took twelve and needed all sixteen keys
 // of a lane in order (62 exchanges; four lists of four: 20).  When n reaches the rank, the key sought is
 // among the heads: the same rounds follow over the lanes' sorted heads, then the lanes sort one value each.
-// ROUNDS rounds are laid out in line with `side(r)`, independent work of the caller, between them.  Every loop
-// ends: a round drops at least one key (the loops are bounded by k all the same).
-template <int G, int ROUNDS, class Side>
-__device__ __forceinline__ uint32_t select_rank16(uint32_t (&l)[4][4], const int k, const int lane, Side&& side) {
+// ROUNDS rounds are laid out in line, the others loop.  Every loop ends: a round drops at least one key (the
+// loops are bounded by k all the same).
+template <int G, int ROUNDS>
+__device__ __forceinline__ uint32_t select_rank16(uint32_t (&l)[4][4], const int k, const int lane) {
     const uint32_t vx = G == 16 && (lane & 16) ? 0xFFFFFFFFu : 0u;
     int rem = k;
     auto round = [&]() {
@@ -252,10 +270,7 @@ __device__ __forceinline__ uint32_t select_rank16(uint32_t (&l)[4][4], const int
     };
     bool go = true;
 #pragma unroll
-    for (int r = 0; r < ROUNDS; ++r) {
-        go = round();
-        side(r);
-    }
+    for (int r = 0; r < ROUNDS; ++r) go = round();
 #pragma unroll 1
     for (int it = 0; it < k && __any_sync(0xffffffffu, go); ++it) go = round();
     uint32_t h[4] = {l[0][0], l[1][0], l[2][0], l[3][0]};
@@ -279,10 +294,8 @@ __device__ __forceinline__ uint32_t select_rank16(uint32_t (&l)[4][4], const int
 // Four lanes per block: k-th smallest of the 64 keys, each lane's sixteen sorted, by popping one minimum per round
 // from exactly one lane (the lowest whose head equals it), k - 1 times.  With rank 7 (p = 0.1) six rounds over
 // two-step minima beat the batch rounds of select_rank16, whose lists collide sooner with fewer lanes (2/2 bit,
-// 2^27 elements: 328 us against 370 us).  `col`: the lane's column of Fast16Shared::sort; `side(r)` as above.
-template <class Side>
-__device__ __forceinline__ uint32_t select_pops4(const uint32_t (&key)[EPT16], const int k, uint32_t* const col, const int lane,
-                                                 Side&& side) {
+// 2^27 elements: 328 us against 370 us).  `col`: the lane's column of Fast16Shared::sort.
+__device__ __forceinline__ uint32_t select_pops4(const uint32_t (&key)[EPT16], const int k, uint32_t* const col, const int lane) {
 #pragma unroll
     for (int j = 1; j < EPT16; ++j) col[(j - 1) * CTA16] = key[j];
     const uint32_t self = 1u << lane;
@@ -299,13 +312,8 @@ __device__ __forceinline__ uint32_t select_pops4(const uint32_t (&key)[EPT16], c
     };
     if (k == 7) {                                                 // p = 0.1
 #pragma unroll
-        for (int r = 0; r < 6; ++r) {
-            pop();
-            side(r);
-        }
+        for (int r = 0; r < 6; ++r) pop();
     } else {
-#pragma unroll
-        for (int r = 0; r < 6; ++r) side(r);
 #pragma unroll 1
         for (int r = 1; r < k; ++r) {
             pop();
@@ -344,12 +352,94 @@ __device__ __forceinline__ void issue_tile_copy16(const StepArgs& a, Fast16Share
     bulk_copy(st.sc[2], a.alpha + j0, bytes_s, bar);
 }
 
-// What a CTA carries from one full tile to the next.
-struct Ahead16 {
-    uint32_t fill = 0;        // number of the next copy to wait for (uniform over the CTA); its parity is the phase
-    bool staged = false;      // that copy has already been issued (uniform)
-    bool failed = false;      // this thread once waited in vain for a copy: it waits no longer and stores nothing
-};
+// Asks the hardware for the tiles of a CTA of this grid that has not started yet: that CTA is cancelled and its
+// number written to s.steal, or the answer says that none is left.  One thread; at most one request in flight.
+template <class Shared>
+__device__ __forceinline__ void steal_request(Shared& s) {
+    const uint32_t bar = smem_u32(&s.mbar_steal);
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");         // the last answer has been read
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], 16;" ::"r"(bar) : "memory");
+    asm volatile("clusterlaunchcontrol.try_cancel.async.shared::cta.mbarrier::complete_tx::bytes.b128 [%0], [%1];"
+                 ::"r"(smem_u32(&s.steal)), "r"(bar) : "memory");
+}
+// The answer: the number of the CTA whose tiles are ours now, or -1.
+template <class Shared>
+__device__ __forceinline__ int steal_answer(Shared& s, int* status) {
+    if (!mbar_wait(smem_u32(&s.mbar_steal), s.walk.phase)) {
+        atomicOr(status, 2);                                            // (its tiles, if it was cancelled, are not stepped)
+        return -1;
+    }
+    s.walk.phase ^= 1u;
+    int cta;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .b128 h;\n\tld.shared.b128 h, [%1];\n\t"
+        "clusterlaunchcontrol.query_cancel.is_canceled.pred.b128 p, h;\n\tmov.b32 %0, -1;\n\t"
+        "@p clusterlaunchcontrol.query_cancel.get_first_ctaid::x.b32.b128 %0, h;\n\t}"
+        : "=r"(cta) : "r"(smem_u32(&s.steal)) : "memory");
+    return cta;
+}
+
+// Finds the CTA's next full tile, issues the copies of its inputs and describes it in `d` (one thread).
+// A CTA owns a.share consecutive tiles of the launch; when they are done it takes over those of a CTA that
+// has not started (requested when it began on its own, so the answer is there), until none is left.  The SMs
+// so end together whatever their speed, a CTA sets up once for many shares, and inputs are copied ahead across
+// tensors and shares.  One share per resident CTA (a static walk) left 5 % of the SM cycles idle at the launch's
+// end and SMs with fewer CTAs before it: LLaMA layers 2357 -> 2170 us, GPT-125M-shaped set 432 -> 390 us, ragged set
+// 3418 -> 3200 us, 2^24 elements 60 -> 55 us.
+template <int BM, int BV, bool PBF, int G>
+__device__ __forceinline__ void produce_tile16(const StepArgs& a, Fast16Shared<BM, BV, PBF, G>& s, typename Fast16Shared<BM, BV, PBF, G>::Desc& d) {
+    constexpr int NG = CTA16 / G, PSZ = PBF ? 2 : 4;
+    typename Fast16Shared<BM, BV, PBF, G>::Walk& w = s.walk;
+    int tile = w.tile, tile_end = w.tile_end;
+    for (;;) {
+        if (++tile >= tile_end) {
+            const int cta = steal_answer(s, a.status);
+            if (cta < 0) {
+                d.valid = 0;
+                return;
+            }
+            steal_request(s);
+            tile = (int)a.tile_first + cta * a.share;
+            tile_end = (int)min((int64_t)tile + a.share, a.total_tiles);
+            w.tile_end = tile_end;
+            if (tile < w.t_lo || tile >= w.t_hi) {
+                w.tensor = (a.num_tensors > 1 ? find_tensor(a.tile_start, a.num_tensors, tile) : 0) - 1;
+                w.t_hi = tile;
+            }
+        }
+        if (tile >= w.t_hi) {
+            int tensor = w.tensor, t_hi;
+            do {
+                ++tensor;
+                t_hi = (int)__ldg(a.tile_start + tensor + 1);
+            } while (tile >= t_hi);
+            const int64_t n = __ldg(a.numel + tensor);
+            char* const pb = (char*)(a.param_list ? a.param_list[tensor] : a.param_single);
+            const char* const gb = (const char*)(a.grad_list ? a.grad_list[tensor] : a.grad_single);
+            const bool aligned = ((((uintptr_t)pb) | ((uintptr_t)gb)) & 15u) == 0;
+            const bool skip = a.numel_check != nullptr && __ldg(a.numel_check + tensor) != n;   // reported by the other launch
+            w.tensor = tensor;
+            w.t_lo = (int)__ldg(a.tile_start + tensor);
+            w.t_hi = t_hi;
+            w.full_tiles = aligned && !skip ? (int)(n / TILE) : 0;
+            w.jb0 = __ldg(a.block_start + tensor);
+            w.p = pb;
+            w.g = gb;
+        }
+        if (tile - w.t_lo < w.full_tiles) break;
+        tile = min(w.t_hi, tile_end) - 1;                                // the rest of the tensor is left to the other launch
+    }
+    w.tile = tile;
+    const int tin = tile - w.t_lo;
+    d.p = w.p + (int64_t)tin * (TILE * PSZ);
+    d.g = w.g + (int64_t)tin * (TILE * 2);
+    d.jb = w.jb0 + (int64_t)tin * NG;
+    d.tensor = w.tensor;
+    d.tin = tin;
+    d.tile = tile;
+    d.valid = 1;
+    issue_tile_copy16<BM, BV, PBF, G>(a, s, d.p, d.g, d.jb, tile + 1 == a.debug_stall_tile_p1 ? 16u : 0u);
+}
 
 // Per-block scalars of the tile's sixteen blocks (one block per calling thread, tid = 0..15), from
 // what the blocks' lanes left in xin: stores Delta_m', Delta_v', alpha' of the blocks whose warp did not
@@ -381,15 +471,13 @@ __device__ __forceinline__ void block_scalars16(const StepArgs& a, Shared& s, co
 // Order of the work, chosen so that at most the two moments and the sort keys (48 registers) are
 // live at once: (A) inputs, Eq. 2-3; (B) the parameter update, parameters read from the stage four
 // at a time; (C) the first moment's scale and codes (each thread divides for itself: the scale is
-// known to all eight lanes after the maximum); (D) the sort and the selection rounds, with the Philox
-// rounds of the thread's two blocks of draws issued between them (they depend on nothing); (E) the
-// exchange with the first warp, the second moment's codes, the stores.
+// known to all eight lanes after the maximum); (D) the sorted lists and the selection rounds; (E) the
+// exchange with the first warp, the thread's two Philox blocks meanwhile, the second moment's codes, the stores.
 template <int BM, int BV, bool PBF, int G, bool DECAY, int MODES>
 __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, BV, PBF, G>& s, const float* s_y, const float* s_mid,
                                             const float4* s_mid4, const float* s_yv, const float4* s_nv,
                                             const float2* s_yg, const float4* s_br,
-                                            char* pbase, const char* gbase, const int tin, const int64_t jb_tile,
-                                            const int tensor, Ahead16& ah, const bool next_full, const int64_t tile_no) {
+                                            const uint32_t fill, bool& failed) {
     using Shared = Fast16Shared<BM, BV, PBF, G>;
     constexpr int KM = 1 << BM, KV = 1 << BV, NG = Shared::NG;    // G lanes per block, NG blocks per tile
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -406,34 +494,25 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     const bool round_v = PLAIN || (a.round_v && !vtab);
     const bool round_m = EXT && a.round_m;                     // Eq. 5 instead of Eq. 1 for the first moment
 
-    const int64_t tile_elem0 = (int64_t)tin * TILE;
     constexpr int PSZ = PBF ? 2 : 4;                              // bytes per parameter
-    char* const pt = pbase + tile_elem0 * PSZ;
-    const char* const gt = gbase + tile_elem0 * 2;
+    const typename Shared::Desc& desc = s.desc[fill & 1u];
+    char* const pt = desc.p;
+    const int64_t jb_tile = desc.jb;
 
     // ---- (A) inputs from the stage ----
     // Copy number f completes phase f of the stage's mbarrier (parity f & 1).  The copy for this tile
-    // was issued after the first barrier of the tile before it (ah.staged), or is issued now (the
-    // CTA's first full tile, or the first after a tensor change or a tile that was not full): every
-    // thread has passed both barriers of the last tile that used the stage, so nobody reads it still.
-    if (!ah.staged && tid == 0)
-        issue_tile_copy16<BM, BV, PBF, G>(a, s, pt, gt, jb_tile, tile_no + 1 == a.debug_stall_tile_p1 ? 16u : 0u);
-    const uint32_t mine = ah.fill;
-    ah.fill += 1u;
-    ah.staged = next_full;
-    if (!mbar_wait(smem_u32(&s.mbar), mine & 1u, ah.failed ? 1 : MBAR_POLLS)) {
-        if (!ah.failed) atomicOr(a.status, 2);
-        ah.failed = true;
+    // was issued after the first barrier of the tile before it (every thread had read the stage by then).
+    if (!mbar_wait(smem_u32(&s.mbar), fill & 1u, failed ? 1 : MBAR_POLLS)) {
+        if (!failed) atomicOr(a.status, 2);
+        failed = true;
     }
-    // A warp in which any lane gave up leaves the tile alone: it stores nothing, flags its four blocks
+    // A warp in which any lane gave up leaves the tile alone: it stores nothing, flags its blocks
     // for the first warp (which stores the per-block scalars), and only keeps the CTA's barriers, the
     // copy-ahead and, if it is the first warp, the other warps' scalars going.
-    if (__any_sync(0xffffffffu, ah.failed)) {
+    if (__any_sync(0xffffffffu, failed)) {
         if (gl == 0) s.xin[grp] = make_uint4(0u, 0u, 0u, 1u);
         bar_sync16(1);
-        if (next_full && tid == 32)
-            issue_tile_copy16<BM, BV, PBF, G>(a, s, pt + TILE * PSZ, gt + TILE * 2, jb_tile + NG,
-                                           tile_no + 2 == a.debug_stall_tile_p1 ? 16u : 0u);
+        if (tid == 32) produce_tile16<BM, BV, PBF, G>(a, s, s.desc[(fill + 1u) & 1u]);
         if (tid < NG) block_scalars16<KV>(a, s, jb_tile, tid, fixed_base, vtab);
         bar_sync16(2);
         return;
@@ -546,8 +625,8 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     // position of the thread's first element in the tensor's random stream (element index / 8): even,
     // so the second group of eight never carries into the high word
     auto stream_position = [&](uint32_t& lo, uint32_t& hi, uint32_t& c3) {
-        const Origin org = origin_of(a, tensor);
-        const uint64_t ctr = org.ctr0 + (uint64_t)((uint32_t)tin * (TILE / 8) + 2u * (uint32_t)tid);
+        const Origin org = origin_of(a, desc.tensor);
+        const uint64_t ctr = org.ctr0 + (uint64_t)((uint32_t)desc.tin * (TILE / 8) + 2u * (uint32_t)tid);
         lo = (uint32_t)ctr;
         hi = (uint32_t)(ctr >> 32);
         c3 = org.stream * 4u;
@@ -766,96 +845,69 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
         if (dm_new < TINY) { om[0] = 0; om[1] = 0; }             // vanishing block: all codes 0
     }
 
-    // ---- (D) second moment: block scale and the p-quantile (k = 13 of 128); the draws of Eq. 6 ----
+    // ---- (D) second moment: block scale and the p-quantile ----
     mx_v = group_max16<G>(mx_v);
     uint32_t x_p;
-    uint32_t w[8];                                                // 16 halfwords: the draws of the 16 elements
-    {
-        // Philox4x32-10 on the counters of the thread's two groups of eight elements,
-        // (ctr, step, 4 * stream) and (ctr + 1, ...), in the thread's order; one round of both per call
-        uint32_t ctr_lo, ctr_hi, c3;
-        stream_position(ctr_lo, ctr_hi, c3);
-        uint32_t ca[4] = {ctr_lo + sw, ctr_hi, a.step32, c3};
-        uint32_t cb[4] = {ctr_lo + (sw ^ 1u), ctr_hi, a.step32, c3};
-        auto philox_round = [&](int r) {
+    uint32_t w[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};             // 16 halfwords: the draws of the 16 elements
+    if (fixed_base) {
+        // every block keeps the given base: no quantile to find
+        if (!round_m) {
 #pragma unroll
-            for (int b = 0; b < 2; ++b) {
-                uint32_t(&c)[4] = b ? cb : ca;
-                const uint64_t p0 = (uint64_t)0xD2511F53u * c[0];
-                const uint64_t p1 = (uint64_t)0xCD9E8D57u * c[2];
-                const uint32_t n0 = (uint32_t)(p1 >> 32) ^ c[1] ^ a.rk[2 * r];
-                const uint32_t n2 = (uint32_t)(p0 >> 32) ^ c[3] ^ a.rk[2 * r + 1];
-                c[1] = (uint32_t)p1;
-                c[3] = (uint32_t)p0;
-                c[0] = n0;
-                c[2] = n2;
-            }
-        };
-        if (fixed_base) {
-            // every block keeps the given base: no quantile to find
-            if (!round_m) {
-#pragma unroll
-                for (int j = EPT16 / 2 - 1; j >= 0; --j) quant_m(j);
-                quant_m_done();
-            }
-            if (round_v) {
-#pragma unroll
-                for (int r = 0; r < 10; ++r) philox_round(r);
-            }
-            x_p = 0u;
-        } else {
-            // the keys are sorted with the first moment's FMA-pipe work issued between the ALU-pipe exchanges
-            if constexpr (G == 4) {
-                uint32_t key[EPT16];
-#pragma unroll
-                for (int i = 0; i < EPT16; ++i) key[i] = __float_as_uint(vh_at(i));
-#pragma unroll
-                for (int k = 0; k < 62; ++k) {
-                    cswap(key[SORT16_PAIRS[k][0]], key[SORT16_PAIRS[k][1]]);
-                    if (!round_m && ((k & 7) == 7 || k == 61)) quant_m(7 - (k >> 3));
-                }
-                cswap(key[13], key[14]);
-                if (!round_m) quant_m_done();
-                x_p = select_pops4(key, a.k_full, &s.sort[0][tid], lane, [&](int r) {
-                    if (round_v) {
-#pragma unroll
-                        for (int q = r * 10 / 6; q < (r + 1) * 10 / 6; ++q) philox_round(q);
-                    }
-                });
-            } else {
-                uint32_t l[4][4];
-#pragma unroll
-                for (int i = 0; i < EPT16; ++i) l[i >> 2][i & 3] = __float_as_uint(vh_at(i));
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    cswap(l[q][0], l[q][1]); cswap(l[q][2], l[q][3]);
-                    if (!round_m) quant_m(7 - 2 * q);
-                    cswap(l[q][0], l[q][2]); cswap(l[q][1], l[q][3]);
-                    if (!round_m) quant_m(6 - 2 * q);
-                    cswap(l[q][1], l[q][2]);
-                }
-                if (!round_m) quant_m_done();
-                constexpr int ROUNDS = G == 16 ? 3 : 2;
-                x_p = select_rank16<G, ROUNDS>(l, a.k_full, lane, [&](int r) {
-                    if (round_v) {
-#pragma unroll
-                        for (int q = r * 10 / ROUNDS; q < (r + 1) * 10 / ROUNDS; ++q) philox_round(q);
-                    }
-                });
-            }
+            for (int j = EPT16 / 2 - 1; j >= 0; --j) quant_m(j);
+            quant_m_done();
         }
+        x_p = 0u;
+    } else {
+        // the keys are sorted with the first moment's FMA-pipe work issued between the ALU-pipe exchanges
+        if constexpr (G == 4) {
+            uint32_t key[EPT16];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) { w[i] = ca[i]; w[4 + i] = cb[i]; }
+            for (int i = 0; i < EPT16; ++i) key[i] = __float_as_uint(vh_at(i));
+#pragma unroll
+            for (int k = 0; k < 62; ++k) {
+                cswap(key[SORT16_PAIRS[k][0]], key[SORT16_PAIRS[k][1]]);
+                if (!round_m && ((k & 7) == 7 || k == 61)) quant_m(7 - (k >> 3));
+            }
+            cswap(key[13], key[14]);
+            if (!round_m) quant_m_done();
+            x_p = select_pops4(key, a.k_full, &s.sort[0][tid], lane);
+        } else {
+            uint32_t l[4][4];
+#pragma unroll
+            for (int i = 0; i < EPT16; ++i) l[i >> 2][i & 3] = __float_as_uint(vh_at(i));
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                cswap(l[q][0], l[q][1]); cswap(l[q][2], l[q][3]);
+                if (!round_m) quant_m(7 - 2 * q);
+                cswap(l[q][0], l[q][2]); cswap(l[q][1], l[q][3]);
+                if (!round_m) quant_m(6 - 2 * q);
+                cswap(l[q][1], l[q][2]);
+            }
+            if (!round_m) quant_m_done();
+            x_p = select_rank16<G, G == 16 ? 3 : 2>(l, a.k_full, lane);
+        }
     }
 
     // ---- (E) per-block scalars by the first warp; the next tile's copies start meanwhile ----
     if (gl == 0) s.xin[grp] = make_uint4(mx_m, mx_v, x_p, 0u);
     bar_sync16(1);
     // every thread has read what it needs from the stage
-    if (next_full && tid == 32)
-        issue_tile_copy16<BM, BV, PBF, G>(a, s, pt + TILE * PSZ, gt + TILE * 2, jb_tile + NG,
-                                       tile_no + 2 == a.debug_stall_tile_p1 ? 16u : 0u);
+    if (tid == 32) produce_tile16<BM, BV, PBF, G>(a, s, s.desc[(fill + 1u) & 1u]);
     if (tid < NG) block_scalars16<KV>(a, s, jb_tile, tid, fixed_base, vtab);
+    // meanwhile every thread draws: Philox4x32-10 on the counters of its two groups of eight elements,
+    // (ctr, step, 4 * stream) and (ctr + 1, ...), in its own order.  (Between the selection's rounds, where the draws
+    // once hid the shuffles' latency, they gain nothing with 28 to 32 resident warps; here they fill the wait for
+    // the first warp: bf16 parameters 536 -> 528 us, 4/4 bit 407 -> 402 us on 2^27 elements.)
+    if (round_v) {
+        uint32_t ctr_lo, ctr_hi, c3, w4[4];
+        stream_position(ctr_lo, ctr_hi, c3);
+        philox_rk(ctr_lo + sw, ctr_hi, a.step32, c3, a.rk, w4);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[i] = w4[i];
+        philox_rk(ctr_lo + (sw ^ 1u), ctr_hi, a.step32, c3, a.rk, w4);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) w[4 + i] = w4[i];
+    }
     bar_sync16(2);
     const float4 sc = s.xout[grp];
 
@@ -975,7 +1027,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
 }
 
 template <int BM, int BV, bool PBF, int G, int MODES>
-__global__ void __launch_bounds__(CTA16, ctas16<BM, G>()) solo_step_fast16_kernel(const StepArgs a) {
+__global__ void __launch_bounds__(CTA16, ctas16<BM, G>()) solo_step_fast16_kernel(const __grid_constant__ StepArgs a) {
     constexpr int KM = 1 << BM;
     constexpr bool EXT = MODES == 2;
     using Shared = Fast16Shared<BM, BV, PBF, G>;
@@ -1046,50 +1098,34 @@ __global__ void __launch_bounds__(CTA16, ctas16<BM, G>()) solo_step_fast16_kerne
     if constexpr (G == 4) s.sort[15][tid] = KEY_MAX;              // never overwritten
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s.mbar)) : "memory");
+        asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s.mbar_steal)) : "memory");
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     __syncthreads();
 
-    // the tile walk of solo_step_fast_kernel (a contiguous share of the tiles per CTA); tiles that are
-    // not full are skipped here
-    const int launch_tiles = (int)(a.total_tiles - a.tile_first);
-    const int share = (launch_tiles + (int)gridDim.x - 1) / (int)gridDim.x;
-    const int tile_begin = (int)min(a.tile_first + (int64_t)blockIdx.x * share, a.total_tiles);
-    const int tile_end = (int)min((int64_t)tile_begin + share, a.total_tiles);
-    int tensor = (a.num_tensors > 1 && tile_begin < tile_end ? find_tensor(a.tile_start, a.num_tensors, tile_begin) : 0) - 1;
-    int t_lo = 0, t_hi = 0, full_tiles = 0;
-    int64_t jb0 = 0;
-    char* pbase = nullptr;
-    const char* gbase = nullptr;
-    bool skip = false;
-    Ahead16 ah;
+    if (tid == 32) {
+        s.walk.phase = 0;
+        s.walk.t_lo = s.walk.t_hi = -1;
+        s.walk.tile = (int)a.tile_first + (int)blockIdx.x * a.share - 1;
+        s.walk.tile_end = (int)min((int64_t)s.walk.tile + 1 + a.share, a.total_tiles);
+        s.walk.tensor = (a.num_tensors > 1 ? find_tensor(a.tile_start, a.num_tensors, s.walk.tile + 1) : 0) - 1;
+        steal_request(s);
+        produce_tile16<BM, BV, PBF, G>(a, s, s.desc[0]);
+    }
+    __syncthreads();
+
+    bool failed = false;          // this thread once waited in vain for a copy: it waits no longer and stores nothing
+    uint32_t fill = 0;            // number of the tile, and of the copy it waits for
     const bool decay = a.decay != 1.0f;
-    for (int tile = tile_begin; tile < tile_end; ++tile) {
-        if (tile >= t_hi) {
-            do {
-                ++tensor;
-                t_hi = (int)__ldg(a.tile_start + tensor + 1);
-            } while (tile >= t_hi);
-            t_lo = (int)__ldg(a.tile_start + tensor);
-            const int64_t n = __ldg(a.numel + tensor);
-            jb0 = __ldg(a.block_start + tensor);
-            pbase = (char*)(a.param_list ? a.param_list[tensor] : a.param_single);
-            gbase = (const char*)(a.grad_list ? a.grad_list[tensor] : a.grad_single);
-            const bool aligned = ((((uintptr_t)pbase) | ((uintptr_t)gbase)) & 15u) == 0;
-            full_tiles = aligned ? (int)(n / TILE) : 0;
-            skip = a.numel_check != nullptr && __ldg(a.numel_check + tensor) != n;   // reported by the other launch
-        }
-        const int tin = tile - t_lo;
-        if (skip || tin >= full_tiles) continue;
-        const bool next_full = tin + 1 < full_tiles && tile + 1 < tile_end;
+    for (; s.desc[fill & 1u].valid; ++fill) {
         if (decay)
-            fast16_tile<BM, BV, PBF, G, true, MODES>(a, s, s_y, s_mid, s_mid4, s_yv, s_nv, s_yg, s_br, pbase, gbase, tin, jb0 + (int64_t)tin * Shared::NG, tensor, ah, next_full, tile);
+            fast16_tile<BM, BV, PBF, G, true, MODES>(a, s, s_y, s_mid, s_mid4, s_yv, s_nv, s_yg, s_br, fill, failed);
         else
-            fast16_tile<BM, BV, PBF, G, false, MODES>(a, s, s_y, s_mid, s_mid4, s_yv, s_nv, s_yg, s_br, pbase, gbase, tin, jb0 + (int64_t)tin * Shared::NG, tensor, ah, next_full, tile);
+            fast16_tile<BM, BV, PBF, G, false, MODES>(a, s, s_y, s_mid, s_mid4, s_yv, s_nv, s_yg, s_br, fill, failed);
     }
     // A thread that gave up on a copy waits once more, again bounded, for the last one that was issued,
     // so that no copy is still writing to the stage when the CTA's shared memory is released.
-    if (ah.failed && ah.fill > 0) mbar_wait(smem_u32(&s.mbar), (ah.fill - 1u) & 1u);
+    if (failed && fill > 0) mbar_wait(smem_u32(&s.mbar), (fill - 1u) & 1u);
 }
 
 }  // namespace solo
