@@ -32,8 +32,8 @@ UNITS = [
     ("solo_fast_inst.cu", "solo_fast_bm3.o", ["-DSOLO_BM=3"]),
     ("solo_fast_inst.cu", "solo_fast_bm4.o", ["-DSOLO_BM=4"]),
     ("solo_fast_inst.cu", "solo_fast_bm8.o", ["-DSOLO_BM=8"]),
-    *[("solo_fast16_inst.cu", f"solo_fast16_g{g}_m{m}.o", [f"-DSOLO_G={g}", f"-DSOLO_MODES={m}"])
-      for g in (4, 8, 16) for m in (0, 1, 2)],
+    *[("solo_fast16_inst.cu", f"solo_fast16_g{g}_m{m}_w{w}.o", [f"-DSOLO_G={g}", f"-DSOLO_MODES={m}", f"-DSOLO_W8={w}"])
+      for w in (1, 0) for m in (2, 1, 0) for g in (16, 8, 4)],
 ]
 
 

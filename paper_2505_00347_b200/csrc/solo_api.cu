@@ -282,6 +282,7 @@ void select_v_codebook(solo_state* s, const solo_hyper_t* h, StepArgs& a) {
     a.tables_v = h->v_codebook == SOLO_V_LOG
                      ? nullptr
                      : s->tables_v + (size_t)(h->v_codebook - 1) * v_table_floats(s->bits_v);
+    a.v_kind = h->v_codebook;
     s->v_codebook = h->v_codebook;
 }
 
@@ -734,6 +735,7 @@ int solo_multi_step_static(int32_t num_tensors, void* const* param_dev, const vo
     a.alpha = st->alpha;
     a.tables = d_tables;
     a.tables_v = vtab ? d_tables_v : nullptr;
+    a.v_kind = hyper->v_codebook;
     a.status = d_status;
     a.origin_id = (const int32_t*)zero_origin;
     a.origin_ctr = zero_origin;

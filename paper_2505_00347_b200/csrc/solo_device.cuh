@@ -52,6 +52,7 @@ struct StepArgs {
     float* alpha;
     const float* tables;               // y[K], mid[K-1], inv_gap[K-1] of the first-moment codebook
     const float* tables_v;             // baseline second-moment codebook y[K], mid[K-1]; null: Eq. 6
+    int32_t v_kind;                    // which one (SOLO_V_DE, ...); 0: Eq. 6
     int* status;                       // device word: non-zero after a descriptor mismatch
     // Position of every tensor of the list in the random stream (device arrays, never null; all zeros:
     // "tensor t of the list is stream t, from its first element"): a shard of a larger tensor names the

@@ -31,24 +31,26 @@ StepKernel fast_kernel(int bits_m, int bits_v, int block, bool param_bf16, bool 
 }
 
 StepKernel fast16_kernel(int bits_m, int bits_v, int block, bool param_bf16, int modes) {
-#define SOLO_PICK16(G)                                                                   \
-    (modes == 0 ? fast16_kernel_g##G##_m0(bits_m, bits_v, param_bf16)                    \
-                : modes == 1 ? fast16_kernel_g##G##_m1(bits_m, bits_v, param_bf16)       \
-                             : fast16_kernel_g##G##_m2(bits_m, bits_v, param_bf16))
+#define SOLO_PICK16(G, W8)                                                                    \
+    (modes == 0 ? fast16_kernel_g##G##_m0##W8(bits_m, bits_v, param_bf16)                     \
+                : modes == 1 ? fast16_kernel_g##G##_m1##W8(bits_m, bits_v, param_bf16)        \
+                             : fast16_kernel_g##G##_m2##W8(bits_m, bits_v, param_bf16))
+    const bool w8 = bits_m == 8 || bits_v == 8;
     switch (block) {
-        case 64: return SOLO_PICK16(4);
-        case 128: return SOLO_PICK16(8);
-        case 256: return SOLO_PICK16(16);   // twenty-five selection rounds
+        case 64: return w8 ? SOLO_PICK16(4, _w8) : SOLO_PICK16(4, );
+        case 128: return w8 ? SOLO_PICK16(8, _w8) : SOLO_PICK16(8, );
+        case 256: return w8 ? SOLO_PICK16(16, _w8) : SOLO_PICK16(16, );
         default: return nullptr;
     }
 #undef SOLO_PICK16
 }
 
 size_t fast16_kernel_smem(int bits_m, int bits_v, int block, bool param_bf16) {
+    const bool w8 = bits_m == 8 || bits_v == 8;
     switch (block) {
-        case 64: return fast16_smem_g4(bits_m, bits_v, param_bf16);
-        case 128: return fast16_smem_g8(bits_m, bits_v, param_bf16);
-        case 256: return fast16_smem_g16(bits_m, bits_v, param_bf16);
+        case 64: return w8 ? fast16_smem_g4_w8(bits_m, bits_v, param_bf16) : fast16_smem_g4(bits_m, bits_v, param_bf16);
+        case 128: return w8 ? fast16_smem_g8_w8(bits_m, bits_v, param_bf16) : fast16_smem_g8(bits_m, bits_v, param_bf16);
+        case 256: return w8 ? fast16_smem_g16_w8(bits_m, bits_v, param_bf16) : fast16_smem_g16(bits_m, bits_v, param_bf16);
         default: return 0;
     }
 }

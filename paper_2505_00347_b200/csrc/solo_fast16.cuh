@@ -1,4 +1,4 @@
-// Sixteen elements per thread: the streamlined step for the plain step (2/3/4-bit states, blocks of
+// Sixteen elements per thread: the streamlined step for the plain step (2/3/4/8-bit states, blocks of
 // 64, 128 or 256, fp32 or bf16 parameters; no L2 term in the gradient, no AdaBelief, base from the
 // p-quantile, xi drawn: MODES = 0).  Two more instantiations read other modes from the arguments:
 // MODES = 1 the L2 term, AdaBelief, a fixed base, no dither; MODES = 2 also stochastic rounding of the
@@ -30,6 +30,13 @@
 // gradients.  Everything that is tied to an element's position (its codes, its Philox draw, where
 // its parameter is stored) follows the swap; nothing else depends on the order.
 //
+// 8-bit states: codes of fixed codebooks by one cell look-up and one comparison (solo_lut8.cuh), alpha^k from a table
+// of the code's low bits that the block's lanes double bit by bit.  Against the eight-per-thread kernel's eight-step
+// searches and eight-factor chains (2^27 elements): 8/8 bit 886 -> 496 us, block 256 947 -> 502, 8/4 bit 816 -> 418; against the
+// general kernel: dynamic exponent for both moments 1754 -> 417 us, Eq. 5 2356 -> 763.  With two fixed codebooks the
+// kernel is bound by shared-memory wavefronts (83 % of their peak: six look-ups per element, two to four
+// different words per bank each).
+//
 // This kernel processes full tiles of 16-byte aligned tensors only; every other tile is left to
 // a second launch with StepArgs::only_partial set: of solo_step_fast_kernel, or of the general kernel
 // where that one has no path (the baseline codebooks).
@@ -37,6 +44,7 @@
 
 #include "solo_dispatch.h"
 #include "solo_fast.cuh"
+#include "solo_lut8.cuh"
 
 namespace solo {
 
@@ -45,9 +53,11 @@ static_assert(CTA16 * EPT16 == TILE, "same tile as the other kernels");
 
 // Resident CTAs per SM an instantiation is compiled for: eight (64 registers), seven (72) for 4-bit first moments
 // and for blocks of 256, which spill more at 64 (2^27 elements: 2/3 bit at block 128 380 us at seven, 367 us at
-// eight; 4/4 bit 422 and 421 us; 4/4 bit at block 256 432 and 434 us).
-template <int BM, int G>
-constexpr int ctas16() { return BM == 4 || G == 16 ? 7 : 8; }
+// eight; 4/4 bit 422 and 421 us; 4/4 bit at block 256 432 and 434 us).  8-bit states, whose tables fill the shared
+// memory: seven, six where the modes' tables come on top (8/8 bit five 516, six 498, seven 496 us; Eq. 5 four 830, five
+// 799, six 763 us).
+template <int BM, int BV, int G, int MODES>
+constexpr int ctas16() { return BM == 8 || BV == 8 ? (MODES == 2 ? 6 : 7) : BM == 4 || G == 16 ? 7 : 8; }
 
 // G: lanes per block (4, 8 or 16 for blocks of 64, 128 or 256 elements); NG = 128 / G blocks per tile.
 template <int BM, int BV, bool PBF, int G>
@@ -62,8 +72,21 @@ struct Fast16Shared {
     // per block spend more on building sixteen pairs than they save (2/2 bit at block 64 on 2^27 elements:
     // 346 us with single levels, 380 us with pairs).
     static constexpr bool PAIRS = G >= 8;
-    alignas(8) float tab_v[NG][BV == 2 && PAIRS ? 32 : 1 << BV];
-    alignas(8) float tab_m[NG][BM == 2 && PAIRS ? 32 : 1 << BM];
+    // 8-bit second moments: alpha^k for the low TB bits of the code, sixteen entries per lane of the block
+    // (eight words of padding put the blocks of a warp on different banks); the factors of the bits above
+    // are multiplied on per element.  With G = 16 that is all eight bits, and Delta_v is in the table.  8-bit first
+    // moments: the codebook itself, scaled per element.
+    static constexpr int TB = BV != 8 ? BV : G == 4 ? 6 : G == 8 ? 7 : 8;
+    alignas(16) float tab_v[NG][BV == 8 ? (1 << TB) + 8 : BV == 2 && PAIRS ? 32 : 1 << BV];
+    alignas(8) float tab_m[BM == 8 ? 1 : NG][BM == 8 ? 2 : BM == 2 && PAIRS ? 32 : 1 << BM];
+    alignas(16) unsigned char lut_m[BM == 8 ? LUT8_M_BYTES : 16];        // cells of the signed codebook (solo_lut8.cuh)
+    // 8-bit baseline second-moment codebook, in the place of tab_v, which it has no use for
+    struct Codebook8 {
+        unsigned char lut[LUT8_V_BYTES];
+        float y[256], mid[256];              // mid[255]: +infinity
+    };
+    static_assert(BV != 8 || sizeof(Codebook8) <= sizeof(float) * NG * ((1 << TB) + 8), "fits the table's place");
+    __device__ Codebook8& v8() { return *reinterpret_cast<Codebook8*>(&tab_v[0][0]); }
     // Exchange with the first warp.  One copy is enough: xin is written before the tile's first
     // barrier and read between its two barriers, xout is written between the barriers and read
     // after the second, and nobody writes either again before passing those barriers.
@@ -122,8 +145,12 @@ struct PairOffsets2 {
 // code words (thread t owns bytes [2 * BITS * t, 2 * BITS * (t + 1)) of them).  sw = 1: the two
 // words are exchanged (h[0] then holds elements 8..15).
 template <int BITS>
-__device__ __forceinline__ void load_codes16(const uint32_t* st, int tid, uint32_t sw, uint32_t (&h)[2]) {
-    if constexpr (BITS == 2) {
+__device__ __forceinline__ void load_codes16(const uint32_t* st, int tid, uint32_t sw, uint32_t (&h)[BITS == 8 ? 4 : 2]) {
+    if constexpr (BITS == 8) {                                    // four codes per word
+        const uint4 c = reinterpret_cast<const uint4*>(st)[tid];
+        h[0] = sw ? c.z : c.x; h[1] = sw ? c.w : c.y;
+        h[2] = sw ? c.x : c.z; h[3] = sw ? c.y : c.w;
+    } else if constexpr (BITS == 2) {
         const uint32_t c = __funnelshift_r(st[tid], st[tid], 16u * sw);
         h[0] = c & 0xFFFFu; h[1] = c >> 16;
     } else if constexpr (BITS == 4) {
@@ -143,8 +170,10 @@ __device__ __forceinline__ void load_codes16(const uint32_t* st, int tid, uint32
 // (48 bits per thread) go through `stage` (48 words of the warp) so that twelve lanes store the
 // warp's 192 bytes as 128-bit words.
 template <int BITS>
-__device__ __forceinline__ void store_codes16(uint8_t* tile_codes, uint32_t* stage, int tid, const uint32_t (&h)[2]) {
-    if constexpr (BITS == 2) {
+__device__ __forceinline__ void store_codes16(uint8_t* tile_codes, uint32_t* stage, int tid, const uint32_t (&h)[BITS == 8 ? 4 : 2]) {
+    if constexpr (BITS == 8) {
+        __stcs(reinterpret_cast<uint4*>(tile_codes) + tid, make_uint4(h[0], h[1], h[2], h[3]));
+    } else if constexpr (BITS == 2) {
         __stcs(reinterpret_cast<uint32_t*>(tile_codes) + tid, h[0] | (h[1] << 16));
     } else if constexpr (BITS == 4) {
         __stcs(reinterpret_cast<uint2*>(tile_codes) + tid, make_uint2(h[0], h[1]));
@@ -177,6 +206,20 @@ __device__ constexpr unsigned char SORT16_PAIRS[62][2] = {
     {0, 8}, {4, 12}, {4, 8}, {2, 10}, {6, 14}, {6, 10}, {2, 4}, {6, 8}, {10, 12},
     {1, 9}, {5, 13}, {5, 9}, {3, 11}, {7, 15}, {7, 11}, {3, 5}, {7, 9}, {11, 13},
     {1, 2}, {3, 4}, {5, 6}, {7, 8}, {9, 10}, {11, 12}};
+
+// Thresholds of the 8-bit codebooks below the cell of r (solo_lut8.cuh).
+__device__ __forceinline__ uint32_t cell8_m(const unsigned char* lut, float r) {
+    const uint32_t t = __float_as_uint(fmaxf(fabsf(r), 0x1p-22f)) ^ ((__float_as_uint(r) >> 3) & 0x10000000u);
+    // (negative values: exponent bit 5 cleared.  Written so that the positive cells follow the negative ones.)
+    return lut[(t >> 17) - LUT8_M_BASE];
+}
+__device__ __forceinline__ uint32_t cell8_v(const unsigned char* lut, float r) {
+    return lut[(__float_as_uint(fmaxf(r, 0x1p-23f)) >> 16) - LUT8_V_BASE];
+}
+// Four codes to a word.
+__device__ __forceinline__ uint32_t pack8(uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    return __byte_perm(__byte_perm(a, b, 0x0040u), __byte_perm(c, d, 0x0040u), 0x5410u);
+}
 
 // Minimum / maximum over the calling lane's group of G lanes.  The shuffle-and-compare steps serve
 // all groups of the warp at once; for groups of eight measured faster here than the full-mask reductions
@@ -525,7 +568,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     uint32_t mx_v = 0;
     float mx_m_f = 0.0f;
     {
-        uint32_t cm[2], cv[2];                                    // eight codes per word
+        uint32_t cm[BM == 8 ? 4 : 2], cv[BV == 8 ? 4 : 2];        // eight codes per word, 8-bit: four
         // (word offsets of codes that do not start on a 16-byte boundary: 0 or 2, see issue_tile_copy16)
         load_codes16<BM>(st.cm + ((int)((jb_tile * (2 * G * BM)) & 15) >> 2), tid, sw, cm);
         load_codes16<BV>(st.cv + ((int)((jb_tile * (2 * G * BV)) & 15) >> 2), tid, sw, cv);
@@ -534,14 +577,34 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
 
         // per-block level tables (Eq. 2), built by the block's G lanes
         float* const tab_vf = s.tab_v[grp];
-        float* const tab_mf = s.tab_m[grp];
+        float* const tab_mf = s.tab_m[BM == 8 ? 0 : grp];
+        float a2[BV];
         {
-            float a2[BV];
             a2[0] = al;
 #pragma unroll
             for (int i = 1; i < BV; ++i) a2[i] = a2[i - 1] * a2[i - 1];
             auto level_v = [&](uint32_t k) { return (vtab ? s_yv[k] : pow_sm<BV>(a2, k)) * dv; };
-            if constexpr (BV == 2 && Shared::PAIRS) {
+            if constexpr (BV == 8) {
+                // entries 2 gl, 2 gl + 1 from the bits that tell the lanes apart, then doubled bit by bit: entry q is
+                // entry (q without its top bit) times the top bit's factor, as in the chain of pow_sm
+                if (!vtab) {
+                    constexpr int LB = Shared::TB - 3;            // bits of 2 gl + 1
+                    float f[LB];
+#pragma unroll
+                    for (int i = 0; i < LB; ++i) f[i] = a2[i];
+                    F2 e[8];
+                    e[0] = F2::pack(pow_sm<LB>(f, (uint32_t)(2 * gl)), pow_sm<LB>(f, (uint32_t)(2 * gl + 1)));
+#pragma unroll
+                    for (int b = 0; b < 3; ++b)
+#pragma unroll
+                        for (int i = 0; i < (1 << b); ++i) e[i + (1 << b)] = mul2(e[i], F2::dup(a2[LB + b]));
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const F2 t = Shared::TB == 8 ? mul2(e[i], F2::dup(dv)) : e[i];
+                        *reinterpret_cast<float2*>(tab_vf + 2 * gl + (i << LB)) = make_float2(t.lo(), t.hi());
+                    }
+                }
+            } else if constexpr (BV == 2 && Shared::PAIRS) {
 #pragma unroll
                 for (int r0 = 0; r0 < 16; r0 += G)
                     *reinterpret_cast<float2*>(tab_vf + 2 * (r0 + gl)) = make_float2(level_v((r0 + gl) & 3), level_v((r0 + gl) >> 2));
@@ -550,7 +613,8 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
                 for (int r0 = 0; r0 < KV; r0 += G)
                     if (r0 + gl < KV) tab_vf[r0 + gl] = level_v(r0 + gl);
             }
-            if constexpr (BM == 2 && Shared::PAIRS) {
+            if constexpr (BM == 8) {
+            } else if constexpr (BM == 2 && Shared::PAIRS) {
 #pragma unroll
                 for (int r0 = 0; r0 < 16; r0 += G)
                     *reinterpret_cast<float2*>(tab_mf + 2 * (r0 + gl)) = make_float2(s_y[(r0 + gl) & 3] * dm, s_y[(r0 + gl) >> 2] * dm);
@@ -566,8 +630,8 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
         const char* const tab_v = reinterpret_cast<const char*>(tab_vf);
         const char* const tab_m = reinterpret_cast<const char*>(tab_mf);
         const PairOffsets2 om16(cm[0] | (cm[1] << 16)), ov16(cv[0] | (cv[1] << 16));   // used for 2-bit codes only
-        const CodeOffsets<BM> om4a(cm[0], 0u), om4b(cm[1], 0u);
-        const CodeOffsets<BV> ov4a(cv[0], 0u), ov4b(cv[1], 0u);
+        const CodeOffsets<BM> om4a(cm[0], cm[1]), om4b(cm[BM == 8 ? 2 : 1], cm[BM == 8 ? 3 : 1]);
+        const CodeOffsets<BV> ov4a(cv[0], cv[1]), ov4b(cv[BV == 8 ? 2 : 1], cv[BV == 8 ? 3 : 1]);
         const unsigned char* const sgb = st.g + 32 * tid;
         const uint4* const sg[2] = {reinterpret_cast<const uint4*>(sgb + 16u * sw),
                                     reinterpret_cast<const uint4*>(sgb + 16u - 16u * sw)};
@@ -599,13 +663,31 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const int j = 4 * h + k;                          // pair of elements 2j, 2j + 1
-                auto code_m = [&](int i) { return *reinterpret_cast<const float*>(tab_m + (i < 8 ? om4a(i) : om4b(i - 8))); };
-                auto code_v = [&](int i) { return *reinterpret_cast<const float*>(tab_v + (i < 8 ? ov4a(i) : ov4b(i - 8))); };
+                auto code_m = [&](int i) {
+                    const char* const t = BM == 8 ? reinterpret_cast<const char*>(s_y) : tab_m;
+                    return *reinterpret_cast<const float*>(t + (i < 8 ? om4a(i) : om4b(i - 8)));
+                };
+                auto code_v = [&](int i) {
+                    if constexpr (BV == 8) {
+                        const uint32_t o = i < 8 ? ov4a(i) : ov4b(i - 8);
+                        if (vtab) return *reinterpret_cast<const float*>(reinterpret_cast<const char*>(s.v8().y) + o);
+                        float x = *reinterpret_cast<const float*>(tab_v + (o & ((4u << Shared::TB) - 4u)));
+#pragma unroll
+                        for (int b = Shared::TB; b < 8; ++b) x = x * ((o >> (b + 2)) & 1u ? a2[b] : 1.0f);
+                        return x;
+                    } else {
+                        return *reinterpret_cast<const float*>(tab_v + (i < 8 ? ov4a(i) : ov4b(i - 8)));
+                    }
+                };
                 F2 mt, vt;
                 if constexpr (BM == 2 && Shared::PAIRS) mt = F2::load(tab_m + om16(j));
                 else mt = F2::pack(code_m(2 * j), code_m(2 * j + 1));
                 if constexpr (BV == 2 && Shared::PAIRS) vt = F2::load(tab_v + ov16(j));
                 else vt = F2::pack(code_v(2 * j), code_v(2 * j + 1));
+                if constexpr (BM == 8) mt = mul2(mt, F2::dup(dm));
+                if constexpr (BV == 8) {
+                    if (Shared::TB < 8 || vtab) vt = mul2(vt, F2::dup(dv));
+                }
                 mh[j] = fma2(beta1, mt, mul2(omb1, g2[k]));
                 if (belief) {                                     // AdaBelief: (g - m^)^2, plus eps
                     const F2 sig = fma2(mh[j], F2::dup(-1.0f), g2[k]);      // g - m^, one rounding
@@ -696,14 +778,14 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
 
     // ---- (C) first moment: block scale, nearest level (Eq. 1), see fast_tile ----
     const uint32_t mx_m = group_max16<G>(__float_as_uint(mx_m_f));
-    uint32_t om[2] = {0u, 0u};                                    // eight codes per word
+    uint32_t om[BM == 8 ? 4 : 2] = {};                            // eight codes per word, 8-bit: four
     const float dm_new = __uint_as_float(mx_m);
     const float inv_m = __frcp_rn(dm_new);
     // code = number of midpoints below r, each comparison as the saturation of (r - mid) * 2^100 on the FMA
     // pipe (exactly 0 or 1, see fast_tile).  The codes of elements 2j and 2j + 1 are accumulated side by side
     // in one pair of binary32 (eight 2- or 3-bit codes per pair, at most 21 bits each: exact).
     constexpr float BIG = 0x1p100f;
-    const float n0 = -s_mid[0] * BIG, n1 = -s_mid[1] * BIG, n2 = -s_mid[2] * BIG;
+    const float n0 = BM == 8 ? 0.0f : -s_mid[0] * BIG, n1 = BM == 8 ? 0.0f : -s_mid[1] * BIG, n2 = BM == 8 ? 0.0f : -s_mid[2] * BIG;
     float n3[4] = {0.0f, 0.0f, 0.0f, 0.0f};
     if constexpr (BM == 3) {
 #pragma unroll
@@ -723,6 +805,15 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     const F2 inv_m2 = F2::dup(inv_m);
     auto quant_m = [&](int j) {                                   // call with j = 7, 6, ..., 0
         const F2 r = mul2(mh[j], inv_m2);
+        if constexpr (BM == 8) {
+            // midpoints below the cell of r, plus one if r is above the cell's own
+            uint32_t q0 = cell8_m(s.lut_m, r.lo()), q1 = cell8_m(s.lut_m, r.hi());
+            q0 += r.lo() > s_mid[q0] ? 1u : 0u;
+            q1 += r.hi() > s_mid[q1] ? 1u : 0u;
+            const uint32_t two = __byte_perm(q0, q1, 0x0040u);
+            om[j >> 1] = (j & 1) ? two : __byte_perm(two, om[j >> 1], 0x5410u);
+            return;
+        }
         F2& acc = omf[2 * j / CPA];
         const F2 up = F2::dup((float)(KM * KM));
         auto step = [&](float n) {
@@ -753,7 +844,26 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
             acc = add2(acc, inner(ra.z, rb.z));
         }
     };
+    // 8-bit codes of a block with a NaN or infinite scale: every comparison with a NaN is false (code 0), zeros are code
+    // 127 (the cell tables know no NaN)
+    auto special_m8 = [&]() {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) om[BM == 8 ? i : 0] = 0u;
+#pragma unroll
+        for (int i = EPT16 - 1; i >= 0; --i) {
+            const float r = mh_at(i) * inv_m;
+            om[BM == 8 ? i >> 2 : 0] = (om[BM == 8 ? i >> 2 : 0] << 8) + (r == r ? 127u : 0u);
+        }
+    };
     auto quant_m_done = [&]() {
+        if constexpr (BM == 8) {
+            if (!(dm_new < __int_as_float(0x7f800000))) special_m8();
+            if (dm_new < TINY) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i) om[BM == 8 ? i : 0] = 0u;
+            }
+            return;
+        }
         uint32_t half[EPT16 / CPA];
 #pragma unroll
         for (int k = 0; k < EPT16 / CPA; ++k) half[k] = (uint32_t)__fmaf_rn(omf[k].hi(), (float)KM, omf[k].lo());
@@ -786,8 +896,9 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
             for (int i = 0; i < 4; ++i) wm[4 + i] = w4[i];
         }
         constexpr int Z = KM / 2 - 1;                             // index of the level 0
-        float nb[BM == 4 ? 3 : KM - 2];                           // nb[j - 1]: threshold of level j, BM == 4: of levels 4, 8, 12
-        if constexpr (BM == 4) {
+        float nb[BM >= 4 ? 3 : KM - 2];                           // nb[j - 1]: threshold of level j, BM == 4: of levels 4, 8, 12
+        if constexpr (BM == 8) {
+        } else if constexpr (BM == 4) {
             const float4 c4 = s_br[4];
             nb[0] = c4.x; nb[1] = c4.y; nb[2] = c4.z;
         } else {
@@ -807,6 +918,16 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
             for (int e = 1; e >= 0; --e) {
                 const int i = 2 * j + e;
                 const float r = mh_at(i) * inv_m;
+                if constexpr (BM == 8) {
+                    // levels reached below the cell of r, plus the cell's own
+                    uint32_t q = cell8_m(s.lut_m, r);
+                    q += r >= s_yg[q + 1].x ? 1u : 0u;
+                    const float2 yg = s_yg[q];
+                    const float frac = (r - yg.x) * yg.y;
+                    q += d[e] < frac * 65536.0f ? 1u : 0u;
+                    om[i >> 2] = (om[i >> 2] << 8) + q;
+                    continue;
+                }
                 const float t = r * BIG;
                 float qf;
                 if constexpr (BM == 4) {
@@ -835,14 +956,20 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
                 else accm[i >> 3] = __fmaf_rn(accm[i >> 3], (float)KM, code);
             }
         }
-        if constexpr (BM == 4) {
+        if constexpr (BM == 8) {
+            // (an infinite scale: r is +-0, level 127 exactly, or NaN)
+            if (!(dm_new < __int_as_float(0x7f800000))) special_m8();
+        } else if constexpr (BM == 4) {
             om[0] = (uint32_t)accm[0] | ((uint32_t)accm[1] << 16);
             om[1] = (uint32_t)accm[2] | ((uint32_t)accm[3] << 16);
         } else {
             om[0] = (uint32_t)accm[0];
             om[1] = (uint32_t)accm[1];
         }
-        if (dm_new < TINY) { om[0] = 0; om[1] = 0; }             // vanishing block: all codes 0
+        if (dm_new < TINY) {                                      // vanishing block: all codes 0
+#pragma unroll
+            for (int i = 0; i < (BM == 8 ? 4 : 2); ++i) om[i] = 0u;
+        }
     }
 
     // ---- (D) second moment: block scale and the p-quantile ----
@@ -912,13 +1039,27 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     const float4 sc = s.xout[grp];
 
     // second moment: Eq. 6, see fast_tile
-    uint32_t ov[2];
+    uint32_t ov[BV == 8 ? 4 : 2];
     if (vtab) {
         // Eq. 1 on the fixed codebook: code = number of midpoints below r, counted like the first
         // moment's (saturated multiply-adds, exactly 0 or 1 each: r and a midpoint, if they differ at all,
         // differ by far more than 2^-100, the smallest midpoint of these codebooks being about 1e-4)
         const float inv = sc.y;
-        if constexpr (BV <= 3) {
+        if constexpr (BV == 8) {
+            // (a NaN falls into the first cell, as a zero does: code 0)
+            const typename Shared::Codebook8& cb = s.v8();
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                uint32_t q[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float r = vh_at(4 * k + i) * inv;
+                    q[i] = cell8_v(cb.lut, r);
+                    q[i] += r > cb.mid[q[i]] ? 1u : 0u;
+                }
+                ov[k] = pack8(q[0], q[1], q[2], q[3]);
+            }
+        } else if constexpr (BV <= 3) {
             const float4 na = s_nv[0], nb = s_nv[1];
             float acc[2] = {0.0f, 0.0f};                         // eight codes, at most 24 bits: exact
 #pragma unroll
@@ -958,7 +1099,10 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
             ov[0] = (uint32_t)acc[0] | ((uint32_t)acc[1] << 16);
             ov[1] = (uint32_t)acc[2] | ((uint32_t)acc[3] << 16);
         }
-        if (sc.x != 0.0f) { ov[0] = 0; ov[1] = 0; }              // vanishing block: all codes 0
+        if (sc.x != 0.0f) {                                       // vanishing block: all codes 0
+#pragma unroll
+            for (int i = 0; i < (BV == 8 ? 4 : 2); ++i) ov[i] = 0u;
+        }
     } else {
         const float inv = sc.y, il = sc.z, lim = sc.w;
         constexpr float KM1 = (float)(KV - 1);
@@ -969,7 +1113,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
         const F2 xs0 = F2::dup(round_v ? (float)((-0.5 + 0x1p-17) / (KV - 1)) : 0.0f);
         const F2 inv2 = F2::dup(inv);
         // codes of elements 2j and 2j + 1 side by side in one pair of binary32, as for the first moment
-        constexpr int CPA = BV == 4 ? 4 : 8;
+        constexpr int CPA = BV >= 4 ? 4 : 8;
         float worst = 0.0f;
         F2 acc[EPT16 / CPA];
 #pragma unroll
@@ -982,22 +1126,30 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
             const F2 r = mul2(vh[j], inv2);
             const F2 ts = F2::pack(__saturatef(__fmaf_rn(lg2_approx(r.lo()), ils, x.lo())),
                                    __saturatef(__fmaf_rn(lg2_approx(r.hi()), ils, x.hi())));
-            const F2 q = add2(fma2(ts, F2::dup(KM1), F2::dup(MAGIC)), F2::dup(-MAGIC));      // the codes, rounded
+            const F2 u = fma2(ts, F2::dup(KM1), F2::dup(MAGIC));  // the codes, rounded, in the low bits
+            const F2 q = add2(u, F2::dup(-MAGIC));
             const F2 off = fma2(ts, F2::dup(-KM1), q);            // their distance from what was rounded
             worst = fmaxf(fmaxf(worst, fabsf(off.lo())), fabsf(off.hi()));
-            acc[2 * j / CPA] = fma2(acc[2 * j / CPA], F2::dup((float)(KV * KV)), q);
+            if constexpr (BV == 8) {                              // (a byte each)
+                const uint32_t two = __byte_perm(__float_as_uint(u.lo()), __float_as_uint(u.hi()), 0x0040u);
+                ov[j >> 1] = (j & 1) ? two : __byte_perm(two, ov[j >> 1], 0x5410u);
+            } else {
+                acc[2 * j / CPA] = fma2(acc[2 * j / CPA], F2::dup((float)(KV * KV)), q);
+            }
         }
-        uint32_t half[EPT16 / CPA];
+        if constexpr (BV != 8) {
+            uint32_t half[EPT16 / CPA];
 #pragma unroll
-        for (int k = 0; k < EPT16 / CPA; ++k) half[k] = (uint32_t)__fmaf_rn(acc[k].hi(), (float)KV, acc[k].lo());
-        ov[0] = BV <= 3 ? half[0] : half[0] | (half[1] << 16);
-        ov[1] = BV <= 3 ? half[1] : half[EPT16 / CPA - 2] | (half[EPT16 / CPA - 1] << 16);
+            for (int k = 0; k < EPT16 / CPA; ++k) half[k] = (uint32_t)__fmaf_rn(acc[k].hi(), (float)KV, acc[k].lo());
+            ov[0] = BV <= 3 ? half[0] : half[0] | (half[1] << 16);
+            ov[1] = BV <= 3 ? half[1] : half[EPT16 / CPA - 2] | (half[EPT16 / CPA - 1] << 16);
+        }
         if (__any_sync(0xffffffffu, worst > lim)) {
             // too close to a rounding boundary for the approximate logarithm somewhere in the warp:
             // the exact sequence for all sixteen
             const float x1 = round_v ? 0x1p-16f : 0.0f, x0 = round_v ? -0.5f + 0x1p-17f : 0.0f;
-            ov[0] = 0;
-            ov[1] = 0;
+#pragma unroll
+            for (int i = 0; i < (BV == 8 ? 4 : 2); ++i) ov[i] = 0u;
 #pragma unroll
             for (int j = EPT16 / 2 - 1; j >= 0; --j) {
                 float d[2];
@@ -1012,22 +1164,29 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
                         t = fminf(fmaxf(t, 0.0f), KM1);
                         q = (uint32_t)__float2int_rn(t);
                     }
-                    ov[i >> 3] = (ov[i >> 3] << BV) + q;
+                    uint32_t& o = ov[BV == 8 ? i >> 2 : i >> 3];
+                    o = (o << BV) + q;
                 }
             }
         }
-        if (sc.x != 0.0f) { ov[0] = 0; ov[1] = 0; }              // vanishing block: all codes 0
+        if (sc.x != 0.0f) {                                       // vanishing block: all codes 0
+#pragma unroll
+            for (int i = 0; i < (BV == 8 ? 4 : 2); ++i) ov[i] = 0u;
+        }
     }
 
     // ---- store the codes ----
-    const uint32_t om_e[2] = {sw ? om[1] : om[0], sw ? om[0] : om[1]};      // back to element order
-    const uint32_t ov_e[2] = {sw ? ov[1] : ov[0], sw ? ov[0] : ov[1]};
+    uint32_t om_e[BM == 8 ? 4 : 2], ov_e[BV == 8 ? 4 : 2];        // back to element order
+#pragma unroll
+    for (int i = 0; i < (BM == 8 ? 4 : 2); ++i) om_e[i] = sw ? om[i ^ (BM == 8 ? 2 : 1)] : om[i];
+#pragma unroll
+    for (int i = 0; i < (BV == 8 ? 4 : 2); ++i) ov_e[i] = sw ? ov[i ^ (BV == 8 ? 2 : 1)] : ov[i];
     store_codes16<BM>(a.codes_m + jb_tile * (2 * G * BM), s.cout[0][BM == 3 ? warp : 0], tid, om_e);
     store_codes16<BV>(a.codes_v + jb_tile * (2 * G * BV), s.cout[(BM == 3 && BV == 3) ? 1 : 0][BV == 3 ? warp : 0], tid, ov_e);
 }
 
 template <int BM, int BV, bool PBF, int G, int MODES>
-__global__ void __launch_bounds__(CTA16, ctas16<BM, G>()) solo_step_fast16_kernel(const __grid_constant__ StepArgs a) {
+__global__ void __launch_bounds__(CTA16, ctas16<BM, BV, G, MODES>()) solo_step_fast16_kernel(const __grid_constant__ StepArgs a) {
     constexpr int KM = 1 << BM;
     constexpr bool EXT = MODES == 2;
     using Shared = Fast16Shared<BM, BV, PBF, G>;
@@ -1037,13 +1196,17 @@ __global__ void __launch_bounds__(CTA16, ctas16<BM, G>()) solo_step_fast16_kerne
     __shared__ float s_mid[KM];
     __shared__ float2 s_yg[EXT ? KM : 1];                    // Eq. 5: see the set-up below
     __shared__ float4 s_br[EXT ? (BM == 4 ? 5 : 2) : 1];
-    __shared__ float s_yv[EXT ? 1 << BV : 1];               // baseline second-moment codebook: its levels,
+    __shared__ float s_yv[EXT && BV != 8 ? 1 << BV : 1];               // baseline second-moment codebook: its levels,
     __shared__ float4 s_nv[EXT ? 8 : 1];                     // its midpoints times -2^100 (rows as the tile function reads them)
     __shared__ float4 s_mid4[4];             // 4-bit first moments: per quarter of the codebook, its three inner midpoints times -2^100
     const int tid = threadIdx.x;
-    if (tid < KM) {
-        s_y[tid] = a.tables[tid];
-        if (tid < KM - 1) s_mid[tid] = a.tables[KM + tid];
+    for (int i = tid; i < KM; i += CTA16) {
+        s_y[i] = a.tables[i];
+        s_mid[i] = i < KM - 1 ? a.tables[KM + i] : __int_as_float(0x7f800000);
+    }
+    if constexpr (BM == 8) {
+        const uint4* const src = reinterpret_cast<const uint4*>(g_lut8_m[EXT && a.round_m ? 1 : 0].q);
+        for (int i = tid; i < LUT8_M_BYTES / 16; i += CTA16) reinterpret_cast<uint4*>(s.lut_m)[i] = src[i];
     }
     if (BM == 4 && tid < 4)
         s_mid4[tid] = make_float4(-a.tables[KM + 4 * tid] * 0x1p100f, -a.tables[KM + 4 * tid + 1] * 0x1p100f,
@@ -1055,11 +1218,15 @@ __global__ void __launch_bounds__(CTA16, ctas16<BM, G>()) solo_step_fast16_kerne
             // 2- and 3-bit, levels 1..6 in rows 0, 1; 4-bit, row s = levels 4s+1..4s+3 and row 4 = levels
             // 4, 8, 12).  The level 0 is compared another way; a level past K-2 gets -infinity: never reached.
             const float* const yk = a.tables;
+            if constexpr (BM == 8) {                              // (the pair past the last bracket is never reached)
+                for (int i = tid; i < KM; i += CTA16)
+                    s_yg[i] = i < KM - 1 ? make_float2(yk[i], a.tables[2 * KM - 1 + i]) : make_float2(__int_as_float(0x7f800000), 0.0f);
+            }
             auto below = [&](int j) {
                 const float y = yk[j];
                 return -__uint_as_float(__float_as_uint(y) + (y < 0.0f ? 1u : 0xFFFFFFFFu)) * 0x1p100f;
             };
-            if (tid < KM - 1) s_yg[tid] = make_float2(yk[tid], a.tables[2 * KM - 1 + tid]);
+            if (BM != 8 && tid < KM - 1) s_yg[tid] = make_float2(yk[tid], a.tables[2 * KM - 1 + tid]);
             if (BM <= 3 && tid < 2) {
                 float t4[4];
 #pragma unroll
@@ -1081,8 +1248,18 @@ __global__ void __launch_bounds__(CTA16, ctas16<BM, G>()) solo_step_fast16_kerne
         if (a.tables_v != nullptr) {
             constexpr int KV = 1 << BV;
             const float* const midv = a.tables_v + KV;            // KV - 1 midpoints
-            if (tid < KV) s_yv[tid] = a.tables_v[tid];
-            if (tid < 2) {                                         // rows 0, 1: midpoints 0..7 (rows of 3 or 7 are padded)
+            if constexpr (BV == 8) {
+                typename Shared::Codebook8& cb = s.v8();
+                for (int i = tid; i < KV; i += CTA16) {
+                    cb.y[i] = a.tables_v[i];
+                    cb.mid[i] = i < KV - 1 ? midv[i] : __int_as_float(0x7f800000);
+                }
+                const uint4* const src = reinterpret_cast<const uint4*>(g_lut8_v[a.v_kind - 1].q);
+                for (int i = tid; i < LUT8_V_BYTES / 16; i += CTA16) reinterpret_cast<uint4*>(cb.lut)[i] = src[i];
+            } else if (tid < KV) {
+                s_yv[tid] = a.tables_v[tid];
+            }
+            if (BV != 8 && tid < 2) {                                         // rows 0, 1: midpoints 0..7 (rows of 3 or 7 are padded)
                 float m4[4];
 #pragma unroll
                 for (int k = 0; k < 4; ++k) m4[k] = 4 * tid + k < KV - 1 ? -midv[4 * tid + k] * 0x1p100f : 0.0f;

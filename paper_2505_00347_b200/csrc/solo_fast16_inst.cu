@@ -1,7 +1,7 @@
 // The sixteen-elements-per-thread kernels for one block size (SOLO_G = 4, 8, 16 lanes per block:
 // blocks of 64, 128, 256 elements) and one set of modes (SOLO_MODES = 0: the paper's plain step, fixed
-// at compile time; 1, 2: read from the arguments, see solo_fast16.cuh): 2/3/4-bit states, fp32 or bf16
-// parameters.
+// at compile time; 1, 2: read from the arguments, see solo_fast16.cuh): fp32 or bf16 parameters, 2/3/4-bit states
+// (SOLO_W8 = 0) or an 8-bit state and any other (SOLO_W8 = 1).
 #include "solo_dispatch.h"
 #include "solo_fast16.cuh"
 
@@ -10,6 +10,10 @@
 #endif
 #ifndef SOLO_MODES
 #error "compile with -DSOLO_MODES=0|1|2"
+#endif
+
+#ifndef SOLO_W8
+#error "compile with -DSOLO_W8=0|1"
 #endif
 
 #define SOLO_CAT_(a, b) a##b
@@ -23,33 +27,29 @@ namespace solo {
 #define SOLO_S16(BM, BV) \
     (param_bf16 ? sizeof(Fast16Shared<BM, BV, true, SOLO_G>) : sizeof(Fast16Shared<BM, BV, false, SOLO_G>))
 
-StepKernel SOLO_CAT4(fast16_kernel_g, SOLO_G, _m, SOLO_MODES)(int bits_m, int bits_v, bool param_bf16) {
+#if SOLO_W8
+#define SOLO_WIDTHS(X) X(2, 8) X(3, 8) X(4, 8) X(8, 2) X(8, 3) X(8, 4) X(8, 8)
+#define SOLO_NAME(stem) SOLO_CAT(stem, _w8)
+#else
+#define SOLO_WIDTHS(X) X(2, 2) X(2, 3) X(2, 4) X(3, 2) X(3, 3) X(3, 4) X(4, 2) X(4, 3) X(4, 4)
+#define SOLO_NAME(stem) stem
+#endif
+
+StepKernel SOLO_NAME(SOLO_CAT4(fast16_kernel_g, SOLO_G, _m, SOLO_MODES))(int bits_m, int bits_v, bool param_bf16) {
     switch (bits_m * 10 + bits_v) {
-        case 22: return SOLO_K16(2, 2);
-        case 23: return SOLO_K16(2, 3);
-        case 24: return SOLO_K16(2, 4);
-        case 32: return SOLO_K16(3, 2);
-        case 33: return SOLO_K16(3, 3);
-        case 34: return SOLO_K16(3, 4);
-        case 42: return SOLO_K16(4, 2);
-        case 43: return SOLO_K16(4, 3);
-        case 44: return SOLO_K16(4, 4);
+#define SOLO_CASE(BM, BV) case BM * 10 + BV: return SOLO_K16(BM, BV);
+        SOLO_WIDTHS(SOLO_CASE)
+#undef SOLO_CASE
         default: return nullptr;
     }
 }
 
 #if SOLO_MODES == 0
-size_t SOLO_CAT(fast16_smem_g, SOLO_G)(int bits_m, int bits_v, bool param_bf16) {
+size_t SOLO_NAME(SOLO_CAT(fast16_smem_g, SOLO_G))(int bits_m, int bits_v, bool param_bf16) {
     switch (bits_m * 10 + bits_v) {
-        case 22: return SOLO_S16(2, 2);
-        case 23: return SOLO_S16(2, 3);
-        case 24: return SOLO_S16(2, 4);
-        case 32: return SOLO_S16(3, 2);
-        case 33: return SOLO_S16(3, 3);
-        case 34: return SOLO_S16(3, 4);
-        case 42: return SOLO_S16(4, 2);
-        case 43: return SOLO_S16(4, 3);
-        case 44: return SOLO_S16(4, 4);
+#define SOLO_CASE(BM, BV) case BM * 10 + BV: return SOLO_S16(BM, BV);
+        SOLO_WIDTHS(SOLO_CASE)
+#undef SOLO_CASE
         default: return 0;
     }
 }
