@@ -288,8 +288,8 @@ float solo_default_beta1(int bits_m, int from_scratch);
 /*
  * Kernel selection.  0 (default): every width and block size with the logarithmic
  * second-moment quantizer, nearest rounding of the first moment and eps >= 1e-12 runs the
- * streamlined kernel (fp32 or bf16 parameters), everything else the general one; tensor sets of
- * at least 8192 tiles of 2048 elements with blocks of 64, 128 or 256 run
+ * streamlined kernel (fp32 or bf16 parameters), everything else the general one; tensor sets from
+ * about a thousand tiles of 2048 elements on with blocks of 64, 128 or 256 run
  * their full tiles in a kernel with sixteen elements per thread and the remaining tiles in the
  * streamlined kernel, or in the general one where the streamlined kernel does not apply (two
  * launches).  That kernel covers every mode of solo_hyper_t (Eq. 5 rounding and the baseline

@@ -211,7 +211,17 @@ int launch_kernel(solo::StepKernel k, const StepArgs& a, int device, int threads
     if (threads == solo::CTA16) grid = (a.total_tiles - a.tile_first + a.share - 1) / a.share;
     if (grid < 1) return SOLO_EINVAL;
     void* params[] = {(void*)&a};
-    cudaError_t e = cudaLaunchKernel((const void*)k, dim3((unsigned)grid), dim3((unsigned)threads), params, dyn_smem, stream);
+    cudaLaunchAttribute attr = {};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;    // see pdl_wait
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = dyn_smem;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaError_t e = cudaLaunchKernelExC(&cfg, (const void*)k, params);
     if (e != cudaSuccess) {
         cudaGetLastError();
         return SOLO_ECUDA;
@@ -230,9 +240,14 @@ int launch_step(solo_state* s, StepArgs& a, cudaStream_t stream) {
     const bool streamlined = fast_ok && !a.tables_v && !a.round_m;
     const bool plain = !a.l2 && !a.belief && a.fixed_alpha == 0.0f && a.round_v && !a.tables_v && !a.round_m;
     solo::StepKernel k16 = nullptr;
-    // worth its second launch only when there is work for many tiles per CTA (measured faster on the
-    // 7B-shaped, the GPT-125M-shaped and the ragged set; a 1 Mi-element tensor is launch-bound)
-    const bool large = s->tiles_total >= 8192;
+    // From one wave of tiles on; below, a tile's latency counts, which is shorter with twice the threads per tile
+    // (4/4 bit: 128 tiles 4.2 us against 5.0 us, 512 tiles, step after step, 8.3 and 9.8, 2048 tiles 23.6 and 18.9; 8/8 bit:
+    // 256 tiles 8.6 and 7.7).
+    // Lists need a second launch for the tiles that are not full (513 tiles 7.6 us against 9.4 us).  What the
+    // streamlined kernel has no path for, one tile on (Eq. 5 at one tile 9.7 us in the general kernel, 7.4 us here).
+    const bool all_full = !a.param_list && s->num_tensors == 1 && s->numel[0] % solo::TILE == 0;
+    const int64_t from = !streamlined ? (all_full ? 1 : 64) : (s->bits_m == 8 || s->bits_v == 8 ? 256 : 768) * (all_full ? 1 : 2);
+    const bool large = s->tiles_total >= from;
     if (fast_ok && ((policy == 0 && large) || policy == 3))
         k16 = solo::fast16_kernel(s->bits_m, s->bits_v, s->block, a.param_bf16 != 0,
                                   plain ? 0 : (a.tables_v || a.round_m) ? 2 : 1);
@@ -247,12 +262,13 @@ int launch_step(solo_state* s, StepArgs& a, cudaStream_t stream) {
         // not 16-byte aligned) by the streamlined kernel, or by the general one where that has no path
         int rc = launch_kernel(k16, a, s->device, solo::CTA16, solo::fast16_kernel_smem(s->bits_m, s->bits_v, s->block, a.param_bf16 != 0), stream);
         if (rc) return rc;
-        const bool all_full = !a.param_list && s->num_tensors == 1 && s->numel[0] % solo::TILE == 0;
         if (all_full) return SOLO_OK;
         a.only_partial = 1;
+        // (a single tensor is aligned: its last tile is all that is left)
+        if (!a.param_list) a.tile_first = s->tiles_total - 1;
     }
     solo::StepKernel k = nullptr;
-    if (streamlined) k = solo::fast_kernel(s->bits_m, s->bits_v, s->block, a.param_bf16 != 0, plain);
+    if (streamlined) k = solo::fast_kernel(s->bits_m, s->bits_v, s->block, a.param_bf16 != 0, plain, a.only_partial != 0);
     size_t dyn_smem = k ? solo::fast_kernel_smem(s->bits_m, s->bits_v) : 0;
     if (!k) k = solo::step_kernel(s->bits_m, s->bits_v, cta_group);
     if (!k) return SOLO_EINVAL;

@@ -70,6 +70,17 @@ struct StepArgs {
 };
 
 // ---------------------------------------------------------------------------
+// Programmatic dependent launch.  Every step kernel is launched so that its CTAs may be placed while the
+// kernel before it on the stream still runs (its launch latency, 2 to 3 us, is hidden); it touches global memory only
+// after that kernel has completed (pdl_wait), and only then lets the kernel after it be placed (pdl_release).  The
+// launch for the tiles that are not full shares no tile with the one for the full tiles before it: it
+// does not wait for that one's end before its work, but its first CTA does before it ends (whoever waits for the
+// second launch has waited for both).  The first launch releases it only after its own pdl_wait, so the inputs are complete.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// ---------------------------------------------------------------------------
 // log2 / exp2 as fixed IEEE operation sequences (see the block comment above).
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ float log2_sp(float x) {
@@ -289,11 +300,102 @@ __device__ __forceinline__ int find_tensor(const int64_t* __restrict__ start, in
     return lo;
 }
 
+// Walk of a launch with StepArgs::only_partial over the tiles the sixteen-per-thread kernel left: the last tile of
+// every aligned tensor that does not end on a tile, all tiles of tensors that are not 16-byte aligned.  The tensors
+// are dealt to the CTAs in turn; an unaligned tensor of more than ALONE tiles is shared by all of them afterwards.
+// (A contiguous share of the launch's tiles per CTA gave one CTA all the short vectors of a layer, one
+// after the other: 18 us for the GPT-125M-shaped set, 141 us for the ragged set.)  Uniform over the CTA.
+// It lives in shared memory and behind a call: in registers it made the streamlined kernel spill (1 Mi elements 7.7 ->
+// 9.5 us).
+struct PartialWalk {
+    static constexpr int ALONE = 16;
+    int tensor;                                  // the tile handed out: its tensor, its position there
+    int64_t tin;
+    int64_t end;                                 // tiles [tin + 1, end) of the tensor are still to do (shared: every grid-th)
+    int group, i;                                // shared tensors: first of the group looked at, position in it
+    int shared;                                  // 0: tensors dealt in turn, 1: unaligned tensors shared by all CTAs
+    unsigned char flag[CTA];
+};
+__device__ __forceinline__ void partial_walk_begin(PartialWalk& w) {
+    if (threadIdx.x == 0) {
+        w.tensor = (int)blockIdx.x - (int)gridDim.x;
+        w.tin = 0;
+        w.end = 0;
+        w.group = -CTA;
+        w.i = CTA;
+        w.shared = 0;
+    }
+}
+// Moves on to the CTA's next tile within the launch's range; false: none left.  All threads of the CTA, converged.
+__device__ __noinline__ inline bool partial_walk_next(const StepArgs& a, PartialWalk& w) {
+    auto aligned = [&](int t) {
+        return (((uintptr_t)(a.param_list ? a.param_list[t] : a.param_single) |
+                 (uintptr_t)(a.grad_list ? a.grad_list[t] : a.grad_single)) & 15u) == 0;
+    };
+    __syncthreads();
+    int t = w.tensor, group = w.group, i = w.i, shared = w.shared;
+    int64_t tin = w.tin + (shared ? gridDim.x : 1), end = w.end;
+    bool found = false;
+    for (;;) {
+        for (; tin < end; tin += shared ? gridDim.x : 1) {
+            const int64_t tile = __ldg(a.tile_start + t) + tin;
+            found = tile >= a.tile_first && tile < a.total_tiles;
+            if (found) break;
+        }
+        if (found) break;
+        if (!shared) {
+            t += (int)gridDim.x;
+            if (t < a.num_tensors) {
+                const int64_t n = __ldg(a.numel + t), tiles = (n + TILE - 1) / TILE;
+                tin = end = 0;
+                if (a.numel_check != nullptr && __ldg(a.numel_check + t) != n) {
+                    if (threadIdx.x == 0) atomicOr(a.status, 1);
+                } else if (aligned(t)) {
+                    tin = n / TILE;
+                    end = tiles;
+                } else if (tiles <= PartialWalk::ALONE) {
+                    end = tiles;
+                }
+                continue;
+            }
+            shared = 1;
+        }
+        while (i < CTA && !w.flag[i]) ++i;
+        if (i == CTA) {                                          // the next group of as many tensors as the CTA has threads
+            group += CTA;
+            if (group >= a.num_tensors) break;
+            const int mine = group + (int)threadIdx.x;
+            const bool f = mine < a.num_tensors && __ldg(a.numel + mine) > (int64_t)PartialWalk::ALONE * TILE && !aligned(mine) &&
+                           (a.numel_check == nullptr || __ldg(a.numel_check + mine) == __ldg(a.numel + mine));
+            __syncthreads();                                     // the flags of the last group have been read
+            w.flag[threadIdx.x] = f;
+            if (__syncthreads_count(f)) i = 0;
+            tin = end = 0;
+            continue;
+        }
+        t = group + i;
+        ++i;
+        tin = blockIdx.x;
+        end = (__ldg(a.numel + t) + TILE - 1) / TILE;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        w.tensor = t;
+        w.tin = tin;
+        w.end = end;
+        w.group = group;
+        w.i = i;
+        w.shared = shared;
+    }
+    __syncthreads();
+    return found;
+}
+
 // ---------------------------------------------------------------------------
 // The fused step.
 // ---------------------------------------------------------------------------
 template <int BM, int BV, bool CTA_GROUP>
-__global__ void __launch_bounds__(CTA) solo_step_kernel(const StepArgs a) {
+__global__ void __launch_bounds__(CTA) solo_step_kernel(const __grid_constant__ StepArgs a) {
     constexpr int KM = 1 << BM, KV = 1 << BV;
     __shared__ float s_y[KM];
     __shared__ float s_mid[KM];
@@ -305,6 +407,8 @@ __global__ void __launch_bounds__(CTA) solo_step_kernel(const StepArgs a) {
     __shared__ uint32_t s_red[8];
 
     const int tid = threadIdx.x;
+    if (!a.only_partial) pdl_wait();
+    pdl_release();
     for (int i = tid; i < KM; i += CTA) {
         s_y[i] = a.tables[i];
         if (i < KM - 1) {
@@ -327,16 +431,21 @@ __global__ void __launch_bounds__(CTA) solo_step_kernel(const StepArgs a) {
     const int gl = tid & (G - 1);                              // thread within its block
     const bool bf16p = a.param_bf16 != 0;
 
-    // Tiles are dealt out in turn.  After a launch that did the full tiles of the aligned tensors
-    // (only_partial) a CTA takes a contiguous share instead and jumps over each tensor's full tiles, so
-    // that it visits a few tiles per tensor of its share rather than every tile of the launch.
-    const int64_t share = (a.total_tiles - a.tile_first + gridDim.x - 1) / gridDim.x;
-    const int64_t tile_begin = a.only_partial ? min(a.tile_first + (int64_t)blockIdx.x * share, a.total_tiles)
-                                              : a.tile_first + blockIdx.x;
-    const int64_t tile_end = a.only_partial ? min(tile_begin + share, a.total_tiles) : a.total_tiles;
-    const int64_t stride = a.only_partial ? 1 : (int64_t)gridDim.x;
-    for (int64_t tile = tile_begin; tile < tile_end; tile += stride) {
-        const int tensor = a.num_tensors > 1 ? find_tensor(a.tile_start, a.num_tensors, tile) : 0;
+    // Tiles are dealt out in turn; after a launch that did the full tiles of the aligned tensors, the rest (PartialWalk).
+    __shared__ PartialWalk walk;
+    partial_walk_begin(walk);
+    for (int64_t tile = a.tile_first + (int64_t)blockIdx.x - gridDim.x;;) {
+        int tensor;
+        if (a.only_partial) {
+            __syncwarp();                                      // (groups of a warp leave a tile one by one)
+            if (!partial_walk_next(a, walk)) break;
+            tensor = walk.tensor;
+            tile = __ldg(a.tile_start + tensor) + walk.tin;
+        } else {
+            tile += gridDim.x;
+            if (tile >= a.total_tiles) break;
+            tensor = a.num_tensors > 1 ? find_tensor(a.tile_start, a.num_tensors, tile) : 0;
+        }
         const int64_t n = __ldg(a.numel + tensor);
         if (a.numel_check != nullptr && __ldg(a.numel_check + tensor) != n) {
             if (tid == 0) atomicOr(a.status, 1);
@@ -346,10 +455,6 @@ __global__ void __launch_bounds__(CTA) solo_step_kernel(const StepArgs a) {
         char* pbase = (char*)(a.param_list ? a.param_list[tensor] : a.param_single);
         const char* gbase = (const char*)(a.grad_list ? a.grad_list[tensor] : a.grad_single);
         const bool aligned = ((((uintptr_t)pbase) | ((uintptr_t)gbase)) & 15u) == 0;
-        if (a.only_partial && aligned && tin < n / TILE) {           // another launch did the full tiles:
-            tile += n / TILE - tin - 1;                               // on to the tensor's first tile that is not full
-            continue;
-        }
         const int64_t e0 = tin * TILE + (int64_t)tid * EPT;
         const int64_t blk_in_tensor = e0 / B;
         const int64_t blk_elem0 = blk_in_tensor * B;
@@ -565,6 +670,7 @@ __global__ void __launch_bounds__(CTA) solo_step_kernel(const StepArgs a) {
             a.alpha[jb] = al_new;
         }
     }
+    if (a.only_partial && blockIdx.x == 0) pdl_wait();
 }
 
 // ---------------------------------------------------------------------------

@@ -1060,8 +1060,9 @@ __device__ __forceinline__ void fast_tile(const StepArgs& a, FastShared<BM, BV>&
     }
 }
 
-template <int BM, int BV, int G, bool PBF, bool PLAIN>
-__global__ void __launch_bounds__(CTA, (BM == 8 || BV == 8) ? 3 : 4) solo_step_fast_kernel(const StepArgs a) {
+// TAILS: the launch after the sixteen-per-thread kernel, for the tiles that one left (PartialWalk); else all tiles.
+template <int BM, int BV, int G, bool PBF, bool PLAIN, bool TAILS>
+__global__ void __launch_bounds__(CTA, (BM == 8 || BV == 8) ? 3 : 4) solo_step_fast_kernel(const __grid_constant__ StepArgs a) {
     constexpr int KM = 1 << BM;
     extern __shared__ __align__(16) unsigned char fast_smem[];   // sizeof(FastShared<BM, BV>), above the static 48 KB limit
     FastShared<BM, BV>& s = *reinterpret_cast<FastShared<BM, BV>*>(fast_smem);
@@ -1069,6 +1070,8 @@ __global__ void __launch_bounds__(CTA, (BM == 8 || BV == 8) ? 3 : 4) solo_step_f
     __shared__ float s_mid[KM];
     __shared__ float4 s_mid4[4];     // 4-bit first moments: per quarter of the codebook, its three inner midpoints times -2^100
     const int tid = threadIdx.x;
+    if constexpr (!TAILS) pdl_wait();
+    pdl_release();
     for (int i = tid; i < KM; i += CTA) {
         s_y[i] = a.tables[i];
         if (i < KM - 1) s_mid[i] = a.tables[KM + i];
@@ -1096,7 +1099,7 @@ __global__ void __launch_bounds__(CTA, (BM == 8 || BV == 8) ? 3 : 4) solo_step_f
     const int step = G == CTA ? (int)gridDim.x : 1;            // to the CTA's next tile
     const int tile_begin = (int)min(a.tile_first + (int64_t)blockIdx.x * (G == CTA ? 1 : share), a.total_tiles);
     const int tile_end = G == CTA ? (int)a.total_tiles : (int)min((int64_t)tile_begin + share, a.total_tiles);
-    int tensor = (a.num_tensors > 1 && tile_begin < tile_end ? find_tensor(a.tile_start, a.num_tensors, tile_begin) : 0) - 1;
+    int tensor = (!TAILS && a.num_tensors > 1 && tile_begin < tile_end ? find_tensor(a.tile_start, a.num_tensors, tile_begin) : 0) - 1;
     int t_lo = 0, t_hi = 0, full_tiles = 0;      // the tensor's tiles [t_lo, t_hi); its first full_tiles are full
     int64_t jb0 = 0;
     char* pbase = nullptr;
@@ -1104,42 +1107,54 @@ __global__ void __launch_bounds__(CTA, (BM == 8 || BV == 8) ? 3 : 4) solo_step_f
     bool skip = false;
     Ahead ah;
     int par = 0;
-    for (int tile = tile_begin; tile < tile_end; tile += step) {
-        if (tile >= t_hi) {
-            do {
-                ++tensor;
-                t_hi = (int)__ldg(a.tile_start + tensor + 1);
-            } while (tile >= t_hi);
-            t_lo = (int)__ldg(a.tile_start + tensor);
-            const int64_t n = __ldg(a.numel + tensor);
-            jb0 = __ldg(a.block_start + tensor);
-            pbase = (char*)(a.param_list ? a.param_list[tensor] : a.param_single);
-            gbase = (const char*)(a.grad_list ? a.grad_list[tensor] : a.grad_single);
-            const bool aligned = ((((uintptr_t)pbase) | ((uintptr_t)gbase)) & 15u) == 0;
-            full_tiles = aligned ? (int)(n / TILE) : 0;
-            skip = a.numel_check != nullptr && __ldg(a.numel_check + tensor) != n;
-            if (skip && tid == 0) atomicOr(a.status, 1);
+    if constexpr (TAILS) {
+        __shared__ PartialWalk walk;
+        partial_walk_begin(walk);
+        while (partial_walk_next(a, walk)) {
+            const int t = walk.tensor, tin = (int)walk.tin;
+            fast_tile<BM, BV, G, false, PBF, PLAIN>(
+                a, s, s_y, s_mid, s_mid4, (char*)(a.param_list ? a.param_list[t] : a.param_single),
+                (const char*)(a.grad_list ? a.grad_list[t] : a.grad_single), __ldg(a.numel + t), tin,
+                __ldg(a.block_start + t) + (int64_t)tin * (CTA / G), t, par, ah, false, 0, 0);
+            par ^= 1;
         }
-        if (skip) continue;
-        const int tin = tile - t_lo;
-        if (a.only_partial && tin < full_tiles) {                 // another launch did the full tiles
-            if (step == 1) tile = t_lo + full_tiles - 1;          // on to the tensor's first tile that is not full
-            continue;
-        }
-        const int64_t jb_tile = jb0 + (int64_t)tin * (CTA / G);
-        if (tin < full_tiles)
-            fast_tile<BM, BV, G, true, PBF, PLAIN>(a, s, s_y, s_mid, s_mid4, pbase, gbase, 0, tin, jb_tile, tensor, par, ah,
-                                       tin + step < full_tiles && tile + step < tile_end, step, tile);
-        else
-            fast_tile<BM, BV, G, false, PBF, PLAIN>(a, s, s_y, s_mid, s_mid4, pbase, gbase, __ldg(a.numel + tensor), tin, jb_tile,
-                                                    tensor, par, ah, false, 0, tile);
-        par ^= 1;
+        if (blockIdx.x == 0) pdl_wait();
+        return;
     }
-    // A thread that gave up on a copy waits once more, again bounded, for the last one that was issued,
-    // so that no copy is still writing to a stage when the CTA's shared memory is released.
-    if (ah.failed && ah.fill > 0) {
-        const uint32_t last = ah.fill - 1u;
-        mbar_wait(smem_u32(&s.mbar[last & 1u]), (last >> 1) & 1u);
+    if constexpr (!TAILS) {
+        for (int tile = tile_begin; tile < tile_end; tile += step) {
+            if (tile >= t_hi) {
+                do {
+                    ++tensor;
+                    t_hi = (int)__ldg(a.tile_start + tensor + 1);
+                } while (tile >= t_hi);
+                t_lo = (int)__ldg(a.tile_start + tensor);
+                const int64_t n = __ldg(a.numel + tensor);
+                jb0 = __ldg(a.block_start + tensor);
+                pbase = (char*)(a.param_list ? a.param_list[tensor] : a.param_single);
+                gbase = (const char*)(a.grad_list ? a.grad_list[tensor] : a.grad_single);
+                const bool aligned = ((((uintptr_t)pbase) | ((uintptr_t)gbase)) & 15u) == 0;
+                full_tiles = aligned ? (int)(n / TILE) : 0;
+                skip = a.numel_check != nullptr && __ldg(a.numel_check + tensor) != n;
+                if (skip && tid == 0) atomicOr(a.status, 1);
+            }
+            if (skip) continue;
+            const int tin = tile - t_lo;
+            const int64_t jb_tile = jb0 + (int64_t)tin * (CTA / G);
+            if (tin < full_tiles)
+                fast_tile<BM, BV, G, true, PBF, PLAIN>(a, s, s_y, s_mid, s_mid4, pbase, gbase, 0, tin, jb_tile, tensor, par, ah,
+                                           tin + step < full_tiles && tile + step < tile_end, step, tile);
+            else
+                fast_tile<BM, BV, G, false, PBF, PLAIN>(a, s, s_y, s_mid, s_mid4, pbase, gbase, __ldg(a.numel + tensor), tin, jb_tile,
+                                                        tensor, par, ah, false, 0, tile);
+            par ^= 1;
+        }
+        // A thread that gave up on a copy waits once more, again bounded, for the last one that was issued,
+        // so that no copy is still writing to a stage when the CTA's shared memory is released.
+        if (ah.failed && ah.fill > 0) {
+            const uint32_t last = ah.fill - 1u;
+            mbar_wait(smem_u32(&s.mbar[last & 1u]), (last >> 1) & 1u);
+        }
     }
 }
 

@@ -1200,6 +1200,8 @@ __global__ void __launch_bounds__(CTA16, ctas16<BM, BV, G, MODES>()) solo_step_f
     __shared__ float4 s_nv[EXT ? 8 : 1];                     // its midpoints times -2^100 (rows as the tile function reads them)
     __shared__ float4 s_mid4[4];             // 4-bit first moments: per quarter of the codebook, its three inner midpoints times -2^100
     const int tid = threadIdx.x;
+    pdl_wait();
+    pdl_release();
     for (int i = tid; i < KM; i += CTA16) {
         s_y[i] = a.tables[i];
         s_mid[i] = i < KM - 1 ? a.tables[KM + i] : __int_as_float(0x7f800000);

@@ -1,9 +1,13 @@
-// Instantiations of the streamlined step kernel for one first-moment width (SOLO_BM = 2, 3, 4, 8).
+// Instantiations of the streamlined step kernel for one first-moment width (SOLO_BM = 2, 3, 4, 8): for all tiles
+// (SOLO_TAILS = 0) or for those the sixteen-per-thread kernel leaves (SOLO_TAILS = 1).
 #include "solo_dispatch.h"
 #include "solo_fast.cuh"
 
 #ifndef SOLO_BM
 #error "compile with -DSOLO_BM=2|3|4|8"
+#endif
+#ifndef SOLO_TAILS
+#error "compile with -DSOLO_TAILS=0|1"
 #endif
 
 #define SOLO_CAT_(a, b) a##b
@@ -11,13 +15,18 @@
 
 namespace solo {
 
-#define SOLO_ROW(BV, PBF, PLAIN)                                                                            \
-    {solo_step_fast_kernel<SOLO_BM, BV, 8, PBF, PLAIN>, solo_step_fast_kernel<SOLO_BM, BV, 16, PBF, PLAIN>, \
-     solo_step_fast_kernel<SOLO_BM, BV, 32, PBF, PLAIN>, solo_step_fast_kernel<SOLO_BM, BV, 256, PBF, PLAIN>}
+#define SOLO_ROW(BV, PBF, PLAIN)                                                                                          \
+    {solo_step_fast_kernel<SOLO_BM, BV, 8, PBF, PLAIN, SOLO_TAILS>, solo_step_fast_kernel<SOLO_BM, BV, 16, PBF, PLAIN, SOLO_TAILS>, \
+     solo_step_fast_kernel<SOLO_BM, BV, 32, PBF, PLAIN, SOLO_TAILS>, solo_step_fast_kernel<SOLO_BM, BV, 256, PBF, PLAIN, SOLO_TAILS>}
 #define SOLO_PLANE(PBF, PLAIN) \
     {SOLO_ROW(2, PBF, PLAIN), SOLO_ROW(3, PBF, PLAIN), SOLO_ROW(4, PBF, PLAIN), SOLO_ROW(8, PBF, PLAIN)}
 
-StepKernel SOLO_CAT(fast_kernel_bm, SOLO_BM)(int bv_index, int block, bool param_bf16, bool plain) {
+#if SOLO_TAILS
+#define SOLO_FAST_NAME SOLO_CAT(fast_tails_kernel_bm, SOLO_BM)
+#else
+#define SOLO_FAST_NAME SOLO_CAT(fast_kernel_bm, SOLO_BM)
+#endif
+StepKernel SOLO_FAST_NAME(int bv_index, int block, bool param_bf16, bool plain) {
     static const StepKernel table[2][2][4][4] = {
         {SOLO_PLANE(false, false), SOLO_PLANE(true, false)},
         {SOLO_PLANE(false, true), SOLO_PLANE(true, true)},
@@ -27,7 +36,7 @@ StepKernel SOLO_CAT(fast_kernel_bm, SOLO_BM)(int bv_index, int block, bool param
     return table[plain ? 1 : 0][param_bf16 ? 1 : 0][bv_index][g];
 }
 
-#if SOLO_BM == 2
+#if SOLO_BM == 2 && !SOLO_TAILS
 // Exhaustive check of the error model used above: for every binary32 x with bit pattern
 // in [lo, hi] (positive, finite) the largest value of
 //   |lg2.approx(x) - log2_sp(x)| - (LG2_REL / 2) |log2_sp(x)|
