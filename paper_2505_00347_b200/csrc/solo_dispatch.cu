@@ -40,6 +40,7 @@ StepKernel fast16_kernel(int bits_m, int bits_v, int block, bool param_bf16, int
         case 64: return w8 ? SOLO_PICK16(4, _w8) : SOLO_PICK16(4, );
         case 128: return w8 ? SOLO_PICK16(8, _w8) : SOLO_PICK16(8, );
         case 256: return w8 ? SOLO_PICK16(16, _w8) : SOLO_PICK16(16, );
+        case 2048: return w8 ? SOLO_PICK16(128, _w8) : SOLO_PICK16(128, );
         default: return nullptr;
     }
 #undef SOLO_PICK16
@@ -51,6 +52,7 @@ size_t fast16_kernel_smem(int bits_m, int bits_v, int block, bool param_bf16) {
         case 64: return w8 ? fast16_smem_g4_w8(bits_m, bits_v, param_bf16) : fast16_smem_g4(bits_m, bits_v, param_bf16);
         case 128: return w8 ? fast16_smem_g8_w8(bits_m, bits_v, param_bf16) : fast16_smem_g8(bits_m, bits_v, param_bf16);
         case 256: return w8 ? fast16_smem_g16_w8(bits_m, bits_v, param_bf16) : fast16_smem_g16(bits_m, bits_v, param_bf16);
+        case 2048: return w8 ? fast16_smem_g128_w8(bits_m, bits_v, param_bf16) : fast16_smem_g128(bits_m, bits_v, param_bf16);
         default: return 0;
     }
 }

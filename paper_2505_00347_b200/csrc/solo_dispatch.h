@@ -43,7 +43,7 @@ StepKernel fast_tails_kernel_bm4(int bv_index, int block, bool param_bf16, bool 
 StepKernel fast_tails_kernel_bm8(int bv_index, int block, bool param_bf16, bool plain);
 // `tails`: the kernel for the tiles that the sixteen-per-thread kernel leaves
 StepKernel fast_kernel(int bits_m, int bits_v, int block, bool param_bf16, bool plain, bool tails);
-// Sixteen elements per thread: blocks of 64, 128 or 256, fp32 or bf16 parameters; `modes`: 0 as `plain` for
+// Sixteen elements per thread: fp32 or bf16 parameters; `modes`: 0 as `plain` for
 // fast_kernel, 1 the modes fast_kernel reads at run time, 2 those plus Eq. 5 rounding and the baseline
 // second-moment codebooks; full tiles
 // of aligned tensors only (the rest is left to a launch of the streamlined or of the general kernel with
@@ -62,6 +62,7 @@ constexpr int CTA16 = 128;         // threads per CTA of that kernel
 SOLO_DECLARE16(4)
 SOLO_DECLARE16(8)
 SOLO_DECLARE16(16)
+SOLO_DECLARE16(128)
 #undef SOLO_DECLARE16
 StepKernel fast16_kernel(int bits_m, int bits_v, int block, bool param_bf16, int modes);
 size_t fast16_kernel_smem(int bits_m, int bits_v, int block, bool param_bf16);

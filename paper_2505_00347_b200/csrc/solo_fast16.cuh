@@ -1,5 +1,5 @@
 // Sixteen elements per thread: the streamlined step for the plain step (2/3/4/8-bit states, blocks of
-// 64, 128 or 256, fp32 or bf16 parameters; no L2 term in the gradient, no AdaBelief, base from the
+// 64, 128, 256 or 2048, fp32 or bf16 parameters; no L2 term in the gradient, no AdaBelief, base from the
 // p-quantile, xi drawn: MODES = 0).  Two more instantiations read other modes from the arguments:
 // MODES = 1 the L2 term, AdaBelief, a fixed base, no dither; MODES = 2 also stochastic rounding of the
 // first moment (Eq. 5) and the baseline second-moment codebooks (a fixed level table instead of the
@@ -11,7 +11,7 @@
 // slot.  2^27 elements, block 128: 2/3 bit 436 -> 416 us, 4/4 bit 491 -> 455 us, 2/2 bit 429 -> 395 us, with the
 // L2 term 596 -> 508 us.  What changes is the work split.  A CTA of 128 threads owns a tile of 2048 consecutive elements, a thread
 // sixteen of them, a block of 64 / 128 / 256 elements G = 4 / 8 / 16 consecutive lanes, a warp eight,
-// four or two blocks.  The per-thread work that does not depend on the element count (waiting for the
+// four or two blocks; a block of 2048 the whole CTA (G = 128).  The per-thread work that does not depend on the element count (waiting for the
 // staged inputs, addressing, the level tables, the exchange with the first warp, the rounds of the
 // selection) is spent once per sixteen elements instead of once per eight.
 //
@@ -57,12 +57,14 @@ static_assert(CTA16 * EPT16 == TILE, "same tile as the other kernels");
 // memory: seven, six where the modes' tables come on top (8/8 bit five 516, six 498, seven 496 us; Eq. 5 four 830, five
 // 799, six 763 us).
 template <int BM, int BV, int G, int MODES>
-constexpr int ctas16() { return BM == 8 || BV == 8 ? (MODES == 2 ? 6 : 7) : BM == 4 || G == 16 ? 7 : 8; }
+constexpr int ctas16() { return BM == 8 || BV == 8 ? (MODES == 2 ? 6 : 7) : BM == 4 || G >= 16 ? 7 : 8; }
 
-// G: lanes per block (4, 8 or 16 for blocks of 64, 128 or 256 elements); NG = 128 / G blocks per tile.
+// G: lanes per block (4, 8, 16 or 128 for blocks of 64, 128, 256 or 2048 elements); NG = 128 / G blocks per tile.
 template <int BM, int BV, bool PBF, int G>
 struct Fast16Shared {
     static constexpr int NG = CTA16 / G;
+    static constexpr int LG = G < 32 ? G : 32;                       // lanes that build a block's level tables,
+    static constexpr int NT = CTA16 / LG;                            // and how many there are: a block of 2048 has one per warp
     // G = 4: sorted keys of the threads, one column per thread: row j holds the (j+2)-th smallest key, row 15 a
     // sentinel above every key
     uint32_t sort[G == 4 ? 16 : 1][G == 4 ? CTA16 : 1];
@@ -77,16 +79,24 @@ struct Fast16Shared {
     // are multiplied on per element.  With G = 16 that is all eight bits, and Delta_v is in the table.  8-bit first
     // moments: the codebook itself, scaled per element.
     static constexpr int TB = BV != 8 ? BV : G == 4 ? 6 : G == 8 ? 7 : 8;
-    alignas(16) float tab_v[NG][BV == 8 ? (1 << TB) + 8 : BV == 2 && PAIRS ? 32 : 1 << BV];
-    alignas(8) float tab_m[BM == 8 ? 1 : NG][BM == 8 ? 2 : BM == 2 && PAIRS ? 32 : 1 << BM];
+    static constexpr int TAB8 = (1 << TB) + (G == 128 ? 64 : 8);
+    alignas(16) float tab_v[NT][BV == 8 ? TAB8 : BV == 2 && PAIRS ? 32 : 1 << BV];
+    alignas(8) float tab_m[BM == 8 ? 1 : NT][BM == 8 ? 2 : BM == 2 && PAIRS ? 32 : 1 << BM];
     alignas(16) unsigned char lut_m[BM == 8 ? LUT8_M_BYTES : 16];        // cells of the signed codebook (solo_lut8.cuh)
     // 8-bit baseline second-moment codebook, in the place of tab_v, which it has no use for
     struct Codebook8 {
         unsigned char lut[LUT8_V_BYTES];
         float y[256], mid[256];              // mid[255]: +infinity
     };
-    static_assert(BV != 8 || sizeof(Codebook8) <= sizeof(float) * NG * ((1 << TB) + 8), "fits the table's place");
+    static_assert(BV != 8 || sizeof(Codebook8) <= sizeof(float) * NT * TAB8, "fits the table's place");
     __device__ Codebook8& v8() { return *reinterpret_cast<Codebook8*>(&tab_v[0][0]); }
+    // Blocks of 2048: what the four warps exchange, the histogram and the list of the selection (select_cta16)
+    struct Cta {
+        uint32_t m[4], v[4], lo[4], failed[4];   // per warp: maxima of |m^| and v^, minimum of v^, gave up on the tile's inputs
+        uint32_t hist[256], list[512], fill;
+    };
+    alignas(16) unsigned char cta_bytes[G == 128 ? sizeof(Cta) : 16];
+    __device__ Cta& cta() { return *reinterpret_cast<Cta*>(cta_bytes); }
     // Exchange with the first warp.  One copy is enough: xin is written before the tile's first
     // barrier and read between its two barriers, xout is written between the barriers and read
     // after the second, and nobody writes either again before passing those barriers.
@@ -100,7 +110,7 @@ struct Fast16Shared {
         alignas(16) unsigned char g[TILE * 2];                // 2048 bf16 gradients
         uint32_t cm[64 * BM + 4];        // packed codes of the tile: 256 * bits bytes, from a 16-byte boundary
         uint32_t cv[64 * BV + 4];
-        float sc[3][NG + 4];             // Delta_m, Delta_v, alpha of the tile's blocks, from a 16-byte boundary
+        float sc[3][NG >= 4 ? NG + 4 : 8];   // Delta_m, Delta_v, alpha of the tile's blocks, from a 16-byte boundary
     };
     alignas(16) Stage stage;
     alignas(8) unsigned long long mbar;      // the stage's copies
@@ -242,7 +252,9 @@ __device__ __forceinline__ uint32_t group_max16(uint32_t x) {
 // maximum serve both groups of the warp, the upper group's keys going in complemented (vx = ~0 there, else 0).
 template <int G>
 __device__ __forceinline__ uint32_t group_min31(uint32_t x, uint32_t vx) {
-    if constexpr (G == 16) {
+    if constexpr (G == 32) {
+        return __reduce_min_sync(0xffffffffu, x);
+    } else if constexpr (G == 16) {
         const uint32_t lo = __reduce_min_sync(0xffffffffu, x ^ vx);
         const uint32_t up = __reduce_max_sync(0xffffffffu, x ^ vx);
         return (vx ? up : lo) ^ vx;
@@ -256,7 +268,9 @@ template <int G>
 __device__ __forceinline__ int group_count4(bool p0, bool p1, bool p2, bool p3, int lane) {
     const uint32_t b0 = __ballot_sync(0xffffffffu, p0), b1 = __ballot_sync(0xffffffffu, p1);
     const uint32_t b2 = __ballot_sync(0xffffffffu, p2), b3 = __ballot_sync(0xffffffffu, p3);
-    if constexpr (G == 16) {
+    if constexpr (G == 32) {
+        return (__popc(b0) + __popc(b1)) + (__popc(b2) + __popc(b3));
+    } else if constexpr (G == 16) {
         const uint32_t sel = (lane & 16) ? 0x7632u : 0x5410u;
         return __popc(__byte_perm(b0, b1, sel)) + __popc(__byte_perm(b2, b3, sel));
     } else {
@@ -318,7 +332,7 @@ __device__ __forceinline__ uint32_t select_rank16(uint32_t (&l)[4][4], const int
     for (int it = 0; it < k && __any_sync(0xffffffffu, go); ++it) go = round();
     uint32_t h[4] = {l[0][0], l[1][0], l[2][0], l[3][0]};
     cswap(h[0], h[1]); cswap(h[2], h[3]); cswap(h[0], h[2]); cswap(h[1], h[3]); cswap(h[1], h[2]);
-    const uint32_t gmask = ((1u << G) - 1u) << (lane & ~(G - 1));
+    const uint32_t gmask = (G == 32 ? 0xFFFFFFFFu : (1u << (G & 31)) - 1u) << (lane & ~(G - 1));
     auto head_round = [&]() {
         const uint32_t t = group_min31<G>(h[1], vx);
         const bool p = h[0] <= t;
@@ -332,6 +346,106 @@ __device__ __forceinline__ uint32_t select_rank16(uint32_t (&l)[4][4], const int
 #pragma unroll 1
     for (int it = 0; it < k && __any_sync(0xffffffffu, go); ++it) head_round();
     return lanes_rank<G>(h[0], rem, lane);
+}
+
+__device__ __forceinline__ void sort_list4(uint32_t (&l)[4]) {
+    cswap(l[0], l[1]); cswap(l[2], l[3]); cswap(l[0], l[2]); cswap(l[1], l[3]); cswap(l[1], l[2]);
+}
+
+// A block of 2048: k-th smallest (1-based, duplicates counted) of the CTA's keys, sixteen per thread; lo and hi are the
+// smallest and the largest.  Returns it in every lane of the first warp (anything in the others).
+// With the eight-per-thread kernel's eleven-bit levels and five barriers each (2^27 elements) 2/2 bit took 602 us, 4/4 bit
+// 655, 8/8 bit 1028; here 491, 594, 667 (dynamic exponent for both moments, no selection: 1304 in the general
+// kernel, 438).  What is left is the wait for the first warp (barrier stalls 2.3 per issue).
+// The block's own range of key values is cut into 256 bins; every warp scans the histogram for itself, so that no
+// barrier is needed to publish the bin that holds the rank.  The bin's keys (a tenth of the block lies
+// in the lowest level of the last step's codes, so often two hundred of them side by side) are collected, up to 512, and
+// ranked by the first warp alone (select_rank16).  A fuller bin is cut again.  hist and fill are zero on entry and on exit.
+// All threads of the CTA, converged; three barriers in the usual case.
+template <class Cta>
+__device__ __forceinline__ uint32_t select_cta16(const uint32_t (&key)[EPT16], const int k, Cta& c, const uint32_t lo,
+                                                 const uint32_t hi, const int tid) {
+    const int lane = tid & 31, warp = tid >> 5;
+    if (hi == lo) return lo;                                      // (uniform)
+    int bits = 32 - __clz(hi - lo);                               // keys of interest: base <= key < base + 2^bits
+    uint32_t base = lo, kk = (uint32_t)k, cnt;
+    for (bool first = true;; first = false) {
+        const int shift = max(bits - 8, 0);
+#pragma unroll
+        for (int i = 0; i < EPT16; ++i) {
+            const uint32_t d = key[i] - base;
+            if (first || d < (1u << bits)) atomicAdd(&c.hist[d >> shift], 1u);
+        }
+        __syncthreads();
+        const uint4 h0 = reinterpret_cast<const uint4*>(c.hist)[2 * lane], h1 = reinterpret_cast<const uint4*>(c.hist)[2 * lane + 1];
+        const uint32_t h[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
+        const uint32_t mine = ((h[0] + h[1]) + (h[2] + h[3])) + ((h[4] + h[5]) + (h[6] + h[7]));
+        uint32_t incl = mine;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += t;
+        }
+        uint32_t run = incl - mine;                               // keys in the bins before this lane's
+        const int src = __ffs(__ballot_sync(0xffffffffu, kk <= incl)) - 1;      // the lane that holds the rank
+        uint32_t bin = 0, n = h[0];
+#pragma unroll
+        for (int j = 0; j < 7; ++j)
+            if (bin == (uint32_t)j && kk > run + h[j]) {
+                run += h[j];
+                bin = j + 1;
+                n = h[j + 1];
+            }
+        bin = __shfl_sync(0xffffffffu, 8u * (uint32_t)lane + bin, src);
+        kk -= __shfl_sync(0xffffffffu, run, src);
+        cnt = __shfl_sync(0xffffffffu, n, src);
+        base += bin << shift;
+        bits = shift;
+        if (shift == 0 || cnt <= 512u) break;
+        __syncthreads();                                          // every warp has read the histogram
+        c.hist[tid] = 0u;
+        c.hist[tid + CTA16] = 0u;
+        __syncthreads();
+    }
+    uint32_t x = base;
+    if (bits > 0) {
+        const uint32_t width = 1u << bits;
+        uint32_t mine = 0;
+#pragma unroll
+        for (int i = 0; i < EPT16; ++i) mine += key[i] - base < width ? 1u : 0u;
+        uint32_t incl = mine;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const uint32_t t = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d) incl += t;
+        }
+        uint32_t at = lane == 31 ? atomicAdd(&c.fill, incl) : 0u;
+        at = smem_u32(c.list) + 4u * (__shfl_sync(0xffffffffu, at, 31) + incl - mine);
+#pragma unroll
+        for (int i = 0; i < EPT16; ++i) {
+            // if (key[i] - base < width) c.list[at++] = key[i];
+            asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.u32 p, %1, %2;\n\t@p st.shared.u32 [%0], %3;\n\t@p add.u32 %0, %0, 4;\n\t}"
+                         : "+r"(at) : "r"(key[i] - base), "r"(width), "r"(key[i]) : "memory");
+        }
+    }
+    __syncthreads();
+    c.hist[tid] = 0u;                                             // (next counted into after the next tile's barriers)
+    c.hist[tid + CTA16] = 0u;
+    if (tid == CTA16 - 1) c.fill = 0u;
+    if (bits > 0 && warp == 0) {
+        uint32_t l[4][4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t j = (uint32_t)(lane + 32 * (4 * q + i));
+                l[q][i] = j < cnt ? c.list[j] : KEY_MAX;
+            }
+            sort_list4(l[q]);
+        }
+        x = select_rank16<32, 2>(l, (int)kk, lane);
+    }
+    return x;
 }
 
 // Four lanes per block: k-th smallest of the 64 keys, each lane's sixteen sorted, by popping one minimum per round
@@ -381,7 +495,8 @@ __device__ __forceinline__ void issue_tile_copy16(const StepArgs& a, Fast16Share
     // 16 bytes more (the state's arrays carry that slack), and read with an offset
     const int64_t bm0 = jb_tile * (2 * G * BM), bv0 = jb_tile * (2 * G * BV);
     const uint32_t bytes_m = 256 * BM + ((bm0 & 15) ? 16u : 0u), bytes_v = 256 * BV + ((bv0 & 15) ? 16u : 0u);
-    const uint32_t bytes_s = (NG + ((jb_tile & 3) ? 4u : 0u)) * 4u;
+    // (a single block's scalar lies within the 16 bytes that start at the boundary)
+    const uint32_t bytes_s = NG < 4 ? 16u : (NG + ((jb_tile & 3) ? 4u : 0u)) * 4u;
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
                  "r"((uint32_t)(TILE * (PBF ? 2 : 4) + TILE * 2) + bytes_m + bytes_v + 3u * bytes_s + extra_tx)
                  : "memory");
@@ -552,7 +667,9 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     // A warp in which any lane gave up leaves the tile alone: it stores nothing, flags its blocks
     // for the first warp (which stores the per-block scalars), and only keeps the CTA's barriers, the
     // copy-ahead and, if it is the first warp, the other warps' scalars going.
-    if (__any_sync(0xffffffffu, failed)) {
+    // A block of 2048 spans the CTA, which leaves the tile as a whole (below).
+    const bool gave_up = __any_sync(0xffffffffu, failed);
+    if (G != 128 && gave_up) {
         if (gl == 0) s.xin[grp] = make_uint4(0u, 0u, 0u, 1u);
         bar_sync16(1);
         if (tid == 32) produce_tile16<BM, BV, PBF, G>(a, s, s.desc[(fill + 1u) & 1u]);
@@ -576,8 +693,10 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
         const float dm = st.sc[0][so], dv = st.sc[1][so], al = st.sc[2][so];
 
         // per-block level tables (Eq. 2), built by the block's G lanes
-        float* const tab_vf = s.tab_v[grp];
-        float* const tab_mf = s.tab_m[BM == 8 ? 0 : grp];
+        constexpr int LG = Shared::LG;
+        const int tl = tid & (LG - 1), tt = tid / LG;             // lane among the table's, its number
+        float* const tab_vf = s.tab_v[tt];
+        float* const tab_mf = s.tab_m[BM == 8 ? 0 : tt];
         float a2[BV];
         {
             a2[0] = al;
@@ -585,43 +704,46 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
             for (int i = 1; i < BV; ++i) a2[i] = a2[i - 1] * a2[i - 1];
             auto level_v = [&](uint32_t k) { return (vtab ? s_yv[k] : pow_sm<BV>(a2, k)) * dv; };
             if constexpr (BV == 8) {
-                // entries 2 gl, 2 gl + 1 from the bits that tell the lanes apart, then doubled bit by bit: entry q is
+                // entries 2 tl, 2 tl + 1 from the bits that tell the lanes apart, then doubled bit by bit: entry q is
                 // entry (q without its top bit) times the top bit's factor, as in the chain of pow_sm
                 if (!vtab) {
-                    constexpr int LB = Shared::TB - 3;            // bits of 2 gl + 1
+                    constexpr int LB = LG == 4 ? 3 : LG == 8 ? 4 : LG == 16 ? 5 : 6;      // bits of 2 tl + 1
+                    constexpr int DB = Shared::TB - LB;
                     float f[LB];
 #pragma unroll
                     for (int i = 0; i < LB; ++i) f[i] = a2[i];
-                    F2 e[8];
-                    e[0] = F2::pack(pow_sm<LB>(f, (uint32_t)(2 * gl)), pow_sm<LB>(f, (uint32_t)(2 * gl + 1)));
+                    F2 e[1 << DB];
+                    e[0] = F2::pack(pow_sm<LB>(f, (uint32_t)(2 * tl)), pow_sm<LB>(f, (uint32_t)(2 * tl + 1)));
 #pragma unroll
-                    for (int b = 0; b < 3; ++b)
+                    for (int b = 0; b < DB; ++b)
 #pragma unroll
                         for (int i = 0; i < (1 << b); ++i) e[i + (1 << b)] = mul2(e[i], F2::dup(a2[LB + b]));
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
+                    for (int i = 0; i < (1 << DB); ++i) {
                         const F2 t = Shared::TB == 8 ? mul2(e[i], F2::dup(dv)) : e[i];
-                        *reinterpret_cast<float2*>(tab_vf + 2 * gl + (i << LB)) = make_float2(t.lo(), t.hi());
+                        *reinterpret_cast<float2*>(tab_vf + 2 * tl + (i << LB)) = make_float2(t.lo(), t.hi());
                     }
                 }
             } else if constexpr (BV == 2 && Shared::PAIRS) {
 #pragma unroll
-                for (int r0 = 0; r0 < 16; r0 += G)
-                    *reinterpret_cast<float2*>(tab_vf + 2 * (r0 + gl)) = make_float2(level_v((r0 + gl) & 3), level_v((r0 + gl) >> 2));
+                for (int r0 = 0; r0 < 16; r0 += LG)
+                    if (r0 + tl < 16)
+                        *reinterpret_cast<float2*>(tab_vf + 2 * (r0 + tl)) = make_float2(level_v((r0 + tl) & 3), level_v((r0 + tl) >> 2));
             } else {
 #pragma unroll
-                for (int r0 = 0; r0 < KV; r0 += G)
-                    if (r0 + gl < KV) tab_vf[r0 + gl] = level_v(r0 + gl);
+                for (int r0 = 0; r0 < KV; r0 += LG)
+                    if (r0 + tl < KV) tab_vf[r0 + tl] = level_v(r0 + tl);
             }
             if constexpr (BM == 8) {
             } else if constexpr (BM == 2 && Shared::PAIRS) {
 #pragma unroll
-                for (int r0 = 0; r0 < 16; r0 += G)
-                    *reinterpret_cast<float2*>(tab_mf + 2 * (r0 + gl)) = make_float2(s_y[(r0 + gl) & 3] * dm, s_y[(r0 + gl) >> 2] * dm);
+                for (int r0 = 0; r0 < 16; r0 += LG)
+                    if (r0 + tl < 16)
+                        *reinterpret_cast<float2*>(tab_mf + 2 * (r0 + tl)) = make_float2(s_y[(r0 + tl) & 3] * dm, s_y[(r0 + tl) >> 2] * dm);
             } else {
 #pragma unroll
-                for (int r0 = 0; r0 < KM; r0 += G)
-                    if (r0 + gl < KM) tab_mf[r0 + gl] = s_y[r0 + gl] * dm;
+                for (int r0 = 0; r0 < KM; r0 += LG)
+                    if (r0 + tl < KM) tab_mf[r0 + tl] = s_y[r0 + tl] * dm;
             }
         }
         __syncwarp();
@@ -701,6 +823,35 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
         }
     }
 
+    uint32_t mx_m = __float_as_uint(mx_m_f), mn_v = 0u;
+    if constexpr (G == 128) {
+        // maxima (and the minimum of v^, for the selection) over the CTA through shared memory
+        typename Shared::Cta& c = s.cta();
+        mn_v = __float_as_uint(vh_at(0));
+#pragma unroll
+        for (int i = 1; i < EPT16; ++i) mn_v = min(mn_v, __float_as_uint(vh_at(i)));
+        mx_m = __reduce_max_sync(0xffffffffu, mx_m);
+        mx_v = __reduce_max_sync(0xffffffffu, mx_v);
+        mn_v = __reduce_min_sync(0xffffffffu, mn_v);
+        if (lane == 0) {
+            c.m[warp] = mx_m;
+            c.v[warp] = mx_v;
+            c.lo[warp] = mn_v;
+            c.failed[warp] = gave_up ? 1u : 0u;
+        }
+        __syncthreads();
+        const uint4 m4 = *reinterpret_cast<const uint4*>(c.m), v4 = *reinterpret_cast<const uint4*>(c.v);
+        const uint4 l4 = *reinterpret_cast<const uint4*>(c.lo), f4 = *reinterpret_cast<const uint4*>(c.failed);
+        if (f4.x | f4.y | f4.z | f4.w) {
+            if (tid == 32) produce_tile16<BM, BV, PBF, G>(a, s, s.desc[(fill + 1u) & 1u]);
+            bar_sync16(2);
+            return;
+        }
+        mx_m = max(max(m4.x, m4.y), max(m4.z, m4.w));
+        mx_v = max(max(v4.x, v4.y), max(v4.z, v4.w));
+        mn_v = min(min(l4.x, l4.y), min(l4.z, l4.w));
+    }
+
     // ---- (B) Adam(W) update, four (fp32) or eight (bf16) elements at a time ----
     // bf16 parameters: IEEE square root and division (see solo_fast.cuh), rounded to nearest even or
     // with the element's Philox draw (purpose 2, one block per eight elements)
@@ -777,7 +928,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     }
 
     // ---- (C) first moment: block scale, nearest level (Eq. 1), see fast_tile ----
-    const uint32_t mx_m = group_max16<G>(__float_as_uint(mx_m_f));
+    if constexpr (G != 128) mx_m = group_max16<G>(mx_m);
     uint32_t om[BM == 8 ? 4 : 2] = {};                            // eight codes per word, 8-bit: four
     const float dm_new = __uint_as_float(mx_m);
     const float inv_m = __frcp_rn(dm_new);
@@ -973,7 +1124,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     }
 
     // ---- (D) second moment: block scale and the p-quantile ----
-    mx_v = group_max16<G>(mx_v);
+    if constexpr (G != 128) mx_v = group_max16<G>(mx_v);
     uint32_t x_p;
     uint32_t w[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};             // 16 halfwords: the draws of the 16 elements
     if (fixed_base) {
@@ -998,6 +1149,16 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
             cswap(key[13], key[14]);
             if (!round_m) quant_m_done();
             x_p = select_pops4(key, a.k_full, &s.sort[0][tid], lane);
+        } else if constexpr (G == 128) {
+            if (!round_m) {
+#pragma unroll
+                for (int j = EPT16 / 2 - 1; j >= 0; --j) quant_m(j);
+                quant_m_done();
+            }
+            uint32_t key[EPT16];
+#pragma unroll
+            for (int i = 0; i < EPT16; ++i) key[i] = __float_as_uint(vh_at(i));
+            x_p = select_cta16(key, a.k_full, s.cta(), mn_v, mx_v, tid);
         } else {
             uint32_t l[4][4];
 #pragma unroll
@@ -1016,6 +1177,20 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     }
 
     // ---- (E) per-block scalars by the first warp; the next tile's copies start meanwhile ----
+    auto draw = [&]() {
+        if (round_v) {
+            uint32_t ctr_lo, ctr_hi, c3, w4[4];
+            stream_position(ctr_lo, ctr_hi, c3);
+            philox_rk(ctr_lo + sw, ctr_hi, a.step32, c3, a.rk, w4);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) w[i] = w4[i];
+            philox_rk(ctr_lo + (sw ^ 1u), ctr_hi, a.step32, c3, a.rk, w4);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) w[4 + i] = w4[i];
+        }
+    };
+    // (a block of 2048: the other warps draw while the first one selects)
+    if (G == 128 && warp != 0) draw();
     if (gl == 0) s.xin[grp] = make_uint4(mx_m, mx_v, x_p, 0u);
     bar_sync16(1);
     // every thread has read what it needs from the stage
@@ -1025,17 +1200,9 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     // (ctr, step, 4 * stream) and (ctr + 1, ...), in its own order.  (Between the selection's rounds, where the draws
     // once hid the shuffles' latency, they gain nothing with 28 to 32 resident warps; here they fill the wait for
     // the first warp: bf16 parameters 536 -> 528 us, 4/4 bit 407 -> 402 us on 2^27 elements.)
-    if (round_v) {
-        uint32_t ctr_lo, ctr_hi, c3, w4[4];
-        stream_position(ctr_lo, ctr_hi, c3);
-        philox_rk(ctr_lo + sw, ctr_hi, a.step32, c3, a.rk, w4);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) w[i] = w4[i];
-        philox_rk(ctr_lo + (sw ^ 1u), ctr_hi, a.step32, c3, a.rk, w4);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) w[4 + i] = w4[i];
-    }
+    if (G != 128) draw();
     bar_sync16(2);
+    if (G == 128 && warp == 0) draw();
     const float4 sc = s.xout[grp];
 
     // second moment: Eq. 6, see fast_tile
@@ -1275,6 +1442,11 @@ __global__ void __launch_bounds__(CTA16, ctas16<BM, BV, G, MODES>()) solo_step_f
         }
     }
     if constexpr (G == 4) s.sort[15][tid] = KEY_MAX;              // never overwritten
+    if constexpr (G == 128) {
+        s.cta().hist[tid] = 0u;
+        s.cta().hist[tid + CTA16] = 0u;
+        if (tid == 0) s.cta().fill = 0u;
+    }
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s.mbar)) : "memory");
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s.mbar_steal)) : "memory");

@@ -30,7 +30,7 @@ def _all_bf16(block):
 @pytest.mark.parametrize("mode", range(len(MODES)))
 @pytest.mark.parametrize("bits_m,bits_v", [(8, 8), (8, 3), (4, 8)])
 def test_every_cell_of_the_codebooks(bits_m, bits_v, mode):
-    for block in (64, 128, 256):
+    for block in (64, 128, 256, 2048):
         g = _all_bf16(block)
         n = g.numel()
         rep = run_lockstep((n,), bits_m, bits_v, block, dict(lr=1e-3, beta1=0.0, beta2=0.0, weight_decay=0.0, seed=21) | MODES[mode],
@@ -40,7 +40,8 @@ def test_every_cell_of_the_codebooks(bits_m, bits_v, mode):
 
 
 @pytest.mark.parametrize("mode", range(len(MODES)))
-@pytest.mark.parametrize("bits_m,bits_v,block", [(8, 8, 64), (8, 8, 128), (8, 8, 256), (2, 8, 128), (3, 8, 64), (4, 8, 256), (8, 2, 128), (8, 4, 64)])
+@pytest.mark.parametrize("bits_m,bits_v,block", [(8, 8, 64), (8, 8, 128), (8, 8, 256), (2, 8, 128), (3, 8, 64), (4, 8, 256), (8, 2, 128), (8, 4, 64),
+                                                 (8, 8, 2048), (2, 3, 2048), (4, 2, 2048), (3, 8, 2048)])
 def test_random_states(bits_m, bits_v, block, mode):
     sizes = (2048 * 3, 2048 * 2 + 77)
     w = synth.workload(3, sizes=sizes)

@@ -1,6 +1,7 @@
 """The p-quantile of the sixteen-per-thread kernel (rank selection over a group of lanes) at any rank, on inputs
 that are hard for it: keys that ascend with the element index (one lane holds all the smallest), equal keys,
-blocks of zeros with a few values, and random states.  The packed state, and with it the base that the quantile
+blocks of zeros with a few values, and random states.  Blocks of 2048 span the CTA: histogram bins that hold few,
+more than 512 or all of the keys.  The packed state, and with it the base that the quantile
 decides, is compared with the oracle's bit for bit; parameters within the bar of every other parity test."""
 import numpy as np
 import pytest
@@ -23,6 +24,8 @@ def _grads(kind, t, n, seed):
         x = 1e-3 * (8.0 - (i % 256) * (7 / 256))
     elif kind == "equal":
         x = torch.full((n,), 2.5e-4)
+    elif kind == "clusters":                                  # most keys within one bin of the block's range, 2-bit levels apart
+        x = 1e-3 * (1.0 + 1e-2 * torch.randn(n, generator=g)) * torch.where(torch.rand(n, generator=g) < 0.8, 1.0, 30.0)
     elif kind == "zeros":
         x = torch.randn(n, generator=g) * 1e-3
         x[torch.rand(n, generator=g) < 0.9] = 0.0
@@ -31,8 +34,8 @@ def _grads(kind, t, n, seed):
     return x.to(torch.bfloat16)
 
 
-@pytest.mark.parametrize("kind", ["ascending", "descending", "equal", "zeros", "random"])
-@pytest.mark.parametrize("block", [64, 128, 256])
+@pytest.mark.parametrize("kind", ["ascending", "descending", "equal", "zeros", "clusters", "random"])
+@pytest.mark.parametrize("block", [64, 128, 256, 2048])
 def test_selection_at_any_rank(block, kind):
     w = synth.workload(3, sizes=SIZES)
     for p in (0.0, 0.05, 0.1, 0.2, 0.5, 0.99):
