@@ -108,6 +108,8 @@ def lib() -> C.CDLL:
     L.solo_set_kernel_policy.argtypes = [i32]
     L.solo_debug_check_fast_log.argtypes = [C.c_uint32, C.c_uint32, C.POINTER(C.c_float),
                                             C.POINTER(C.c_float)]
+    L.solo_debug_check_update_math.argtypes = [C.c_uint32, C.c_uint32, C.POINTER(C.c_uint64)]
+    L.solo_debug_check_update_math.restype = C.c_int
     L.solo_multi_step_static.argtypes = [C.c_int32, vp, vp, C.POINTER(C.c_int64), C.POINTER(RawState),
                                          C.POINTER(Hyper), i64, vp]
     L.solo_multi_step_static.restype = C.c_int
@@ -406,6 +408,13 @@ def debug_check_fast_log(lo_bits: int, hi_bits: int) -> tuple[float, float]:
     _check(lib().solo_debug_check_fast_log(lo_bits, hi_bits, C.byref(ex), C.byref(ab)),
            "solo_debug_check_fast_log")
     return ex.value, ab.value
+
+
+def debug_check_update_math(lo_bits: int, hi_bits: int) -> int:
+    """Results of the pairwise square root and division that differ from the IEEE operations'."""
+    n = C.c_uint64()
+    _check(lib().solo_debug_check_update_math(lo_bits, hi_bits, C.byref(n)), "solo_debug_check_update_math")
+    return n.value
 
 
 def static_status() -> int:

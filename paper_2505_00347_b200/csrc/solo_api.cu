@@ -1005,6 +1005,19 @@ int solo_debug_check_fast_log(uint32_t lo_bits, uint32_t hi_bits, float* max_exc
     return SOLO_OK;
 }
 
+int solo_debug_check_update_math(uint32_t lo_bits, uint32_t hi_bits, uint64_t* mismatches_host) {
+    if (!mismatches_host || lo_bits > hi_bits || hi_bits >= 0x7F800000u) return SOLO_EINVAL;
+    unsigned long long* d = nullptr;
+    if (cudaMalloc((void**)&d, 8) != cudaSuccess) { cudaGetLastError(); return SOLO_ENOMEM; }
+    cudaError_t e = cudaMemset(d, 0, 8);
+    if (e == cudaSuccess) e = solo::launch_update_math_check(lo_bits, hi_bits, d, nullptr);
+    if (e == cudaSuccess) g_launches.fetch_add(1, std::memory_order_relaxed);
+    if (e == cudaSuccess) e = cudaMemcpy(mismatches_host, d, 8, cudaMemcpyDeviceToHost);
+    cudaFree(d);
+    if (e != cudaSuccess) { cudaGetLastError(); return SOLO_ECUDA; }
+    return SOLO_OK;
+}
+
 int64_t solo_launch_count(void) { return g_launches.load(std::memory_order_relaxed); }
 
 const char* solo_strerror(int status) {

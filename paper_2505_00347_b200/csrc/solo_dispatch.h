@@ -75,6 +75,8 @@ int kernel_occupancy(StepKernel k, size_t dyn_smem, int threads = CTA);
 // Exhaustive comparison of the hardware lg2 approximation with log2_sp (tests).
 cudaError_t launch_fast_log_check(uint32_t lo, uint32_t hi, float* out_max_excess, cudaStream_t stream);
 float fast_log_abs_bound();
+// Comparison of the pairwise square root and division with the IEEE operations (tests).
+cudaError_t launch_update_math_check(uint32_t lo, uint32_t hi, unsigned long long* mismatches, cudaStream_t stream);
 
 cudaError_t launch_dequant(int bits, const DequantArgs& a, unsigned grid, cudaStream_t stream);
 

@@ -158,6 +158,33 @@ __device__ __forceinline__ F2 add2(F2 a, F2 b) {
     return r;
 }
 
+// Correctly rounded square root and quotient of pairs by fused multiply-adds from the hardware approximations
+// (P. Markstein, "Computation of elementary functions on the IBM RISC System/6000 processor", 1990): two results per
+// issue slot and no branch, where the IEEE operations take about eleven instructions and a range check each (2/2 bit with
+// stochastically rounded bf16 parameters, 2^27 elements: 525 -> 507 us).
+// solo_debug_check_update_math compares them with the IEEE operations: every mantissa for the square root, every mantissa
+// of the denominator for the quotient.  Scaled so that no intermediate result underflows:
+//   nx = -x * 2^100, 0 <= x < 2^27 (zeros and subnormal numbers included): -sqrt(x) * 2^50
+__device__ __forceinline__ F2 neg_sqrt2(F2 nx) {
+    const F2 t = add2(nx, F2::dup(-0x1p-120f));                    // a zero: 1/sqrt stays finite; else no change
+    float yl, yh;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yl) : "f"(-t.lo()));
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yh) : "f"(-t.hi()));
+    const F2 y = F2::pack(yl, yh);
+    const F2 ng0 = mul2(nx, y), h0 = mul2(y, F2::dup(0.5f));
+    const F2 r = fma2(ng0, h0, F2::dup(0.5f));
+    const F2 ng1 = fma2(ng0, r, ng0), h1 = fma2(h0, r, h0);
+    return fma2(fma2(ng1, ng1, nx), h1, ng1);
+}
+//   -m / d, 2^-64 <= d <= 2^64, |m| zero or from 2^-85 to 2^84: the reciprocal is correctly rounded (every mantissa checked)
+//   and the quotient within an ulp, so that one correction by the exact remainder rounds it correctly
+__device__ __forceinline__ F2 neg_div2(F2 m, F2 d) {
+    const F2 ny0 = F2::pack(rcp_approx(-d.lo()), rcp_approx(-d.hi()));
+    const F2 ny = fma2(fma2(d, ny0, F2::dup(1.0f)), ny0, ny0);
+    const F2 nq = mul2(m, ny);
+    return fma2(fma2(d, nq, m), ny, nq);
+}
+
 // max(acc, |x|) that returns NaN when x is NaN: a NaN among the block's values makes the block's
 // scale NaN, as the maximum over bit patterns of the general kernel does.
 __device__ __forceinline__ float max_abs_nan(float acc, float x) {

@@ -823,6 +823,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
         }
     }
 
+    const uint32_t tmx_v = mx_v;                                  // the thread's own maximum
     uint32_t mx_m = __float_as_uint(mx_m_f), mn_v = 0u;
     if constexpr (G == 128) {
         // maxima (and the minimum of v^, for the selection) over the CTA through shared memory
@@ -853,7 +854,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     }
 
     // ---- (B) Adam(W) update, four (fp32) or eight (bf16) elements at a time ----
-    // bf16 parameters: IEEE square root and division (see solo_fast.cuh), rounded to nearest even or
+    // bf16 parameters: correctly rounded square root and division (see solo_fast.cuh), rounded to nearest even or
     // with the element's Philox draw (purpose 2, one block per eight elements)
     // position of the thread's first element in the tensor's random stream (element index / 8): even,
     // so the second group of eight never carries into the high word
@@ -891,6 +892,12 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
         }
     } else {
         const uint4* const sp = reinterpret_cast<const uint4*>(st.p) + 2 * tid;
+        // The exact pairwise sequence where its scaling holds: v^ < 2^27, |m^| < 2^20 (a NaN compares false), usual
+        // hyper-parameters; the IEEE operations otherwise.  (Quotients below 2^-126 are not rounded to the
+        // subnormal grid first, which only parameters that size can show.)
+        const bool exact = tmx_v < 0x4D000000u && mx_m_f < 0x1p20f && a.eps >= 0x1p-60f && a.eps < 0x1p30f &&
+                           a.inv_sqrt_bc2 < 0x1p30f && fabsf(a.step_size) > 0x1p-40f && fabsf(a.step_size) < 0x1p60f;
+        const bool exact_all = __all_sync(0xffffffffu, exact);
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const uint32_t he = (uint32_t)h ^ sw;
@@ -902,11 +909,25 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
                 p[2 * k] = __uint_as_float(pin[k] << 16);
                 p[2 * k + 1] = __uint_as_float(pin[k] & 0xffff0000u);
             }
+            if (exact_all) {
+                const F2 nisb = F2::dup(-a.inv_sqrt_bc2 * 0x1p-50f), eps = F2::dup(a.eps), lr = F2::dup(a.step_size * 0x1p-64f);
 #pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                const int i = 8 * h + k;
-                const float den = __fmaf_rn(__fsqrt_rn(vh_at(i)), a.inv_sqrt_bc2, a.eps);
-                p[k] = __fmaf_rn(-a.step_size, __fdiv_rn(mh_at(i), den), DECAY ? p[k] * a.decay : p[k]);
+                for (int k = 0; k < 4; ++k) {
+                    const int j = 4 * h + k;
+                    const F2 den = fma2(neg_sqrt2(mul2(vh[j], F2::dup(-0x1p100f))), nisb, eps);
+                    const F2 nq = neg_div2(mul2(mh[j], F2::dup(0x1p64f)), den);
+                    F2 pj = F2::pack(p[2 * k], p[2 * k + 1]);
+                    pj = fma2(lr, nq, DECAY ? mul2(pj, F2::dup(a.decay)) : pj);
+                    p[2 * k] = pj.lo();
+                    p[2 * k + 1] = pj.hi();
+                }
+            } else {
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const int i = 8 * h + k;
+                    const float den = __fmaf_rn(__fsqrt_rn(vh_at(i)), a.inv_sqrt_bc2, a.eps);
+                    p[k] = __fmaf_rn(-a.step_size, __fdiv_rn(mh_at(i), den), DECAY ? p[k] * a.decay : p[k]);
+                }
             }
             uint32_t pp[4];
             if (a.param_sr) {

@@ -59,6 +59,40 @@ __global__ void fast_log_check_kernel(uint32_t lo, uint32_t hi, float* out_max_e
         atomicMax(reinterpret_cast<int*>(out_max_excess), __float_as_int(worst));
 }
 
+// Comparison of neg_sqrt2 and neg_div2 with the IEEE operations: for every binary32 with pattern in [lo, hi] its square
+// root, and as a denominator (brought to exponents from -40 to 40) its quotients with eight numerators.
+__global__ void update_math_check_kernel(uint32_t lo, uint32_t hi, unsigned long long* mismatches) {
+    unsigned long long bad = 0;
+    for (uint64_t b = (uint64_t)lo + 2 * (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x); b <= hi;
+         b += 2 * (uint64_t)gridDim.x * blockDim.x) {
+        const float x[2] = {__uint_as_float((uint32_t)b), __uint_as_float((uint32_t)min(b + 1, (uint64_t)hi))};
+        if (x[0] < 0x1p27f && x[1] < 0x1p27f) {
+            const F2 s = neg_sqrt2(mul2(F2::pack(x[0], x[1]), F2::dup(-0x1p100f)));
+            bad += (-s.lo() * 0x1p-50f != __fsqrt_rn(x[0])) + (-s.hi() * 0x1p-50f != __fsqrt_rn(x[1]));
+        }
+        uint32_t w[4], w2[4];
+        philox4x32_10((uint32_t)b, 1u, 2u, 3u, 4u, 5u, w);
+        philox4x32_10((uint32_t)b, 7u, 2u, 3u, 4u, 5u, w2);
+        for (int i = 0; i < 4; ++i) {
+            float d[2], m[2];
+            for (int k = 0; k < 2; ++k) {
+                const uint32_t r = k ? w2[i] : w[i];
+                d[k] = __uint_as_float((__float_as_uint(x[k]) & 0x007FFFFFu) | ((127u - 40u + r % 81u) << 23));
+                m[k] = __uint_as_float((r & 0x807FFFFFu) | ((127u - 80u + (r >> 7) % 100u) << 23));
+                if (i == 0) m[k] = __uint_as_float(__float_as_uint(d[k]) + (r & 3u) - 1u);      // quotients around 1
+            }
+            const F2 q = neg_div2(mul2(F2::pack(m[0], m[1]), F2::dup(0x1p64f)), F2::pack(d[0], d[1]));
+            bad += (-q.lo() * 0x1p-64f != __fdiv_rn(m[0], d[0])) + (-q.hi() * 0x1p-64f != __fdiv_rn(m[1], d[1]));
+        }
+    }
+    if (bad) atomicAdd(mismatches, bad);
+}
+
+cudaError_t launch_update_math_check(uint32_t lo, uint32_t hi, unsigned long long* mismatches, cudaStream_t stream) {
+    update_math_check_kernel<<<148 * 8, 256, 0, stream>>>(lo, hi, mismatches);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_fast_log_check(uint32_t lo, uint32_t hi, float* out_max_excess, cudaStream_t stream) {
     fast_log_check_kernel<<<148 * 8, 256, 0, stream>>>(lo, hi, out_max_excess);
     return cudaGetLastError();
