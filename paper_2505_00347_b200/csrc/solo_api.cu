@@ -246,11 +246,10 @@ int launch_step(solo_state* s, StepArgs& a, cudaStream_t stream) {
     // Lists need a second launch for the tiles that are not full (513 tiles 7.6 us against 9.4 us).  What the
     // streamlined kernel has no path for, one tile on (Eq. 5 at one tile 9.7 us in the general kernel, 7.4 us here).
     const bool all_full = !a.param_list && s->num_tensors == 1 && s->numel[0] % solo::TILE == 0;
-    // Blocks of 2048, where a CTA of four warps meets at five barriers: from a few waves on (4/4 bit: 4096 tiles 47.9 us against
-    // 50.9, 65,536 tiles 655 and 592; 8/8 bit: 512 tiles 16.4 and 12.9).
+    // Blocks of 2048 (4/4 bit): 512 tiles 12.3 us against 14.4, 1024 tiles 18.5 and 15.8, 4096 tiles 48.0 and 46.7.
     const bool w8 = s->bits_m == 8 || s->bits_v == 8;
     const int64_t from = !streamlined ? (all_full ? 1 : 64)
-                                      : (cta_group ? (w8 ? 512 : 8192) : w8 ? 256 : 768) * (all_full || (cta_group && !w8) ? 1 : 2);
+                                      : (cta_group ? (w8 ? 512 : 1024) : w8 ? 256 : 768) * (all_full ? 1 : 2);
     const bool large = s->tiles_total >= from;
     if (fast_ok && ((policy == 0 && large) || policy == 3))
         k16 = solo::fast16_kernel(s->bits_m, s->bits_v, s->block, a.param_bf16 != 0,
