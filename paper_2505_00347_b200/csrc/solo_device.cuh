@@ -71,11 +71,10 @@ struct StepArgs {
 
 // ---------------------------------------------------------------------------
 // Programmatic dependent launch.  Every step kernel is launched so that its CTAs may be placed while the
-// kernel before it on the stream still runs (its launch latency, 2 to 3 us, is hidden); it touches global memory only
-// after that kernel has completed (pdl_wait), and only then lets the kernel after it be placed (pdl_release).  The
-// launch for the tiles that are not full shares no tile with the one for the full tiles before it: it
-// does not wait for that one's end before its work, but its first CTA does before it ends (whoever waits for the
-// second launch has waited for both).  The first launch releases it only after its own pdl_wait, so the inputs are complete.
+// kernel before it on the stream still runs (its launch latency, 2 to 3 us, is hidden); every CTA reads and writes global
+// memory only after that kernel has completed and its writes are visible (pdl_wait), and only then lets the kernel after it
+// be placed (pdl_release).  That holds for the launch for the tiles that are not full too, although it shares no tile
+// with the one before it: what both read was written by earlier work, and only the wait makes those writes visible.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_release() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
@@ -407,7 +406,7 @@ __global__ void __launch_bounds__(CTA) solo_step_kernel(const __grid_constant__ 
     __shared__ uint32_t s_red[8];
 
     const int tid = threadIdx.x;
-    if (!a.only_partial) pdl_wait();
+    pdl_wait();
     pdl_release();
     for (int i = tid; i < KM; i += CTA) {
         s_y[i] = a.tables[i];
@@ -670,7 +669,6 @@ __global__ void __launch_bounds__(CTA) solo_step_kernel(const __grid_constant__ 
             a.alpha[jb] = al_new;
         }
     }
-    if (a.only_partial && blockIdx.x == 0) pdl_wait();
 }
 
 // ---------------------------------------------------------------------------

@@ -1097,7 +1097,7 @@ __global__ void __launch_bounds__(CTA, (BM == 8 || BV == 8) ? 3 : 4) solo_step_f
     __shared__ float s_mid[KM];
     __shared__ float4 s_mid4[4];     // 4-bit first moments: per quarter of the codebook, its three inner midpoints times -2^100
     const int tid = threadIdx.x;
-    if constexpr (!TAILS) pdl_wait();
+    pdl_wait();
     pdl_release();
     for (int i = tid; i < KM; i += CTA) {
         s_y[i] = a.tables[i];
@@ -1145,7 +1145,6 @@ __global__ void __launch_bounds__(CTA, (BM == 8 || BV == 8) ? 3 : 4) solo_step_f
                 __ldg(a.block_start + t) + (int64_t)tin * (CTA / G), t, par, ah, false, 0, 0);
             par ^= 1;
         }
-        if (blockIdx.x == 0) pdl_wait();
         return;
     }
     if constexpr (!TAILS) {
