@@ -391,7 +391,8 @@ int solo_static_status(int* status_out, void* stream);
  * the inputs of tile number `tile` (tiles of 2048 elements, counted over the tensor list), so the
  * wait for that tile's inputs runs out after its fixed number of polls: the waiting warps set
  * status bit 1, store nothing for that tile and the tiles their CTA processes after it, and the
- * kernel returns.  Nothing faults and nothing spins without limit.  One-shot and process-wide;
+ * kernel returns.  (In the sixteen-per-thread kernel a CTA takes at most three tiles at a time and a CTA whose wait ran
+ * out takes none after those it already has, at most six: the others are stepped as usual.)  Nothing faults and nothing spins without limit.  One-shot and process-wide;
  * tiles that are not staged (not full, or in the general kernel) ignore it.  (No counterpart
  * in the paper.)
  */

@@ -124,6 +124,8 @@ struct Fast16Shared {
         int tensor, t_lo, t_hi, full_tiles;  // tensor: tiles [t_lo, t_hi), the first full_tiles of them full
         int tile, tile_end;                  // last tile handed out; end of the tiles taken
         uint32_t phase;                      // parity of mbar_steal's next phase
+        bool unanswered;                     // the wait for an answer ran out: it may still come
+        bool gave_up;                        // some thread waited in vain for a copy: the CTA takes no further tile
     } walk;
     struct Desc {
         char* p;                             // the tile's parameters, gradients, first block
@@ -525,6 +527,7 @@ template <class Shared>
 __device__ __forceinline__ int steal_answer(Shared& s, int* status) {
     if (!mbar_wait(smem_u32(&s.mbar_steal), s.walk.phase)) {
         atomicOr(status, 2);                                            // (its tiles, if it was cancelled, are not stepped)
+        s.walk.unanswered = true;
         return -1;
     }
     s.walk.phase ^= 1u;
@@ -544,15 +547,18 @@ __device__ __forceinline__ int steal_answer(Shared& s, int* status) {
 // tensors and shares.  One share per resident CTA (a static walk) left 5 % of the SM cycles idle at the launch's
 // end and SMs with fewer CTAs before it: LLaMA layers 2357 -> 2170 us, GPT-125M-shaped set 432 -> 390 us, ragged set
 // 3418 -> 3200 us, 2^24 elements 60 -> 55 us.
+// A CTA that waited in vain for a copy ends here: it takes in the answer to its last request, so that nothing writes to its
+// shared memory any more, and asks for no other.  What it then leaves unstepped (and has reported in the status word) is
+// the rest of its share and at most the one that answer brought, however many CTAs have not started yet.
 template <int BM, int BV, bool PBF, int G>
 __device__ __forceinline__ void produce_tile16(const StepArgs& a, Fast16Shared<BM, BV, PBF, G>& s, typename Fast16Shared<BM, BV, PBF, G>::Desc& d) {
     constexpr int NG = CTA16 / G, PSZ = PBF ? 2 : 4;
     typename Fast16Shared<BM, BV, PBF, G>::Walk& w = s.walk;
-    int tile = w.tile, tile_end = w.tile_end;
+    int tile_end = w.tile_end, tile = w.gave_up ? tile_end : w.tile;
     for (;;) {
         if (++tile >= tile_end) {
             const int cta = steal_answer(s, a.status);
-            if (cta < 0) {
+            if (cta < 0 || w.gave_up) {                                  // (one request is under way as long as there are tiles)
                 d.valid = 0;
                 return;
             }
@@ -662,10 +668,11 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     if (!mbar_wait(smem_u32(&s.mbar), fill & 1u, failed ? 1 : MBAR_POLLS)) {
         if (!failed) atomicOr(a.status, 2);
         failed = true;
+        s.walk.gave_up = true;
     }
     // A warp in which any lane gave up leaves the tile alone: it stores nothing, flags its blocks
-    // for the first warp (which stores the per-block scalars), and only keeps the CTA's barriers, the
-    // copy-ahead and, if it is the first warp, the other warps' scalars going.
+    // for the first warp (which stores the per-block scalars), and only keeps the CTA's barriers and, if it is
+    // the first warp, the other warps' scalars going.  It is the CTA's last tile (produce_tile16).
     // A block of 2048 spans the CTA, which leaves the tile as a whole (below).
     const bool gave_up = __any_sync(0xffffffffu, failed);
     if (G != 128 && gave_up) {
@@ -1485,6 +1492,7 @@ __global__ void __launch_bounds__(CTA16, ctas16<BM, BV, G, MODES>()) solo_step_f
 
     if (tid == 32) {
         s.walk.phase = 0;
+        s.walk.gave_up = s.walk.unanswered = false;
         s.walk.t_lo = s.walk.t_hi = -1;
         s.walk.tile = (int)a.tile_first + (int)blockIdx.x * a.share - 1;
         s.walk.tile_end = (int)min((int64_t)s.walk.tile + 1 + a.share, a.total_tiles);
@@ -1494,7 +1502,7 @@ __global__ void __launch_bounds__(CTA16, ctas16<BM, BV, G, MODES>()) solo_step_f
     }
     __syncthreads();
 
-    bool failed = false;          // this thread once waited in vain for a copy: it waits no longer and stores nothing
+    bool failed = false;          // this thread waited in vain for a copy: it stores nothing
     uint32_t fill = 0;            // number of the tile, and of the copy it waits for
     const bool decay = a.decay != 1.0f;
     for (; s.desc[fill & 1u].valid; ++fill) {
@@ -1504,8 +1512,9 @@ __global__ void __launch_bounds__(CTA16, ctas16<BM, BV, G, MODES>()) solo_step_f
             fast16_tile<BM, BV, PBF, G, false, MODES>(a, s, s_y, s_mid, s_mid4, s_yv, s_nv, s_yg, s_br, fill, failed);
     }
     // A thread that gave up on a copy waits once more, again bounded, for the last one that was issued,
-    // so that no copy is still writing to the stage when the CTA's shared memory is released.
+    // so that no copy is still writing to the stage when the CTA's shared memory is released; likewise for an answer.
     if (failed && fill > 0) mbar_wait(smem_u32(&s.mbar), (fill - 1u) & 1u);
+    if (tid == 32 && s.walk.unanswered) mbar_wait(smem_u32(&s.mbar_steal), s.walk.phase);
 }
 
 }  // namespace solo
