@@ -219,7 +219,7 @@ __device__ constexpr unsigned char SORT16_PAIRS[62][2] = {
     {1, 9}, {5, 13}, {5, 9}, {3, 11}, {7, 15}, {7, 11}, {3, 5}, {7, 9}, {11, 13},
     {1, 2}, {3, 4}, {5, 6}, {7, 8}, {9, 10}, {11, 12}};
 
-// Thresholds of the 8-bit codebooks below the cell of r (solo_lut8.cuh).
+// Thresholds of the 8-bit codebooks below the cell of r (solo_lut8.cuh); |r| < 1 + 1/64 or NaN.
 __device__ __forceinline__ uint32_t cell8_m(const unsigned char* lut, float r) {
     const uint32_t t = __float_as_uint(fmaxf(fabsf(r), 0x1p-22f)) ^ ((__float_as_uint(r) >> 3) & 0x10000000u);
     // (negative values: exponent bit 5 cleared.  Written so that the positive cells follow the negative ones.)
@@ -614,7 +614,7 @@ __device__ __forceinline__ void block_scalars16(const StepArgs& a, Shared& s, co
     const uint4 in = s.xin[tid];
     const float dm_new = __uint_as_float(in.x), dv_new = __uint_as_float(in.y);
     const bool zero_m = dm_new < TINY, zero_v = dv_new < TINY;
-    const float inv_dv = __frcp_rn(dv_new);
+    const float inv_dv = zero_v ? 0.0f : __frcp_rn(dv_new);      // (no infinity: the ratios index the cell tables)
     const float rho = fminf(fmaxf(__uint_as_float(in.z) * inv_dv, RHO_MIN), RHO_MAX);
     const float lam = log2_sp(rho) * (1.0f / (float)(KV - 1));
     // (a baseline codebook has no base: the array keeps its initial 1/2)
@@ -958,7 +958,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     if constexpr (G != 128) mx_m = group_max16<G>(mx_m);
     uint32_t om[BM == 8 ? 4 : 2] = {};                            // eight codes per word, 8-bit: four
     const float dm_new = __uint_as_float(mx_m);
-    const float inv_m = __frcp_rn(dm_new);
+    const float inv_m = dm_new < TINY ? 0.0f : __frcp_rn(dm_new);   // (no infinity: the ratios index the cell tables)
     // code = number of midpoints below r, each comparison as the saturation of (r - mid) * 2^100 on the FMA
     // pipe (exactly 0 or 1, see fast_tile).  The codes of elements 2j and 2j + 1 are accumulated side by side
     // in one pair of binary32 (eight 2- or 3-bit codes per pair, at most 21 bits each: exact).

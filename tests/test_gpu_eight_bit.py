@@ -61,3 +61,16 @@ def test_nan_and_infinite_blocks():
         run_lockstep(sizes, 8, 8, 128, dict(lr=1e-3, beta1=0.9, beta2=0.99, weight_decay=0.0, seed=5) | mode, steps=1,
                      grads_fn=lambda t: [g], params0=[torch.zeros(sizes[0])], policies=(3,), multi=True,
                      state0=synth.make_state(sizes, 8, 8, 128, seed=2), update_tol=RANDOM_STATE_TOL)
+
+
+@pytest.mark.parametrize("block", [64, 128, 256, 2048])
+@pytest.mark.parametrize("bits_m,bits_v,bf16", [(8, 8, 0), (2, 8, 1), (8, 3, 0)])
+def test_blocks_whose_largest_value_has_no_finite_reciprocal(bits_m, bits_v, bf16, block):
+    """Scales between 0 and 2^-128, for the second moment (gradients of 1e-19) and for both (1e-39): a vanishing block."""
+    sizes = (2048 * 6,)
+    scale = torch.tensor([1e-19, 1.0, 1e-39, 1e-19, 0.0, 1e-3]).repeat_interleave(2048)
+    for mode in (dict(), dict(v_codebook=1), dict(v_codebook=2), dict(round_m=1), dict(round_m=1, v_codebook=3)):
+        g = (synth.make_grad(synth.workload(3, sizes=sizes), 0, 1).float() * 1e3).clamp(-1, 1).mul(scale).bfloat16()
+        run_lockstep(sizes, bits_m, bits_v, block, dict(lr=1e-3, beta1=0.9, beta2=0.99, weight_decay=0.0, seed=5, param_dtype=bf16) | mode,
+                     steps=2, grads_fn=lambda t: [g], params0=[torch.zeros(sizes[0], dtype=torch.bfloat16 if bf16 else torch.float32)],
+                     policies=(3,), multi=True, update_tol=RANDOM_STATE_TOL)
