@@ -315,8 +315,8 @@ int solo_debug_check_fast_log(uint32_t lo_bits, uint32_t hi_bits, float* max_exc
 /*
  * Test hook for the square root and division of bf16 parameters' update: for every binary32 whose bit pattern lies in
  * [lo_bits, hi_bits] (finite, not negative) compares the fused multiply-add sequences with the IEEE operations, for
- * the square root (below 2^27) and, with its mantissa in the denominator, for eight quotients.  Writes the number of
- * results that differ to HOST *mismatches_host.  Synchronous; allocates 8 bytes of device memory.
+ * the square root (below 2^27) and, with its mantissa in a denominator of 2^-40 to 2^44, for eight quotients that are
+ * normal numbers (numerators below 2^20, subnormal ones included).  Writes the number of results that differ to HOST *mismatches_host.  Synchronous; allocates 8 bytes of device memory.
  */
 int solo_debug_check_update_math(uint32_t lo_bits, uint32_t hi_bits, uint64_t* mismatches_host);
 

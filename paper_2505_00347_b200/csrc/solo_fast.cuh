@@ -176,8 +176,9 @@ __device__ __forceinline__ F2 neg_sqrt2(F2 nx) {
     const F2 ng1 = fma2(ng0, r, ng0), h1 = fma2(h0, r, h0);
     return fma2(fma2(ng1, ng1, nx), h1, ng1);
 }
-//   -m / d, 2^-64 <= d <= 2^64, |m| zero or from 2^-85 to 2^84: the reciprocal is correctly rounded (every mantissa checked)
-//   and the quotient within an ulp, so that one correction by the exact remainder rounds it correctly
+//   -m / d, 2^-40 <= d <= 2^44, |m| zero or from 2^-85 to 2^84, |m / d| zero or at least 2^-62: the reciprocal is
+//   correctly rounded (every mantissa checked) and the quotient within an ulp, so that one correction by the exact
+//   remainder rounds it correctly
 __device__ __forceinline__ F2 neg_div2(F2 m, F2 d) {
     const F2 ny0 = F2::pack(rcp_approx(-d.lo()), rcp_approx(-d.hi()));
     const F2 ny = fma2(fma2(d, ny0, F2::dup(1.0f)), ny0, ny0);

@@ -60,7 +60,8 @@ __global__ void fast_log_check_kernel(uint32_t lo, uint32_t hi, float* out_max_e
 }
 
 // Comparison of neg_sqrt2 and neg_div2 with the IEEE operations: for every binary32 with pattern in [lo, hi] its square
-// root, and as a denominator (brought to exponents from -40 to 40) its quotients with eight numerators.
+// root, and as a denominator (brought to exponents from -40 to 43) its quotients with eight numerators: one close to the
+// denominator, the others below 2^20 down to the smallest subnormal number, where the quotient is a normal number.
 __global__ void update_math_check_kernel(uint32_t lo, uint32_t hi, unsigned long long* mismatches) {
     unsigned long long bad = 0;
     for (uint64_t b = (uint64_t)lo + 2 * (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x); b <= hi;
@@ -77,12 +78,16 @@ __global__ void update_math_check_kernel(uint32_t lo, uint32_t hi, unsigned long
             float d[2], m[2];
             for (int k = 0; k < 2; ++k) {
                 const uint32_t r = k ? w2[i] : w[i];
-                d[k] = __uint_as_float((__float_as_uint(x[k]) & 0x007FFFFFu) | ((127u - 40u + r % 81u) << 23));
-                m[k] = __uint_as_float((r & 0x807FFFFFu) | ((127u - 80u + (r >> 7) % 100u) << 23));
-                if (i == 0) m[k] = __uint_as_float(__float_as_uint(d[k]) + (r & 3u) - 1u);      // quotients around 1
+                d[k] = __uint_as_float((__float_as_uint(x[k]) & 0x007FFFFFu) | ((127u - 40u + r % 84u) << 23));
+                // exponents from 2^-126 on, a fifth of the numerators subnormal with 1 to 23 bits
+                const uint32_t e = (r >> 7) % 183u;
+                m[k] = __uint_as_float((r & 0x80000000u) | (e < 146u ? (r & 0x007FFFFFu) | ((e + 1u) << 23)
+                                                                     : (0x00400000u | (r & 0x003FFFFFu)) >> ((r >> 15) % 23u)));
+                if (i == 0) m[k] = __uint_as_float(__float_as_uint(min(d[k], 0x1p19f)) + (r & 3u) - 1u);   // quotients around 1
             }
             const F2 q = neg_div2(mul2(F2::pack(m[0], m[1]), F2::dup(0x1p64f)), F2::pack(d[0], d[1]));
-            bad += (-q.lo() * 0x1p-64f != __fdiv_rn(m[0], d[0])) + (-q.hi() * 0x1p-64f != __fdiv_rn(m[1], d[1]));
+            auto differs = [](float a, float b) { return fabsf(b) > 0x1p-126f && a != b; };
+            bad += differs(-q.lo() * 0x1p-64f, __fdiv_rn(m[0], d[0])) + differs(-q.hi() * 0x1p-64f, __fdiv_rn(m[1], d[1]));
         }
     }
     if (bad) atomicAdd(mismatches, bad);
