@@ -288,11 +288,15 @@ float solo_default_beta1(int bits_m, int from_scratch);
 /*
  * Kernel selection.  0 (default): every width and block size with the logarithmic
  * second-moment quantizer, nearest rounding of the first moment and eps >= 1e-12 runs the
- * streamlined kernel (fp32 or bf16 parameters), everything else the general one; tensor sets from
- * about a thousand tiles of 2048 elements on (more with blocks of 2048) run
- * their full tiles in a kernel with sixteen elements per thread and the remaining tiles in the
+ * streamlined kernel (fp32 or bf16 parameters), everything else the general one; tensor sets with
+ * enough full tiles of 2048 elements run
+ * them in a kernel with sixteen elements per thread and the remaining tiles in the
  * streamlined kernel, or in the general one where the streamlined kernel does not apply (two
- * launches).  That kernel covers every mode of solo_hyper_t (Eq. 5 rounding and the baseline
+ * launches).  Enough: for one tensor of whole tiles (one launch) 768, 256 with an 8-bit state, 1024 or 512 with
+ * blocks of 2048, one where the streamlined kernel does not apply; for lists and other tensors, with r
+ * tiles that are not full, 2048 + 6 r (2048 + 2 r with an 8-bit state, 2048 - 4 r with blocks of 2048), or 768 (1536 with
+ * blocks of 2048) where the streamlined kernel does not apply; the chunks of solo_multi_step_host each count for
+ * themselves, except in the last case.  That kernel covers every mode of solo_hyper_t (Eq. 5 rounding and the baseline
  * second-moment codebooks included) and every p.  1: always the general kernel.  2: like 0 without the
  * sixteen-per-thread kernel.  3: like 0 with the sixteen-per-thread kernel whatever the tensor
  * sizes.  All produce the same packed state and the same bf16 parameters; the fp32 parameters

@@ -19,7 +19,7 @@ using solo::StepArgs;
 struct solo_state {
     int device = 0;
     int bits_m = 0, bits_v = 0, block = 0, num_tensors = 0;
-    int64_t numel_total = 0, nblk_total = 0, tiles_total = 0;
+    int64_t numel_total = 0, nblk_total = 0, tiles_total = 0, full_tiles = 0;      // full_tiles: tiles of TILE elements
     std::vector<int64_t> numel, block_start, tile_start, elem_start;  // host copies
     // device
     uint8_t* codes_m = nullptr;
@@ -230,7 +230,8 @@ int launch_kernel(solo::StepKernel k, const StepArgs& a, int device, int threads
     return SOLO_OK;
 }
 
-int launch_step(solo_state* s, StepArgs& a, cudaStream_t stream) {
+// `full`: full tiles among the launch's (of tensors that are not 16-byte aligned too: the lists are device memory)
+int launch_step(solo_state* s, StepArgs& a, int64_t full, cudaStream_t stream) {
     a.debug_stall_tile_p1 = g_stall_tile_p1.exchange(0, std::memory_order_relaxed);
     const bool cta_group = s->block == 2048;
     const int policy = g_policy.load(std::memory_order_relaxed);
@@ -240,17 +241,32 @@ int launch_step(solo_state* s, StepArgs& a, cudaStream_t stream) {
     const bool streamlined = fast_ok && !a.tables_v && !a.round_m;
     const bool plain = !a.l2 && !a.belief && a.fixed_alpha == 0.0f && a.round_v && !a.tables_v && !a.round_m;
     solo::StepKernel k16 = nullptr;
-    // From one wave of tiles on; below, a tile's latency counts, which is shorter with twice the threads per tile
-    // (4/4 bit: 128 tiles 4.2 us against 5.0 us, 512 tiles, step after step, 8.3 and 9.8, 2048 tiles 23.6 and 18.9; 8/8 bit:
-    // 256 tiles 8.6 and 7.7).
-    // Lists need a second launch for the tiles that are not full (513 tiles 7.6 us against 9.4 us).  What the
-    // streamlined kernel has no path for, one tile on (Eq. 5 at one tile 9.7 us in the general kernel, 7.4 us here).
-    const bool all_full = !a.param_list && s->num_tensors == 1 && s->numel[0] % solo::TILE == 0;
-    // Blocks of 2048 (4/4 bit): 512 tiles 12.3 us against 14.4, 1024 tiles 18.5 and 15.8, 4096 tiles 48.0 and 46.7.
+    const int64_t rest = a.total_tiles - a.tile_first - full;
+    const bool all_full = !a.param_list && rest == 0;
     const bool w8 = s->bits_m == 8 || s->bits_v == 8;
-    const int64_t from = !streamlined ? (all_full ? 1 : 64)
-                                      : (cta_group ? (w8 ? 512 : 1024) : w8 ? 256 : 768) * (all_full ? 1 : 2);
-    const bool large = s->tiles_total >= from;
+    bool large;
+    if (all_full) {
+        // One launch either way.  From one wave of tiles on; below, a tile's latency counts, which is shorter with twice
+        // the threads per tile (4/4 bit: 128 tiles 4.2 us against 5.0 us, 512 tiles, step after step, 8.3 and 9.8, 2048 tiles
+        // 23.6 and 18.9; 8/8 bit: 256 tiles 8.6 and 7.7; blocks of 2048, 4/4 bit: 512 tiles 12.3 and 14.4, 1024 tiles 18.5
+        // and 15.8).  What the streamlined kernel has no path for, one tile on (Eq. 5 at one tile: general kernel 9.7, here 7.4).
+        large = full >= (!streamlined ? 1 : cta_group ? (w8 ? 512 : 1024) : w8 ? 256 : 768);
+    } else if (!streamlined) {
+        // The general kernel's fp32 parameters differ in the last bits, so the whole set decides, not the chunk of a
+        // host-buffer call.  Lists (us in one launch of the general kernel / in two): 768 full tiles 24.7 / 18.7, with 192
+        // others 33.9 / 26.4; 256 and 64 others 13.4 / 24.9; blocks of 2048, 768 and 48 others 23.3 / 30.6, 2048 and 128 55.8 / 48.3.
+        large = s->full_tiles >= (cta_group ? 1536 : 768);
+    } else if (cta_group) {
+        // Two launches against one (2/3 bit): 1024 full tiles and 64 others 31.6 / 18.5, 3072 and 192 49.2 / 54.0; 1024 and 512
+        // 36.7 / 50.6, 2048 and 2048 95.8 / 171.8: the streamlined kernel deals these tiles in turn and searches their tensors.
+        large = full + 4 * rest >= 2048;
+    } else {
+        // The second launch takes 6 us and per tile 8 us a thousand more than the streamlined kernel's own tails; the first
+        // saves 1.3 us a thousand (8-bit states 4).  2/3 bit, two launches against one: 3072 full tiles 30.0 / 34.3, 3072 and 192 others
+        // 35.3 / 35.2, 4608 and 288 46.2 / 50.2, 16384 and 4096 207 / 191; 8/8 bit: 2048 27.9 / 33.9, 3072 and 768 55.8 / 59.7,
+        // 8192 and 4096 183 / 190.
+        large = full >= 2048 + (w8 ? 2 : 6) * rest;
+    }
     if (fast_ok && ((policy == 0 && large) || policy == 3))
         k16 = solo::fast16_kernel(s->bits_m, s->bits_v, s->block, a.param_bf16 != 0,
                                   plain ? 0 : (a.tables_v || a.round_m) ? 2 : 1);
@@ -285,6 +301,7 @@ void fill_state_args(const solo_state* s, StepArgs& a) {
     a.tile_start = s->geom + T + (T + 1);
     a.num_tensors = T;
     a.total_tiles = s->tiles_total;
+    a.tensor_end = T;
     a.codes_m = s->codes_m;
     a.codes_v = s->codes_v;
     a.scale_m = s->scale_m;
@@ -391,6 +408,7 @@ int solo_state_create_multi(const int64_t* numel_host, int num_tensors, int bits
     s->numel_total = s->elem_start[T];
     s->nblk_total = s->block_start[T];
     s->tiles_total = s->tile_start[T];
+    for (int t = 0; t < T; ++t) s->full_tiles += numel_host[t] / solo::TILE;
     s->bytes_codes_m = (size_t)s->nblk_total * (size_t)(block * bits_m / 8);
     s->bytes_codes_v = (size_t)s->nblk_total * (size_t)(block * bits_v / 8);
 
@@ -516,7 +534,7 @@ int solo_step(void* param_dev, const void* grad_dev, solo_state_t* s, const solo
     select_v_codebook(s, hyper, a);
     a.param_single = param_dev;
     a.grad_single = grad_dev;
-    return launch_step(s, a, (cudaStream_t)stream);
+    return launch_step(s, a, s->full_tiles, (cudaStream_t)stream);
 }
 
 int solo_multi_step(const solo_tensor_list_t* list, const solo_hyper_t* hyper, int64_t step,
@@ -534,7 +552,7 @@ int solo_multi_step(const solo_tensor_list_t* list, const solo_hyper_t* hyper, i
     a.param_list = list->param;
     a.grad_list = list->grad;
     a.numel_check = list->numel;
-    return launch_step(s, a, (cudaStream_t)stream);
+    return launch_step(s, a, s->full_tiles, (cudaStream_t)stream);
 }
 
 namespace {
@@ -624,12 +642,14 @@ int solo_multi_step_host(const solo_host_list_t* list, const solo_hyper_t* hyper
         const int tensor_first = tensor;
         // upload: one piece per tensor that the chunk touches, each from a 16-byte boundary of the slot
         size_t off = 0;
+        int64_t full = 0;
         int t = tensor;
         for (; t < T && s->tile_start[t] < last; ++t) {
             const int64_t e_lo = (std::max<int64_t>(s->tile_start[t], first) - s->tile_start[t]) * solo::TILE;
             const int64_t e_hi = std::min<int64_t>(s->numel[t],
                                                    (std::min<int64_t>(s->tile_start[t + 1], last) - s->tile_start[t]) * solo::TILE);
             const size_t bytes = (size_t)(e_hi - e_lo) * 2;
+            full += (e_hi - e_lo) / solo::TILE;
             chk(cudaMemcpyAsync(hp->d_grad[slot] + off, (const char*)list->grad_host[t] + e_lo * 2, bytes,
                                 cudaMemcpyHostToDevice, st));
             // the kernel indexes gradients by the element's position in its tensor
@@ -644,7 +664,9 @@ int solo_multi_step_host(const solo_host_list_t* list, const solo_hyper_t* hyper
         a.grad_list = (const void* const*)hp->d_grad_list[slot];
         a.tile_first = first;
         a.total_tiles = last;
-        rc = launch_step(s, a, st);
+        a.tensor_first = tensor_first;
+        a.tensor_end = t_end;
+        rc = launch_step(s, a, full, st);
         if (rc) break;
         if (list->param_out_host) {
             for (t = tensor_first; t < t_end; ++t) {
@@ -699,11 +721,13 @@ int solo_multi_step_static(int32_t num_tensors, void* const* param_dev, const vo
     int64_t* tile_start = geom + T + (T + 1);
     block_start[0] = 0;
     tile_start[0] = 0;
+    int64_t full = 0;
     for (int t = 0; t < T; ++t) {
         if (numel_host[t] < 1) return SOLO_EINVAL;
         numel[t] = numel_host[t];
         block_start[t + 1] = block_start[t] + (numel_host[t] + block - 1) / block;
         tile_start[t + 1] = tile_start[t] + (numel_host[t] + solo::TILE - 1) / solo::TILE;
+        full += numel_host[t] / solo::TILE;
     }
     float tables[3 * 256 - 2];
     {
@@ -739,6 +763,7 @@ int solo_multi_step_static(int32_t num_tensors, void* const* param_dev, const vo
     tmp.device = device;
     tmp.bits_m = st->bits_m; tmp.bits_v = st->bits_v; tmp.block = block; tmp.num_tensors = T;
     tmp.tiles_total = tile_start[T];
+    tmp.full_tiles = full;
     tmp.nblk_total = block_start[T];
     StepArgs a;
     std::memset(&a, 0, sizeof(a));
@@ -747,6 +772,7 @@ int solo_multi_step_static(int32_t num_tensors, void* const* param_dev, const vo
     a.tile_start = d_geom + T + (T + 1);
     a.num_tensors = T;
     a.total_tiles = tmp.tiles_total;
+    a.tensor_end = T;
     a.codes_m = (uint8_t*)st->codes_m;
     a.codes_v = (uint8_t*)st->codes_v;
     a.scale_m = st->scale_m;
@@ -762,7 +788,7 @@ int solo_multi_step_static(int32_t num_tensors, void* const* param_dev, const vo
     a.param_list = param_dev;
     a.grad_list = grad_dev;
     a.numel_check = nullptr;
-    return launch_step(&tmp, a, stream);
+    return launch_step(&tmp, a, full, stream);
 }
 
 int solo_static_status(int* status_out, void* stream_) {

@@ -40,6 +40,7 @@ struct StepArgs {
     int32_t num_tensors;
     int64_t total_tiles;               // the launch covers tiles [tile_first, total_tiles)
     int64_t tile_first;
+    int32_t tensor_first, tensor_end;  // those tiles belong to tensors [tensor_first, tensor_end): no other entry of a list is read
     int32_t share;                     // sixteen-per-thread kernel: tiles of one CTA
     int32_t only_partial;              // streamlined and general kernel: skip full tiles of aligned tensors (another launch did them)
     int64_t debug_stall_tile_p1;       // test hook of the staged kernels: 1 + the number of the tile whose input copy
@@ -315,12 +316,12 @@ struct PartialWalk {
     int shared;                                  // 0: tensors dealt in turn, 1: unaligned tensors shared by all CTAs
     unsigned char flag[CTA];
 };
-__device__ __forceinline__ void partial_walk_begin(PartialWalk& w) {
+__device__ __forceinline__ void partial_walk_begin(const StepArgs& a, PartialWalk& w) {
     if (threadIdx.x == 0) {
-        w.tensor = (int)blockIdx.x - (int)gridDim.x;
+        w.tensor = a.tensor_first + (int)blockIdx.x - (int)gridDim.x;
         w.tin = 0;
         w.end = 0;
-        w.group = -CTA;
+        w.group = a.tensor_first - CTA;
         w.i = CTA;
         w.shared = 0;
     }
@@ -344,7 +345,7 @@ __device__ __noinline__ inline bool partial_walk_next(const StepArgs& a, Partial
         if (found) break;
         if (!shared) {
             t += (int)gridDim.x;
-            if (t < a.num_tensors) {
+            if (t < a.tensor_end) {
                 const int64_t n = __ldg(a.numel + t), tiles = (n + TILE - 1) / TILE;
                 tin = end = 0;
                 if (a.numel_check != nullptr && __ldg(a.numel_check + t) != n) {
@@ -362,9 +363,9 @@ __device__ __noinline__ inline bool partial_walk_next(const StepArgs& a, Partial
         while (i < CTA && !w.flag[i]) ++i;
         if (i == CTA) {                                          // the next group of as many tensors as the CTA has threads
             group += CTA;
-            if (group >= a.num_tensors) break;
+            if (group >= a.tensor_end) break;
             const int mine = group + (int)threadIdx.x;
-            const bool f = mine < a.num_tensors && __ldg(a.numel + mine) > (int64_t)PartialWalk::ALONE * TILE && !aligned(mine) &&
+            const bool f = mine < a.tensor_end && __ldg(a.numel + mine) > (int64_t)PartialWalk::ALONE * TILE && !aligned(mine) &&
                            (a.numel_check == nullptr || __ldg(a.numel_check + mine) == __ldg(a.numel + mine));
             __syncthreads();                                     // the flags of the last group have been read
             w.flag[threadIdx.x] = f;
@@ -432,7 +433,7 @@ __global__ void __launch_bounds__(CTA) solo_step_kernel(const __grid_constant__ 
 
     // Tiles are dealt out in turn; after a launch that did the full tiles of the aligned tensors, the rest (PartialWalk).
     __shared__ PartialWalk walk;
-    partial_walk_begin(walk);
+    partial_walk_begin(a, walk);
     for (int64_t tile = a.tile_first + (int64_t)blockIdx.x - gridDim.x;;) {
         int tensor;
         if (a.only_partial) {

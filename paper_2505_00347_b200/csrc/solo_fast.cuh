@@ -1137,7 +1137,7 @@ __global__ void __launch_bounds__(CTA, (BM == 8 || BV == 8) ? 3 : 4) solo_step_f
     int par = 0;
     if constexpr (TAILS) {
         __shared__ PartialWalk walk;
-        partial_walk_begin(walk);
+        partial_walk_begin(a, walk);
         while (partial_walk_next(a, walk)) {
             const int t = walk.tensor, tin = (int)walk.tin;
             fast_tile<BM, BV, G, false, PBF, PLAIN>(
