@@ -147,9 +147,19 @@ def _check(rc: int, what: str) -> None:
         raise SoloError(rc, what)
 
 
+_raw_stream = None            # (device) -> handle of its current stream, once CUDA is initialised
+
+
 def _stream() -> int:
-    # (torch.cuda.current_stream() builds a Stream object on every call: 1 us of a 4 us launch)
-    return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())
+    # torch.cuda.current_stream() builds a Stream object on every call: 1 us of a 4 us launch.  The functions beneath it are
+    # not public: the first call goes through the public one, which also initialises CUDA, and so do all where they are missing.
+    global _raw_stream
+    if _raw_stream is not None:
+        return _raw_stream(torch._C._cuda_getDevice())
+    handle = torch.cuda.current_stream().cuda_stream
+    if hasattr(torch._C, "_cuda_getDevice"):
+        _raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    return handle
 
 
 RAW = {"codes_m": 0, "codes_v": 1, "scale_m": 2, "scale_v": 3, "alpha": 4}
@@ -319,7 +329,7 @@ class TensorSet:
 
 
 def solo_multi_step(ts: TensorSet, h: Hyper, step: int) -> None:
-    """One fused step over the whole tensor list in one launch, on the current stream."""
+    """One fused step over the whole tensor list, in one launch or two (solo_multi_step in solo.h), on the current stream."""
     rc = (_lib or lib()).solo_multi_step(C.byref(ts.desc), C.byref(h), step, _stream())
     if rc:
         _check(rc, "solo_multi_step")
