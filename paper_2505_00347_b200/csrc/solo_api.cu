@@ -287,7 +287,9 @@ int launch_step(solo_state* s, StepArgs& a, int64_t full, cudaStream_t stream) {
         if (!a.param_list) a.tile_first = s->tiles_total - 1;
     }
     solo::StepKernel k = nullptr;
-    if (streamlined) k = solo::fast_kernel(s->bits_m, s->bits_v, s->block, a.param_bf16 != 0, plain, a.only_partial != 0);
+    if (streamlined)
+        k = a.only_partial ? solo::fast_tails_kernel(s->bits_m, s->bits_v, s->block, a.param_bf16 != 0)
+                           : solo::fast_kernel(s->bits_m, s->bits_v, s->block, a.param_bf16 != 0, plain);
     size_t dyn_smem = k ? solo::fast_kernel_smem(s->bits_m, s->bits_v) : 0;
     if (!k) k = solo::step_kernel(s->bits_m, s->bits_v, cta_group);
     if (!k) return SOLO_EINVAL;

@@ -18,14 +18,24 @@ StepKernel step_kernel(int bits_m, int bits_v, bool cta_group) {
     }
 }
 
-StepKernel fast_kernel(int bits_m, int bits_v, int block, bool param_bf16, bool plain, bool tails) {
+StepKernel fast_kernel(int bits_m, int bits_v, int block, bool param_bf16, bool plain) {
     const int bv = bits_index(bits_v);
-    if (bv < 0) return nullptr;
     switch (bits_m) {
-        case 2: return (tails ? fast_tails_kernel_bm2 : fast_kernel_bm2)(bv, block, param_bf16, plain);
-        case 3: return (tails ? fast_tails_kernel_bm3 : fast_kernel_bm3)(bv, block, param_bf16, plain);
-        case 4: return (tails ? fast_tails_kernel_bm4 : fast_kernel_bm4)(bv, block, param_bf16, plain);
-        case 8: return (tails ? fast_tails_kernel_bm8 : fast_kernel_bm8)(bv, block, param_bf16, plain);
+        case 2: return fast_kernel_bm2(bv, block, param_bf16, plain);
+        case 3: return fast_kernel_bm3(bv, block, param_bf16, plain);
+        case 4: return fast_kernel_bm4(bv, block, param_bf16, plain);
+        case 8: return fast_kernel_bm8(bv, block, param_bf16, plain);
+        default: return nullptr;
+    }
+}
+
+StepKernel fast_tails_kernel(int bits_m, int bits_v, int block, bool param_bf16) {
+    const int bv = bits_index(bits_v);
+    switch (bits_m) {
+        case 2: return fast_tails_kernel_bm2(bv, block, param_bf16);
+        case 3: return fast_tails_kernel_bm3(bv, block, param_bf16);
+        case 4: return fast_tails_kernel_bm4(bv, block, param_bf16);
+        case 8: return fast_tails_kernel_bm8(bv, block, param_bf16);
         default: return nullptr;
     }
 }

@@ -37,12 +37,13 @@ StepKernel fast_kernel_bm2(int bv_index, int block, bool param_bf16, bool plain)
 StepKernel fast_kernel_bm3(int bv_index, int block, bool param_bf16, bool plain);
 StepKernel fast_kernel_bm4(int bv_index, int block, bool param_bf16, bool plain);
 StepKernel fast_kernel_bm8(int bv_index, int block, bool param_bf16, bool plain);
-StepKernel fast_tails_kernel_bm2(int bv_index, int block, bool param_bf16, bool plain);
-StepKernel fast_tails_kernel_bm3(int bv_index, int block, bool param_bf16, bool plain);
-StepKernel fast_tails_kernel_bm4(int bv_index, int block, bool param_bf16, bool plain);
-StepKernel fast_tails_kernel_bm8(int bv_index, int block, bool param_bf16, bool plain);
-// `tails`: the kernel for the tiles that the sixteen-per-thread kernel leaves
-StepKernel fast_kernel(int bits_m, int bits_v, int block, bool param_bf16, bool plain, bool tails);
+StepKernel fast_tails_kernel_bm2(int bv_index, int block, bool param_bf16);
+StepKernel fast_tails_kernel_bm3(int bv_index, int block, bool param_bf16);
+StepKernel fast_tails_kernel_bm4(int bv_index, int block, bool param_bf16);
+StepKernel fast_tails_kernel_bm8(int bv_index, int block, bool param_bf16);
+StepKernel fast_kernel(int bits_m, int bits_v, int block, bool param_bf16, bool plain);
+// The kernel for the tiles that the sixteen-per-thread kernel leaves; it reads the modes at run time.
+StepKernel fast_tails_kernel(int bits_m, int bits_v, int block, bool param_bf16);
 // Sixteen elements per thread: fp32 or bf16 parameters; `modes`: 0 as `plain` for
 // fast_kernel, 1 the modes fast_kernel reads at run time, 2 those plus Eq. 5 rounding and the baseline
 // second-moment codebooks; full tiles

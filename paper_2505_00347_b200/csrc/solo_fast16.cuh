@@ -276,11 +276,10 @@ __device__ __forceinline__ int group_count4(bool p0, bool p1, bool p2, bool p3, 
         const uint32_t sel = (lane & 16) ? 0x7632u : 0x5410u;
         return __popc(__byte_perm(b0, b1, sel)) + __popc(__byte_perm(b2, b3, sel));
     } else {
-        // the byte of each ballot that holds the group (two groups of four)
+        static_assert(G == 8, "groups of four select by pops");
+        // the byte of each ballot that holds the group
         const uint32_t sel = 0x40u + 0x11u * ((uint32_t)lane >> 3);
-        uint32_t b = __byte_perm(__byte_perm(b0, b1, sel), __byte_perm(b2, b3, sel), 0x5410u);
-        if constexpr (G == 4) b &= (lane & 4) ? 0xF0F0F0F0u : 0x0F0F0F0Fu;
-        return __popc(b);
+        return __popc(__byte_perm(__byte_perm(b0, b1, sel), __byte_perm(b2, b3, sel), 0x5410u));
     }
 }
 

@@ -1,5 +1,5 @@
 // Instantiations of the streamlined step kernel for one first-moment width (SOLO_BM = 2, 3, 4, 8): for all tiles
-// (SOLO_TAILS = 0) or for those the sixteen-per-thread kernel leaves (SOLO_TAILS = 1).
+// (SOLO_TAILS = 0) or for those the sixteen-per-thread kernel leaves (SOLO_TAILS = 1: a few tiles, modes read at run time).
 #include "solo_dispatch.h"
 #include "solo_fast.cuh"
 
@@ -21,20 +21,28 @@ namespace solo {
 #define SOLO_PLANE(PBF, PLAIN) \
     {SOLO_ROW(2, PBF, PLAIN), SOLO_ROW(3, PBF, PLAIN), SOLO_ROW(4, PBF, PLAIN), SOLO_ROW(8, PBF, PLAIN)}
 
+static int block_index(int block) {
+    return block == 64 ? 0 : block == 128 ? 1 : block == 256 ? 2 : block == 2048 ? 3 : -1;
+}
+
 #if SOLO_TAILS
-#define SOLO_FAST_NAME SOLO_CAT(fast_tails_kernel_bm, SOLO_BM)
+StepKernel SOLO_CAT(fast_tails_kernel_bm, SOLO_BM)(int bv_index, int block, bool param_bf16) {
+    static const StepKernel table[2][4][4] = {SOLO_PLANE(false, false), SOLO_PLANE(true, false)};
+    const int g = block_index(block);
+    if (bv_index < 0 || bv_index > 3 || g < 0) return nullptr;
+    return table[param_bf16 ? 1 : 0][bv_index][g];
+}
 #else
-#define SOLO_FAST_NAME SOLO_CAT(fast_kernel_bm, SOLO_BM)
-#endif
-StepKernel SOLO_FAST_NAME(int bv_index, int block, bool param_bf16, bool plain) {
+StepKernel SOLO_CAT(fast_kernel_bm, SOLO_BM)(int bv_index, int block, bool param_bf16, bool plain) {
     static const StepKernel table[2][2][4][4] = {
         {SOLO_PLANE(false, false), SOLO_PLANE(true, false)},
         {SOLO_PLANE(false, true), SOLO_PLANE(true, true)},
     };
-    const int g = block == 64 ? 0 : block == 128 ? 1 : block == 256 ? 2 : block == 2048 ? 3 : -1;
+    const int g = block_index(block);
     if (bv_index < 0 || bv_index > 3 || g < 0) return nullptr;
     return table[plain ? 1 : 0][param_bf16 ? 1 : 0][bv_index][g];
 }
+#endif
 
 #if SOLO_BM == 2 && !SOLO_TAILS
 // Exhaustive check of the error model used above: for every binary32 x with bit pattern
