@@ -17,6 +17,7 @@ OBJ_DIR = PKG / "_build"
 NVCC_FLAGS = [
     "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
     "-fmad=false", "-prec-div=true", "-prec-sqrt=true", "-ftz=false",
+    "--compress-mode=size",
     "-Xcompiler", "-fPIC", f"-I{INCLUDE}", f"-I{CSRC}",
 ]
 
@@ -73,7 +74,7 @@ def build(force: bool = False, verbose: bool = False, ptxas_info: bool = False) 
                 raise RuntimeError(f"nvcc failed on {unit[0]} ({unit[2]})")
     objs = [str(OBJ_DIR / u[1]) for u in UNITS]
     tmp = LIB.with_suffix(f".tmp{os.getpid()}.so")
-    subprocess.run([nvcc, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "-o", str(tmp),
+    subprocess.run([nvcc, "-shared", "-gencode", "arch=compute_100a,code=sm_100a", "--compress-mode=size", "-o", str(tmp),
                     *objs], check=True)
     os.replace(tmp, LIB)
     stamp.write_text(key)
