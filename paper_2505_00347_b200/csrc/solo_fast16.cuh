@@ -233,6 +233,13 @@ __device__ __forceinline__ uint32_t pack8(uint32_t a, uint32_t b, uint32_t c, ui
     return __byte_perm(__byte_perm(a, b, 0x0040u), __byte_perm(c, d, 0x0040u), 0x5410u);
 }
 
+// A block's scale for its reciprocal: a vanishing one (below TINY; its codes are zeroed) counts as TINY, so that no ratio exceeds 1
+// and the ratios index the cell tables; a NaN stays one.  On the pattern: a selection of 0 instead made 4/4 bit at block 2048
+// spill twice as much (ragged set 5411 -> 5821 us).
+__device__ __forceinline__ float at_least_tiny(uint32_t scale) {
+    return __uint_as_float(max(scale, 0x0D800000u));
+}
+
 // Minimum / maximum over the calling lane's group of G lanes.  The shuffle-and-compare steps serve
 // all groups of the warp at once; for groups of eight measured faster here than the full-mask reductions
 // over a transformed value that solo_fast.cuh uses for its groups of sixteen (four REDUX plus selects for
@@ -613,7 +620,7 @@ __device__ __forceinline__ void block_scalars16(const StepArgs& a, Shared& s, co
     const uint4 in = s.xin[tid];
     const float dm_new = __uint_as_float(in.x), dv_new = __uint_as_float(in.y);
     const bool zero_m = dm_new < TINY, zero_v = dv_new < TINY;
-    const float inv_dv = zero_v ? 0.0f : __frcp_rn(dv_new);      // (no infinity: the ratios index the cell tables)
+    const float inv_dv = __frcp_rn(at_least_tiny(in.y));
     const float rho = fminf(fmaxf(__uint_as_float(in.z) * inv_dv, RHO_MIN), RHO_MAX);
     const float lam = log2_sp(rho) * (1.0f / (float)(KV - 1));
     // (a baseline codebook has no base: the array keeps its initial 1/2)
@@ -970,7 +977,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     if constexpr (G != 128) mx_m = group_max16<G>(mx_m);
     uint32_t om[BM == 8 ? 4 : 2] = {};                            // eight codes per word, 8-bit: four
     const float dm_new = __uint_as_float(mx_m);
-    const float inv_m = dm_new < TINY ? 0.0f : __frcp_rn(dm_new);   // (no infinity: the ratios index the cell tables)
+    const float inv_m = __frcp_rn(at_least_tiny(mx_m));
     // code = number of midpoints below r, each comparison as the saturation of (r - mid) * 2^100 on the FMA
     // pipe (exactly 0 or 1, see fast_tile).  The codes of elements 2j and 2j + 1 are accumulated side by side
     // in one pair of binary32 (eight 2- or 3-bit codes per pair, at most 21 bits each: exact).
