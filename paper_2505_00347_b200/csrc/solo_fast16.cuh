@@ -909,67 +909,80 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
         // below 2^-126 is not rounded to the subnormal grid before it is multiplied, which shows in results below
         // 2^-99 |step_size| <= 2^-80 only (in others it is lost against the parameter): a warp that gets one takes the IEEE
         // operations instead, the parameters being in the stage still.  Two looks: exponent bit 6 is set in all results
-        // from 2^-63 to 2 (one operation per four of them), whatever lacks it is compared.
+        // from 2^-63 to 2 (one operation per four of them), whatever lacks it is compared.  The two passes one after the other,
+        // and not two sides of a branch per half: LLaMA layer, 2/2 bit, 757 -> 716 us (one loop around both 747, and 2/2 bit with Eq. 5
+        // spilled: 659 -> 723 us on 2^27 elements, as it is 646).
         bool exact = __all_sync(0xffffffffu, tmx_v < 0x4D000000u && mx_m_f < 0x1p20f && a.eps < 0x1p30f && a.inv_sqrt_bc2 < 0x1p30f &&
                                                  fabsf(a.step_size) > 0x1p-40f && fabsf(a.step_size) < 0x1p19f);
-        for (;;) {
+        auto load8 = [&](int h, float (&p)[8]) {
+            const uint4 pw = sp[(uint32_t)h ^ sw];
+            const uint32_t pin[4] = {pw.x, pw.y, pw.z, pw.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                p[2 * k] = __uint_as_float(pin[k] << 16);
+                p[2 * k + 1] = __uint_as_float(pin[k] & 0xffff0000u);
+            }
+        };
+        auto store8 = [&](int h, const float (&p)[8]) {             // returns the conjunction of the patterns
+            const uint32_t he = (uint32_t)h ^ sw;
+            uint32_t pp[4];
+            if (a.param_sr) {
+                uint32_t wp[4], ctr_lo, ctr_hi, c3;
+                stream_position(ctr_lo, ctr_hi, c3);
+                philox_rk(ctr_lo + he, ctr_hi, a.step32, c3 + 2u, a.rk, wp);
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    pp[k] = bf16_sr(p[2 * k], wp[k] & 0xFFFFu) | (bf16_sr(p[2 * k + 1], wp[k] >> 16) << 16);
+            } else {
+#pragma unroll
+                for (int k = 0; k < 4; ++k) {
+                    const __nv_bfloat162 h2 = __floats2bfloat162_rn(p[2 * k], p[2 * k + 1]);
+                    pp[k] = *reinterpret_cast<const uint32_t*>(&h2);
+                }
+            }
+            __stcs(reinterpret_cast<uint4*>(pt) + 2 * tid + he, make_uint4(pp[0], pp[1], pp[2], pp[3]));
+            return (pp[0] & pp[1]) & (pp[2] & pp[3]);
+        };
+        if (exact) {
             uint32_t all = 0xFFFFFFFFu;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
-                const uint32_t he = (uint32_t)h ^ sw;
-                const uint4 pw = sp[he];
-                const uint32_t pin[4] = {pw.x, pw.y, pw.z, pw.w};
                 float p[8];
+                load8(h, p);
+                const F2 nisb = F2::dup(-a.inv_sqrt_bc2 * 0x1p-50f), eps = F2::dup(a.eps), lr = F2::dup(a.step_size * 0x1p-64f);
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    p[2 * k] = __uint_as_float(pin[k] << 16);
-                    p[2 * k + 1] = __uint_as_float(pin[k] & 0xffff0000u);
+                    const int j = 4 * h + k;
+                    const F2 den = fma2(neg_sqrt2(mul2(vh[j], F2::dup(-0x1p100f))), nisb, eps);
+                    const F2 nq = neg_div2(mul2(mh[j], F2::dup(0x1p64f)), den);
+                    F2 pj = F2::pack(p[2 * k], p[2 * k + 1]);
+                    pj = fma2(lr, nq, DECAY ? mul2(pj, F2::dup(a.decay)) : pj);
+                    p[2 * k] = pj.lo();
+                    p[2 * k + 1] = pj.hi();
                 }
-                if (exact) {
-                    const F2 nisb = F2::dup(-a.inv_sqrt_bc2 * 0x1p-50f), eps = F2::dup(a.eps), lr = F2::dup(a.step_size * 0x1p-64f);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const int j = 4 * h + k;
-                        const F2 den = fma2(neg_sqrt2(mul2(vh[j], F2::dup(-0x1p100f))), nisb, eps);
-                        const F2 nq = neg_div2(mul2(mh[j], F2::dup(0x1p64f)), den);
-                        F2 pj = F2::pack(p[2 * k], p[2 * k + 1]);
-                        pj = fma2(lr, nq, DECAY ? mul2(pj, F2::dup(a.decay)) : pj);
-                        p[2 * k] = pj.lo();
-                        p[2 * k + 1] = pj.hi();
-                    }
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 8; ++k) {
-                        const int i = 8 * h + k;
-                        const float den = __fmaf_rn(__fsqrt_rn(vh_at(i)), a.inv_sqrt_bc2, a.eps);
-                        p[k] = __fmaf_rn(-a.step_size, __fdiv_rn(mh_at(i), den), DECAY ? p[k] * a.decay : p[k]);
-                    }
-                }
-                uint32_t pp[4];
-                if (a.param_sr) {
-                    uint32_t wp[4], ctr_lo, ctr_hi, c3;
-                    stream_position(ctr_lo, ctr_hi, c3);
-                    philox_rk(ctr_lo + he, ctr_hi, a.step32, c3 + 2u, a.rk, wp);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        pp[k] = bf16_sr(p[2 * k], wp[k] & 0xFFFFu) | (bf16_sr(p[2 * k + 1], wp[k] >> 16) << 16);
-                } else {
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const __nv_bfloat162 h2 = __floats2bfloat162_rn(p[2 * k], p[2 * k + 1]);
-                        pp[k] = *reinterpret_cast<const uint32_t*>(&h2);
-                    }
-                }
-                all &= (pp[0] & pp[1]) & (pp[2] & pp[3]);
-                __stcs(reinterpret_cast<uint4*>(pt) + 2 * tid + he, make_uint4(pp[0], pp[1], pp[2], pp[3]));
+                all &= store8(h, p);
             }
-            if (!exact || !__any_sync(0xffffffffu, (~all & 0x20002000u) != 0u)) break;
-            uint32_t least = 0x7FFFu;                             // of the patterns stored, signs off
+            if (__any_sync(0xffffffffu, (~all & 0x20002000u) != 0u)) {
+                uint32_t least = 0x7FFFu;                         // of the patterns stored, signs off
 #pragma unroll 1
-            for (int i = 0; i < EPT16; ++i)
-                least = min(least, reinterpret_cast<const unsigned short*>(pt)[EPT16 * tid + i] & 0x7FFFu);
-            if (!__any_sync(0xffffffffu, least < 0x1800u)) break;                 // 2^-79: no result below 2^-80 was rounded up to it
-            exact = false;
+                for (int i = 0; i < EPT16; ++i)
+                    least = min(least, reinterpret_cast<const unsigned short*>(pt)[EPT16 * tid + i] & 0x7FFFu);
+                exact = !__any_sync(0xffffffffu, least < 0x1800u);        // 2^-79: no result below 2^-80 was rounded up to it
+            }
+        }
+        if (!exact) {
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                float p[8];
+                load8(h, p);
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    const int i = 8 * h + k;
+                    const float den = __fmaf_rn(__fsqrt_rn(vh_at(i)), a.inv_sqrt_bc2, a.eps);
+                    p[k] = __fmaf_rn(-a.step_size, __fdiv_rn(mh_at(i), den), DECAY ? p[k] * a.decay : p[k]);
+                }
+                store8(h, p);
+            }
         }
     }
 
