@@ -16,7 +16,8 @@
 // selection) is spent once per sixteen elements instead of once per eight.
 //
 // Resources are cut for seven or eight resident CTAs per SM (ctas16): at most 72 or 64 registers per thread
-// and one input stage of 13.6 KB (15 KB of shared memory in all; 23 KB for blocks of 64).  The stage is read only
+// and one input stage of 13.6 KB (15 KB of shared memory in all; 23 KB for blocks of 64); with 8-bit states six or seven CTAs,
+// at most 80 or 72 registers and up to 39 KB.  The stage is read only
 // before the tile's first CTA barrier, so the copies of the CTA's next tile are issued right after
 // that barrier and land while the tile's second half (per-block scalars, random draws,
 // quantization) runs.  Parameters stay in the stage until the update of their four elements needs
@@ -39,7 +40,7 @@
 //
 // This kernel processes full tiles of 16-byte aligned tensors only; every other tile is left to
 // a second launch with StepArgs::only_partial set: of solo_step_fast_kernel, or of the general kernel
-// where that one has no path (the baseline codebooks).
+// where that one has no path (Eq. 5, the baseline codebooks).
 #pragma once
 
 #include "solo_dispatch.h"
@@ -552,7 +553,8 @@ __device__ __forceinline__ int steal_answer(Shared& s, int* status) {
 // so end together whatever their speed, a CTA sets up once for many shares, and inputs are copied ahead across
 // tensors and shares.  One share per resident CTA (a static walk) left 5 % of the SM cycles idle at the launch's
 // end and SMs with fewer CTAs before it: LLaMA layers 2357 -> 2170 us, GPT-125M-shaped set 432 -> 390 us, ragged set
-// 3418 -> 3200 us, 2^24 elements 60 -> 55 us.
+// 3418 -> 3200 us, 2^24 elements 60 -> 55 us (bursts of ten steps; for seconds on end, at the power limit, the
+// GPT-125M-shaped set takes 416 us and the ragged one 3480).
 // A CTA that waited in vain for a copy ends here: it takes in the answer to its last request, so that nothing writes to its
 // shared memory any more, and asks for no other.  What it then leaves unstepped (and has reported in the status word) is
 // the rest of its share and at most the one that answer brought, however many CTAs have not started yet.
