@@ -292,11 +292,10 @@ float solo_default_beta1(int bits_m, int from_scratch);
  * enough full tiles of 2048 elements run
  * them in a kernel with sixteen elements per thread and the remaining tiles in the
  * streamlined kernel, or in the general one where the streamlined kernel does not apply (two
- * launches).  Enough: for one tensor of whole tiles (one launch) 768, 256 with an 8-bit state, 1024 or 512 with
- * blocks of 2048, one where the streamlined kernel does not apply; for lists and other tensors, with r
- * tiles that are not full, 2048 + 6 r (2048 + 2 r with an 8-bit state, 2048 - 4 r with blocks of 2048), or 768 (1536 with
- * blocks of 2048) where the streamlined kernel does not apply; the chunks of solo_multi_step_host each count for
- * themselves, except in the last case.  That kernel covers every mode of solo_hyper_t (Eq. 5 rounding and the baseline
+ * launches).  Enough is, for one tensor of whole tiles (one launch), 768, 256 with an 8-bit state, 1024 or 512 with
+ * blocks of 2048, one where the streamlined kernel does not apply; for lists and other tensors some 2000 and more the more
+ * tiles are not full, 320 to 1664 where the streamlined kernel does not apply.  The chunks of solo_multi_step_host
+ * each count for themselves, except in the last case.  That kernel covers every mode of solo_hyper_t (Eq. 5 rounding and the baseline
  * second-moment codebooks included) and every p.  1: always the general kernel.  2: like 0 without the
  * sixteen-per-thread kernel.  3: like 0 with the sixteen-per-thread kernel whatever the tensor
  * sizes.  All produce the same packed state and the same bf16 parameters; the fp32 parameters

@@ -252,20 +252,27 @@ int launch_step(solo_state* s, StepArgs& a, int64_t full, cudaStream_t stream) {
         // and 15.8).  What the streamlined kernel has no path for, one tile on (Eq. 5 at one tile: general kernel 9.7, here 7.4).
         large = full >= (!streamlined ? 1 : cta_group ? (w8 ? 512 : 1024) : w8 ? 256 : 768);
     } else if (!streamlined) {
-        // The general kernel's fp32 parameters differ in the last bits, so the whole set decides, not the chunk of a
-        // host-buffer call.  Lists (us in one launch of the general kernel / in two): 768 full tiles 24.7 / 18.7, with 192
-        // others 33.9 / 26.4; 256 and 64 others 13.4 / 24.9; blocks of 2048, 768 and 48 others 23.3 / 30.6, 2048 and 128 55.8 / 48.3.
-        large = s->full_tiles >= (cta_group ? 1536 : 768);
+        // Lists, and tensors with a tail, need a second launch: 6 to 10 us after the first.  Here the whole set decides and not the
+        // chunk of a host-buffer call, because the general kernel's fp32 parameters differ in the last bits.  Us in one launch of the
+        // general kernel / in two (4/2 bit Eq. 5): full tiles only 256 13.3 / 13.0, 768 24.7 / 18.7; with a tail 512 19.2 / 21.8, 768
+        // 22.6 / 23.7, 1024 29.9 / 25.4 (8-bit dynamic exponent 512 18.0 / 19.3, 768 25.6 / 20.4); blocks of 2048: full tiles
+        // only 768 23.5 / 21.9, with a tail 1536 41.0 / 41.5, 2048 50.9 / 43.1.
+        const bool others = s->tiles_total != s->full_tiles;
+        large = s->full_tiles >= (cta_group ? (others ? 1664 : 768) : (others ? 640 : 320));
     } else if (cta_group) {
-        // Two launches against one (2/3 bit): 1024 full tiles and 64 others 31.6 / 18.5, 3072 and 192 49.2 / 54.0; 1024 and 512
-        // 36.7 / 50.6, 2048 and 2048 95.8 / 171.8: the streamlined kernel deals these tiles in turn and searches their tensors.
-        large = full + 4 * rest >= 2048;
+        // One launch / two, 2/3 bit (8/8 bit): full tiles only 1024 21.4 / 18.5 (29.9 / 21.6); 2048 and 128 others 36.6 / 39.5 (46.8 / 44.4),
+        // 3072 and 192 54.0 / 49.2; 1024 and 256 32.0 / 35.1 (36.5 / 39.7), 1536 and 384 47.3 / 36.8: the streamlined kernel
+        // deals these tiles in turn and searches their tensors.  One tensor with a tail needs no search: 3072 34.9 / 42.7, the
+        // second launch being made up for by 1.5 us a thousand tiles (8/8 bit: 2048 37.6 / 38.2, 3072 51.6 / 49.3).
+        large = s->num_tensors == 1 ? full >= (w8 ? 2304 : 6144)
+                : rest == 0         ? full >= 1024
+                                    : full + 4 * rest >= (w8 ? 2400 : 2816);
     } else {
-        // The second launch takes 6 us and per tile 8 us a thousand more than the streamlined kernel's own tails; the first
-        // saves 1.3 us a thousand (8-bit states 4).  2/3 bit, two launches against one: 3072 full tiles 30.0 / 34.3, 3072 and 192 others
-        // 35.3 / 35.2, 4608 and 288 46.2 / 50.2, 16384 and 4096 207 / 191; 8/8 bit: 2048 27.9 / 33.9, 3072 and 768 55.8 / 59.7,
-        // 8192 and 4096 183 / 190.
-        large = full >= 2048 + (w8 ? 2 : 6) * rest;
+        // The second launch takes 6 us, and per tile 8 us a thousand more than the streamlined kernel's own tails; the first
+        // saves 1.3 us a thousand (8-bit states 4).  One launch / two, 2/3 bit: full tiles only 2048 23.9 / 23.5, 3072 34.3 / 30.0, with
+        // a tail 2048 22.6 / 24.7, 3072 32.5 / 27.5; 3072 and 192 others 35.2 / 35.3, 4608 and 288 50.2 / 46.2, 16384 and 4096
+        // 191 / 207; 8/8 bit: 1536 26.2 / 28.5, 2048 31.7 / 29.4, 3072 and 768 59.7 / 55.8, 8192 and 4096 190 / 183.
+        large = full >= (w8 ? 1664 + 2 * rest : 2048 + 6 * rest);
     }
     if (fast_ok && ((policy == 0 && large) || policy == 3))
         k16 = solo::fast16_kernel(s->bits_m, s->bits_v, s->block, a.param_bf16 != 0,
