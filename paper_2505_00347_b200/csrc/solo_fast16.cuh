@@ -292,19 +292,35 @@ __device__ __forceinline__ int group_count4(bool p0, bool p1, bool p2, bool p3, 
 }
 
 // The rank-th smallest (1-based) of the values that the G lanes of a group hold, one each: the lanes sort
-// them among themselves (bitonic network over shuffles) and read the lane of that rank.
+// them among themselves (bitonic network over shuffles, every stage ascending, the first of each merge against the mirrored
+// lane) and read the lane of that rank.
 template <int G>
 __device__ __forceinline__ uint32_t lanes_rank(uint32_t x, int rank, int lane) {
 #pragma unroll
     for (int size = 2; size <= G; size <<= 1) {
 #pragma unroll
         for (int d = size >> 1; d >= 1; d >>= 1) {
-            const uint32_t y = __shfl_xor_sync(0xffffffffu, x, d);
-            const bool upper = ((lane & d) != 0) != (size < G && (lane & size) != 0);      // this lane keeps the larger one
-            x = (y < x) != upper ? y : x;
+            const uint32_t y = __shfl_xor_sync(0xffffffffu, x, 2 * d == size ? size - 1 : d);
+            x = (y < x) != ((lane & d) != 0) ? y : x;
         }
     }
     return __shfl_sync(0xffffffffu, x, (lane & ~(G - 1)) + rank - 1);
+}
+
+// Drops the head of a sorted list if it is at most t and n < rem (`p`, `go`: the same as predicates).  Groups of eight: the entries
+// move up by predicated additions of `zero`, which the compiler does not know: an addition goes to any of the integer pipes at
+// one warp a cycle, a selection to one that takes a warp every other cycle (2^26 elements, 2/3 bit 186.7 -> 183.5 us, 3/3 bit 204.3 ->
+// 201; bf16 parameters, 2/2 bit, 249 -> 240).  Groups of sixteen and the CTA's selections are faster (4/4 bit 220 us against 232).
+template <int G>
+__device__ __forceinline__ void list_drop(uint32_t (&l)[4], const bool p, const bool go, const int n, const int rem, const uint32_t t,
+                                          const uint32_t zero) {
+    if constexpr (G == 8) {
+        asm("{\n\t.reg .pred g, p;\n\tsetp.lt.s32 g, %4, %5;\n\tsetp.le.and.u32 p, %0, %6, g;\n\t@p add.u32 %0, %1, %7;\n\t@p add.u32 %1, %2, %7;\n\t"
+            "@p add.u32 %2, %3, %7;\n\t@p add.u32 %3, %7, 0x7FFFFFFF;\n\t}"
+            : "+r"(l[0]), "+r"(l[1]), "+r"(l[2]), "+r"(l[3]) : "r"(n), "r"(rem), "r"(t), "r"(zero));
+    } else if (p && go) {
+        l[0] = l[1]; l[1] = l[2]; l[2] = l[3]; l[3] = KEY_MAX;
+    }
 }
 
 // k-th smallest (1-based, duplicates counted) of the 16 * G keys of a group of G lanes; each lane holds its
@@ -318,7 +334,7 @@ __device__ __forceinline__ uint32_t lanes_rank(uint32_t x, int rank, int lane) {
 // ROUNDS rounds are laid out in line, the others loop.  Every loop ends: a round drops at least one key (the
 // loops are bounded by k all the same).
 template <int G, int ROUNDS>
-__device__ __forceinline__ uint32_t select_rank16(uint32_t (&l)[4][4], const int k, const int lane) {
+__device__ __forceinline__ uint32_t select_rank16(uint32_t (&l)[4][4], const int k, const int lane, const uint32_t zero) {
     const uint32_t vx = G == 16 && (lane & 16) ? 0xFFFFFFFFu : 0u;
     int rem = k;
     auto round = [&]() {
@@ -329,8 +345,7 @@ __device__ __forceinline__ uint32_t select_rank16(uint32_t (&l)[4][4], const int
         const int n = group_count4<G>(p[0], p[1], p[2], p[3], lane);
         const bool go = n < rem;
 #pragma unroll
-        for (int q = 0; q < 4; ++q)
-            if (p[q] && go) { l[q][0] = l[q][1]; l[q][1] = l[q][2]; l[q][2] = l[q][3]; l[q][3] = KEY_MAX; }
+        for (int q = 0; q < 4; ++q) list_drop<G>(l[q], p[q], go, n, rem, t, zero);
         if (go) rem -= n;
         return go;
     };
@@ -347,7 +362,7 @@ __device__ __forceinline__ uint32_t select_rank16(uint32_t (&l)[4][4], const int
         const bool p = h[0] <= t;
         const int n = __popc(__ballot_sync(0xffffffffu, p) & gmask);
         go = n < rem;
-        if (p && go) { h[0] = h[1]; h[1] = h[2]; h[2] = h[3]; h[3] = KEY_MAX; }
+        list_drop<G>(h, p, go, n, rem, t, zero);
         if (go) rem -= n;
     };
     head_round();
@@ -452,7 +467,7 @@ __device__ __forceinline__ uint32_t select_cta16(const uint32_t (&key)[EPT16], c
             }
             sort_list4(l[q]);
         }
-        x = select_rank16<32, 2>(l, (int)kk, lane);
+        x = select_rank16<32, 2>(l, (int)kk, lane, 0u);
     }
     return x;
 }
@@ -1242,7 +1257,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
                 cswap(l[q][1], l[q][2]);
             }
             if (!round_m) quant_m_done();
-            x_p = select_rank16<G, G == 16 ? 3 : 2>(l, a.k_full, lane);
+            x_p = select_rank16<G, G == 16 ? 3 : 2>(l, a.k_full, lane, (uint32_t)a.only_partial);
         }
     }
 
