@@ -31,7 +31,7 @@ UNITS = [
     ("solo_step_inst.cu", "solo_step_bm8.o", ["-DSOLO_BM=8"]),
     *[("solo_fast_inst.cu", f"solo_fast_bm{b}_t{t}.o", [f"-DSOLO_BM={b}", f"-DSOLO_TAILS={t}"]) for t in (0, 1) for b in (8, 4, 3, 2)],
     *[("solo_fast16_inst.cu", f"solo_fast16_g{g}_m{m}_w{w}.o", [f"-DSOLO_G={g}", f"-DSOLO_MODES={m}", f"-DSOLO_W8={w}"])
-      for w in (1, 0) for m in (2, 1, 0) for g in (128, 16, 8, 4)],
+      for w in (1, 0) for m in (2, 3, 1, 0, 4) for g in (128, 16, 8, 4)],
 ]
 
 

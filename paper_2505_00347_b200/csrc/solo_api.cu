@@ -240,6 +240,9 @@ int launch_step(solo_state* s, StepArgs& a, int64_t full, cudaStream_t stream) {
     // the eight-per-thread streamlined kernel has neither the baseline second-moment codebooks nor Eq. 5
     const bool streamlined = fast_ok && !a.tables_v && !a.round_m;
     const bool plain = !a.l2 && !a.belief && a.fixed_alpha == 0.0f && a.round_v && !a.tables_v && !a.round_m;
+    // Eq. 5 alone and a baseline codebook alone have instantiations of their own (a codebook has no base and no dither)
+    const bool alone = !a.l2 && !a.belief && (a.tables_v ? !a.round_m : a.fixed_alpha == 0.0f && a.round_v);
+    const int modes = plain ? 0 : !(a.tables_v || a.round_m) ? 1 : !alone ? 2 : a.tables_v ? 4 : 3;
     solo::StepKernel k16 = nullptr;
     const int64_t rest = a.total_tiles - a.tile_first - full;
     const bool all_full = !a.param_list && rest == 0;
@@ -275,8 +278,7 @@ int launch_step(solo_state* s, StepArgs& a, int64_t full, cudaStream_t stream) {
         large = full >= (w8 ? 1664 + 2 * rest : 2048 + 6 * rest);
     }
     if (fast_ok && ((policy == 0 && large) || policy == 3))
-        k16 = solo::fast16_kernel(s->bits_m, s->bits_v, s->block, a.param_bf16 != 0,
-                                  plain ? 0 : (a.tables_v || a.round_m) ? 2 : 1);
+        k16 = solo::fast16_kernel(s->bits_m, s->bits_v, s->block, a.param_bf16 != 0, modes);
     if (k16) {
         // Three tiles per CTA once every resident CTA has some eight shares to take over in turn, fewer below: with
         // 8192 tiles one per CTA 55 us, three 59 us; with 395,000 (LLaMA layers) one 2172 us, three 2110 us, eight 2223 us.

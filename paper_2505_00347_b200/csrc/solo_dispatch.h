@@ -45,8 +45,8 @@ StepKernel fast_kernel(int bits_m, int bits_v, int block, bool param_bf16, bool 
 // The kernel for the tiles that the sixteen-per-thread kernel leaves; it reads the modes at run time.
 StepKernel fast_tails_kernel(int bits_m, int bits_v, int block, bool param_bf16);
 // Sixteen elements per thread: fp32 or bf16 parameters; `modes`: 0 as `plain` for
-// fast_kernel, 1 the modes fast_kernel reads at run time, 2 those plus Eq. 5 rounding and the baseline
-// second-moment codebooks; full tiles
+// fast_kernel, 1 the modes fast_kernel reads at run time, 3 `plain` with Eq. 5 rounding, 4 `plain` with a baseline second-moment
+// codebook (StepArgs::tables_v set), 2 any of these together; full tiles
 // of aligned tensors only (the rest is left to a launch of the streamlined or of the general kernel with
 // StepArgs::only_partial).  Launched with CTA16 = 128 threads.
 // Null / 0 for other block sizes.  One translation unit per block size, set of modes and group of widths.
@@ -55,9 +55,13 @@ constexpr int CTA16 = 128;         // threads per CTA of that kernel
     StepKernel fast16_kernel_g##G##_m0(int bits_m, int bits_v, bool param_bf16);      \
     StepKernel fast16_kernel_g##G##_m1(int bits_m, int bits_v, bool param_bf16);      \
     StepKernel fast16_kernel_g##G##_m2(int bits_m, int bits_v, bool param_bf16);      \
+    StepKernel fast16_kernel_g##G##_m3(int bits_m, int bits_v, bool param_bf16);      \
+    StepKernel fast16_kernel_g##G##_m4(int bits_m, int bits_v, bool param_bf16);      \
     StepKernel fast16_kernel_g##G##_m0_w8(int bits_m, int bits_v, bool param_bf16);   \
     StepKernel fast16_kernel_g##G##_m1_w8(int bits_m, int bits_v, bool param_bf16);   \
     StepKernel fast16_kernel_g##G##_m2_w8(int bits_m, int bits_v, bool param_bf16);   \
+    StepKernel fast16_kernel_g##G##_m3_w8(int bits_m, int bits_v, bool param_bf16);   \
+    StepKernel fast16_kernel_g##G##_m4_w8(int bits_m, int bits_v, bool param_bf16);   \
     size_t fast16_smem_g##G(int bits_m, int bits_v, bool param_bf16);                 \
     size_t fast16_smem_g##G##_w8(int bits_m, int bits_v, bool param_bf16);
 SOLO_DECLARE16(4)

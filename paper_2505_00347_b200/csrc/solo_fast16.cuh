@@ -1,10 +1,11 @@
 // Sixteen elements per thread: the streamlined step for the plain step (2/3/4/8-bit states, blocks of
 // 64, 128, 256 or 2048, fp32 or bf16 parameters; no L2 term in the gradient, no AdaBelief, base from the
-// p-quantile, xi drawn: MODES = 0).  Two more instantiations read other modes from the arguments:
-// MODES = 1 the L2 term, AdaBelief, a fixed base, no dither; MODES = 2 also stochastic rounding of the
-// first moment (Eq. 5) and the baseline second-moment codebooks (a fixed level table instead of the
-// logarithmic levels: no quantile, no draws, nearest level).  (One instantiation for all of them
-// measured 11 % slower on the modes of MODES = 1 than the one that leaves Eq. 5 and the tables out.)
+// p-quantile, xi drawn: MODES = 0).  The other instantiations: MODES = 1 reads the L2 term, AdaBelief, a fixed base and no dither from
+// the arguments; MODES = 3 is the plain step with stochastic rounding of the first moment (Eq. 5), MODES = 4 the plain step
+// with a baseline second-moment codebook (a fixed level table instead of the logarithmic levels: no quantile, no draws, nearest
+// level), both fixed at compile time; MODES = 2 reads all of them, for the combinations.  What an instantiation leaves out costs
+// twice, in branches and in places of the instruction cache: MODES = 1 read as MODES = 2 is 11 % slower, Eq. 5 took 295 us as
+// MODES = 2 and takes 260 (4/2 bit, 2^26 elements; 8/8 bit 388 and 319), dynamic exponent for both moments 219 and 209.
 //
 // Same arithmetic, element for element, as solo_step_fast_kernel (solo_fast.cuh), in packed pairs of
 // binary32 (F2): the kernel is bound by instruction issue and a packed operation gives two results per issue
@@ -58,7 +59,7 @@ static_assert(CTA16 * EPT16 == TILE, "same tile as the other kernels");
 // memory: seven, six where the modes' tables come on top (8/8 bit five 516, six 498, seven 496 us; Eq. 5 four 830, five
 // 799, six 763 us).
 template <int BM, int BV, int G, int MODES>
-constexpr int ctas16() { return BM == 8 || BV == 8 ? (MODES == 2 ? 6 : 7) : BM == 4 || G >= 16 ? 7 : 8; }
+constexpr int ctas16() { return BM == 8 || BV == 8 ? (MODES >= 2 ? 6 : 7) : BM == 4 || G >= 16 ? 7 : 8; }
 
 // G: lanes per block (4, 8, 16 or 128 for blocks of 64, 128, 256 or 2048 elements); NG = 128 / G blocks per tile.
 template <int BM, int BV, bool PBF, int G>
@@ -679,15 +680,15 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     const int gl = tid & (G - 1), grp = tid / G;
     const uint32_t sw = ((uint32_t)tid >> 2) & 1u;               // 1: this thread takes elements 8..15 first (see the top of the file)
     // PLAIN: the step of the paper as it stands (no L2 term in the gradient, no AdaBelief, base from the
-    // p-quantile, xi drawn); the other instantiations read these modes from the arguments, EXT also
-    // Eq. 5 and the baseline codebooks
-    constexpr bool PLAIN = MODES == 0, EXT = MODES == 2;
+    // p-quantile, xi drawn), with Eq. 5 (MODES 3) or a baseline codebook (MODES 4) or without; the other
+    // instantiations read these modes from the arguments, MODES 2 also Eq. 5 and the baseline codebooks
+    constexpr bool PLAIN = MODES == 0 || MODES >= 3;
     const bool l2 = !PLAIN && a.l2, belief = !PLAIN && a.belief;
     // baseline codebook for the second moment: levels s_yv, nearest level by the midpoints in s_nv
-    const bool vtab = EXT && a.tables_v != nullptr;
-    const bool fixed_base = !PLAIN && (a.fixed_alpha > 0.0f || vtab);   // no quantile to find
-    const bool round_v = PLAIN || (a.round_v && !vtab);
-    const bool round_m = EXT && a.round_m;                     // Eq. 5 instead of Eq. 1 for the first moment
+    const bool vtab = MODES == 4 || (MODES == 2 && a.tables_v != nullptr);
+    const bool fixed_base = MODES == 4 || (!PLAIN && (a.fixed_alpha > 0.0f || vtab));   // no quantile to find
+    const bool round_v = MODES != 4 && (PLAIN || (a.round_v && !vtab));
+    const bool round_m = MODES == 3 || (MODES == 2 && a.round_m);   // Eq. 5 instead of Eq. 1 for the first moment
 
     const typename Shared::Desc& desc = s.desc[fill & 1u];
     char* const pt = desc.p;
@@ -1448,16 +1449,16 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
 template <int BM, int BV, bool PBF, int G, int MODES>
 __global__ void __launch_bounds__(CTA16, ctas16<BM, BV, G, MODES>()) solo_step_fast16_kernel(const __grid_constant__ StepArgs a) {
     constexpr int KM = 1 << BM;
-    constexpr bool EXT = MODES == 2;
+    constexpr bool EXT = MODES >= 2, EQ5 = MODES == 2 || MODES == 3;
     using Shared = Fast16Shared<BM, BV, PBF, G>;
     extern __shared__ __align__(16) unsigned char fast16_smem[];
     Shared& s = *reinterpret_cast<Shared*>(fast16_smem);
     __shared__ float s_y[KM];
     __shared__ float s_mid[KM];
-    __shared__ float2 s_yg[EXT ? KM : 1];                    // Eq. 5: see the set-up below
-    __shared__ float4 s_br[EXT ? (BM == 4 ? 5 : 2) : 1];
-    __shared__ float s_yv[EXT && BV != 8 ? 1 << BV : 1];               // baseline second-moment codebook: its levels,
-    __shared__ float4 s_nv[EXT ? 8 : 1];                     // its midpoints times -2^100 (rows as the tile function reads them)
+    __shared__ float2 s_yg[EQ5 ? KM : 1];                    // Eq. 5: see the set-up below
+    __shared__ float4 s_br[EQ5 ? (BM == 4 ? 5 : 2) : 1];
+    __shared__ float s_yv[(MODES == 2 || MODES == 4) && BV != 8 ? 1 << BV : 1];               // baseline second-moment codebook: its levels,
+    __shared__ float4 s_nv[MODES == 2 || MODES == 4 ? 8 : 1];                     // its midpoints times -2^100 (rows as the tile function reads them)
     __shared__ float4 s_mid4[4];             // 4-bit first moments: per quarter of the codebook, its three inner midpoints times -2^100
     const int tid = threadIdx.x;
     pdl_wait();
@@ -1467,14 +1468,14 @@ __global__ void __launch_bounds__(CTA16, ctas16<BM, BV, G, MODES>()) solo_step_f
         s_mid[i] = i < KM - 1 ? a.tables[KM + i] : __int_as_float(0x7f800000);
     }
     if constexpr (BM == 8) {
-        const uint4* const src = reinterpret_cast<const uint4*>(g_lut8_m[EXT && a.round_m ? 1 : 0].q);
+        const uint4* const src = reinterpret_cast<const uint4*>(g_lut8_m[MODES == 3 || (MODES == 2 && a.round_m) ? 1 : 0].q);
         for (int i = tid; i < LUT8_M_BYTES / 16; i += CTA16) reinterpret_cast<uint4*>(s.lut_m)[i] = src[i];
     }
     if (BM == 4 && tid < 4)
         s_mid4[tid] = make_float4(-a.tables[KM + 4 * tid] * 0x1p100f, -a.tables[KM + 4 * tid + 1] * 0x1p100f,
                                   -a.tables[KM + 4 * tid + 2] * 0x1p100f, 0.0f);
     if constexpr (EXT) {
-        if (a.round_m) {
+        if (MODES == 3 || (MODES == 2 && a.round_m)) {
             // Eq. 5: per level q <= K-2 the pair (y_q, 1 / (y_{q+1} - y_q)); thresholds of "r >= y_j" as
             // -y'_j * 2^100, y'_j the binary32 just below y_j (rows as the tile function reads them:
             // 2- and 3-bit, levels 1..6 in rows 0, 1; 4-bit, row s = levels 4s+1..4s+3 and row 4 = levels
@@ -1507,7 +1508,7 @@ __global__ void __launch_bounds__(CTA16, ctas16<BM, BV, G, MODES>()) solo_step_f
             }
             if (BM == 4 && tid == 4) s_br[4] = make_float4(below(4), below(8), below(12), 0.0f);
         }
-        if (a.tables_v != nullptr) {
+        if (MODES == 4 || (MODES == 2 && a.tables_v != nullptr)) {
             constexpr int KV = 1 << BV;
             const float* const midv = a.tables_v + KV;            // KV - 1 midpoints
             if constexpr (BV == 8) {

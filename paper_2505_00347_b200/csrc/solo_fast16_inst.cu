@@ -1,6 +1,6 @@
 // The sixteen-elements-per-thread kernels for one block size (SOLO_G = 4, 8, 16, 128 lanes per
-// block: blocks of 64, 128, 256, 2048 elements) and one set of modes (SOLO_MODES = 0: the paper's plain step, fixed
-// at compile time; 1, 2: read from the arguments, see solo_fast16.cuh): fp32 or bf16 parameters, 2/3/4-bit states
+// block: blocks of 64, 128, 256, 2048 elements) and one set of modes (SOLO_MODES = 0: the paper's plain step, 3 with
+// Eq. 5, 4 with a baseline codebook, fixed at compile time; 1, 2: read from the arguments, see solo_fast16.cuh): fp32 or bf16 parameters, 2/3/4-bit states
 // (SOLO_W8 = 0) or an 8-bit state and any other (SOLO_W8 = 1).
 #include "solo_dispatch.h"
 #include "solo_fast16.cuh"
@@ -9,7 +9,7 @@
 #error "compile with -DSOLO_G=4|8|16|128"
 #endif
 #ifndef SOLO_MODES
-#error "compile with -DSOLO_MODES=0|1|2"
+#error "compile with -DSOLO_MODES=0|1|2|3|4"
 #endif
 
 #ifndef SOLO_W8
