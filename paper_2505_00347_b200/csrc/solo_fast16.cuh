@@ -61,6 +61,43 @@ static_assert(CTA16 * EPT16 == TILE, "same tile as the other kernels");
 template <int BM, int BV, int G, int MODES>
 constexpr int ctas16() { return BM == 8 || BV == 8 ? (MODES >= 2 ? 6 : 7) : BM == 4 || G >= 16 ? 7 : 8; }
 
+// What the first rounds of Philox4x32-10 leave of the counter's words that are the same for a whole tile: (position, high word,
+// step, 4 * stream) differ in the position's low word only, which reaches half of the second round and all of the third.
+// Computed per tensor by the thread that walks (draw_keys): a call is 16 wide multiplications instead of 20, and no thread looks up its
+// tensor's stream (2^26 elements: 2/3 bit 183.5 -> 181.7 us, bf16 parameters stochastically rounded 240 -> 236).
+struct DrawKeys {
+    uint32_t k2, k3, k4, k6;
+};
+__device__ __forceinline__ DrawKeys draw_keys(const uint32_t (&rk)[20], uint32_t ctr_hi, uint32_t step, uint32_t stream4) {
+    const uint64_t p1 = (uint64_t)0xCD9E8D57u * step;
+    const uint64_t p0 = (uint64_t)0xD2511F53u * ((uint32_t)(p1 >> 32) ^ ctr_hi ^ rk[0]);
+    return {stream4 ^ rk[1], (uint32_t)p1 ^ rk[2], (uint32_t)(p0 >> 32) ^ rk[3], (uint32_t)p0 ^ rk[5]};
+}
+// philox_rk(c0, ctr_hi, step, stream4 + purpose, rk, out)
+__device__ __forceinline__ void philox_keys(uint32_t c0, const DrawKeys& k, uint32_t purpose, const uint32_t (&rk)[20], uint32_t (&out)[4]) {
+    constexpr uint64_t M0 = 0xD2511F53u, M1 = 0xCD9E8D57u;
+    uint64_t p0 = M0 * c0;
+    uint64_t p1 = M1 * ((uint32_t)(p0 >> 32) ^ k.k2 ^ purpose);
+    c0 = (uint32_t)(p1 >> 32) ^ k.k3;
+    uint32_t c1 = (uint32_t)p1, c2 = (uint32_t)p0 ^ k.k4;
+    p0 = M0 * c0;
+    p1 = M1 * c2;
+    c0 = (uint32_t)(p1 >> 32) ^ c1 ^ rk[4];
+    c2 = (uint32_t)(p0 >> 32) ^ k.k6;
+    c1 = (uint32_t)p1;
+    uint32_t c3 = (uint32_t)p0;
+#pragma unroll
+    for (int r = 3; r < 10; ++r) {
+        p0 = M0 * c0;
+        p1 = M1 * c2;
+        c0 = (uint32_t)(p1 >> 32) ^ c1 ^ rk[2 * r];
+        c2 = (uint32_t)(p0 >> 32) ^ c3 ^ rk[2 * r + 1];
+        c1 = (uint32_t)p1;
+        c3 = (uint32_t)p0;
+    }
+    out[0] = c0; out[1] = c1; out[2] = c2; out[3] = c3;
+}
+
 // G: lanes per block (4, 8, 16 or 128 for blocks of 64, 128, 256 or 2048 elements); NG = 128 / G blocks per tile.
 template <int BM, int BV, bool PBF, int G>
 struct Fast16Shared {
@@ -123,6 +160,9 @@ struct Fast16Shared {
         char* p;                             // tensor: its parameters, gradients, first block
         const char* g;
         int64_t jb0;
+        uint64_t ctr0;                       // its place in the random stream
+        uint32_t stream4, ctr_hi;
+        alignas(16) DrawKeys keys[2];        // for the high word of ctr0, and for the one after
         int tensor, t_lo, t_hi, full_tiles;  // tensor: tiles [t_lo, t_hi), the first full_tiles of them full
         int tile, tile_end;                  // last tile handed out; end of the tiles taken
         uint32_t phase;                      // parity of mbar_steal's next phase
@@ -133,9 +173,11 @@ struct Fast16Shared {
         char* p;                             // the tile's parameters, gradients, first block
         const char* g;
         int64_t jb;
-        int tensor, tin, tile, valid;        // valid 0: no tile left
+        int tile, valid;                     // valid 0: no tile left
+        uint32_t ctr;                        // low word of the stream position of its first element (element index / 8)
+        alignas(16) DrawKeys keys[2];        // [1]: of the elements behind a change of the high word
     };
-    alignas(8) Desc desc[2];                 // written for the next tile between the two barriers of this one
+    alignas(16) Desc desc[2];                 // written for the next tile between the two barriers of this one
 };
 
 __device__ __forceinline__ void bar_sync16(int id) {
@@ -582,7 +624,8 @@ __device__ __forceinline__ int steal_answer(Shared& s, int* status) {
 // A CTA that waited in vain for a copy ends here: it takes in the answer to its last request, so that nothing writes to its
 // shared memory any more, and asks for no other.  What it then leaves unstepped (and has reported in the status word) is
 // the rest of its share and at most the one that answer brought, however many CTAs have not started yet.
-template <int BM, int BV, bool PBF, int G>
+// DRAWS: the step draws random numbers, so that the tile's Philox keys are wanted.
+template <int BM, int BV, bool PBF, int G, bool DRAWS>
 __device__ __forceinline__ void produce_tile16(const StepArgs& a, Fast16Shared<BM, BV, PBF, G>& s, typename Fast16Shared<BM, BV, PBF, G>::Desc& d) {
     constexpr int NG = CTA16 / G, PSZ = PBF ? 2 : 4;
     typename Fast16Shared<BM, BV, PBF, G>::Walk& w = s.walk;
@@ -621,6 +664,14 @@ __device__ __forceinline__ void produce_tile16(const StepArgs& a, Fast16Shared<B
             w.jb0 = __ldg(a.block_start + tensor);
             w.p = pb;
             w.g = gb;
+            if constexpr (DRAWS) {
+                const Origin org = origin_of(a, tensor);
+                w.ctr0 = org.ctr0;
+                w.stream4 = org.stream * 4u;
+                w.ctr_hi = (uint32_t)(org.ctr0 >> 32);
+                w.keys[0] = draw_keys(a.rk, w.ctr_hi, a.step32, w.stream4);
+                w.keys[1] = draw_keys(a.rk, w.ctr_hi + 1u, a.step32, w.stream4);
+            }
         }
         if (tile - w.t_lo < w.full_tiles) break;
         tile = min(w.t_hi, tile_end) - 1;                                // the rest of the tensor is left to the other launch
@@ -630,8 +681,17 @@ __device__ __forceinline__ void produce_tile16(const StepArgs& a, Fast16Shared<B
     d.p = w.p + (int64_t)tin * (TILE * PSZ);
     d.g = w.g + (int64_t)tin * (TILE * 2);
     d.jb = w.jb0 + (int64_t)tin * NG;
-    d.tensor = w.tensor;
-    d.tin = tin;
+    if constexpr (DRAWS) {
+        const uint64_t ctr = w.ctr0 + (uint64_t)(uint32_t)tin * (TILE / 8);
+        d.ctr = (uint32_t)ctr;
+        if ((uint32_t)(ctr >> 32) != w.ctr_hi) {
+            w.ctr_hi = (uint32_t)(ctr >> 32);
+            w.keys[0] = draw_keys(a.rk, w.ctr_hi, a.step32, w.stream4);
+            w.keys[1] = draw_keys(a.rk, w.ctr_hi + 1u, a.step32, w.stream4);
+        }
+        d.keys[0] = w.keys[0];
+        d.keys[1] = w.keys[1];
+    }
     d.tile = tile;
     d.valid = 1;
     issue_tile_copy16<BM, BV, PBF, G>(a, s, d.p, d.g, d.jb, tile + 1 == a.debug_stall_tile_p1 ? 16u : 0u);
@@ -710,7 +770,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     if (G != 128 && gave_up) {
         if (gl == 0) s.xin[grp] = make_uint4(0u, 0u, 0u, 1u);
         bar_sync16(1);
-        if (tid == 32) produce_tile16<BM, BV, PBF, G>(a, s, s.desc[(fill + 1u) & 1u]);
+        if (tid == 32) produce_tile16<BM, BV, PBF, G, MODES != 4 || PBF>(a, s, s.desc[(fill + 1u) & 1u]);
         if (tid < NG) block_scalars16<KV>(a, s, jb_tile, tid, fixed_base, vtab);
         bar_sync16(2);
         return;
@@ -882,7 +942,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
         const uint4 m4 = *reinterpret_cast<const uint4*>(c.m), v4 = *reinterpret_cast<const uint4*>(c.v);
         const uint4 l4 = *reinterpret_cast<const uint4*>(c.lo), f4 = *reinterpret_cast<const uint4*>(c.failed);
         if (f4.x | f4.y | f4.z | f4.w) {
-            if (tid == 32) produce_tile16<BM, BV, PBF, G>(a, s, s.desc[(fill + 1u) & 1u]);
+            if (tid == 32) produce_tile16<BM, BV, PBF, G, MODES != 4 || PBF>(a, s, s.desc[(fill + 1u) & 1u]);
             bar_sync16(2);
             return;
         }
@@ -894,14 +954,12 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     // ---- (B) Adam(W) update, four (fp32) or eight (bf16) elements at a time ----
     // bf16 parameters: correctly rounded square root and division (see solo_fast.cuh), rounded to nearest even or
     // with the element's Philox draw (purpose 2, one block per eight elements)
-    // position of the thread's first element in the tensor's random stream (element index / 8): even,
-    // so the second group of eight never carries into the high word
-    auto stream_position = [&](uint32_t& lo, uint32_t& hi, uint32_t& c3) {
-        const Origin org = origin_of(a, desc.tensor);
-        const uint64_t ctr = org.ctr0 + (uint64_t)((uint32_t)desc.tin * (TILE / 8) + 2u * (uint32_t)tid);
-        lo = (uint32_t)ctr;
-        hi = (uint32_t)(ctr >> 32);
-        c3 = org.stream * 4u;
+    // The draws of the thread's eight elements `half` (0: the first in its own order).  Positions in the stream count eights of
+    // elements; a tensor starts at a multiple of eight of them, so that the thread's two share the high word.
+    auto draw8 = [&](uint32_t half, uint32_t purpose, uint32_t (&out)[4]) {
+        const uint32_t c0 = desc.ctr + 2u * (uint32_t)tid;
+        const DrawKeys k = desc.keys[c0 < desc.ctr ? 1 : 0];
+        philox_keys(c0 + half, k, purpose, a.rk, out);
     };
     if constexpr (!PBF) {
         // the thread's first eight elements (in its own order) at `sp[0]`, the others at `sp[1]`
@@ -953,9 +1011,8 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
             const uint32_t he = (uint32_t)h ^ sw;
             uint32_t pp[4];
             if (a.param_sr) {
-                uint32_t wp[4], ctr_lo, ctr_hi, c3;
-                stream_position(ctr_lo, ctr_hi, c3);
-                philox_rk(ctr_lo + he, ctr_hi, a.step32, c3 + 2u, a.rk, wp);
+                uint32_t wp[4];
+                draw8(he, 2u, wp);
 #pragma unroll
                 for (int k = 0; k < 4; ++k)
                     pp[k] = bf16_sr(p[2 * k], wp[k] & 0xFFFFu) | (bf16_sr(p[2 * k + 1], wp[k] >> 16) << 16);
@@ -1122,13 +1179,11 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
         // operation exists (4/2 bit, 2^27 elements: 601 -> 582 us).
         uint32_t wm[8];
         {
-            uint32_t ctr_lo, ctr_hi, c3;
-            stream_position(ctr_lo, ctr_hi, c3);
             uint32_t w4[4];
-            philox_rk(ctr_lo + sw, ctr_hi, a.step32, c3 + 1u, a.rk, w4);
+            draw8(sw, 1u, w4);
 #pragma unroll
             for (int i = 0; i < 4; ++i) wm[i] = w4[i];
-            philox_rk(ctr_lo + (sw ^ 1u), ctr_hi, a.step32, c3 + 1u, a.rk, w4);
+            draw8(sw ^ 1u, 1u, w4);
 #pragma unroll
             for (int i = 0; i < 4; ++i) wm[4 + i] = w4[i];
         }
@@ -1273,12 +1328,11 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     // ---- (E) per-block scalars by the first warp; the next tile's copies start meanwhile ----
     auto draw = [&]() {
         if (round_v) {
-            uint32_t ctr_lo, ctr_hi, c3, w4[4];
-            stream_position(ctr_lo, ctr_hi, c3);
-            philox_rk(ctr_lo + sw, ctr_hi, a.step32, c3, a.rk, w4);
+            uint32_t w4[4];
+            draw8(sw, 0u, w4);
 #pragma unroll
             for (int i = 0; i < 4; ++i) w[i] = w4[i];
-            philox_rk(ctr_lo + (sw ^ 1u), ctr_hi, a.step32, c3, a.rk, w4);
+            draw8(sw ^ 1u, 0u, w4);
 #pragma unroll
             for (int i = 0; i < 4; ++i) w[4 + i] = w4[i];
         }
@@ -1288,7 +1342,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     if (gl == 0) s.xin[grp] = make_uint4(mx_m, mx_v, x_p, 0u);
     bar_sync16(1);
     // every thread has read what it needs from the stage
-    if (tid == 32) produce_tile16<BM, BV, PBF, G>(a, s, s.desc[(fill + 1u) & 1u]);
+    if (tid == 32) produce_tile16<BM, BV, PBF, G, MODES != 4 || PBF>(a, s, s.desc[(fill + 1u) & 1u]);
     if (tid < NG) block_scalars16<KV>(a, s, jb_tile, tid, fixed_base, vtab);
     // meanwhile every thread draws: Philox4x32-10 on the counters of its two groups of eight elements,
     // (ctr, step, 4 * stream) and (ctr + 1, ...), in its own order.  (Between the selection's rounds, where the draws
@@ -1556,7 +1610,7 @@ __global__ void __launch_bounds__(CTA16, ctas16<BM, BV, G, MODES>()) solo_step_f
         s.walk.tile_end = (int)min((int64_t)s.walk.tile + 1 + a.share, a.total_tiles);
         s.walk.tensor = (a.num_tensors > 1 ? find_tensor(a.tile_start, a.num_tensors, s.walk.tile + 1) : 0) - 1;
         steal_request(s);
-        produce_tile16<BM, BV, PBF, G>(a, s, s.desc[0]);
+        produce_tile16<BM, BV, PBF, G, MODES != 4 || PBF>(a, s, s.desc[0]);
     }
     __syncthreads();
 
