@@ -156,13 +156,16 @@ struct Fast16Shared {
     // The CTA's walk over the tiles (see produce_tile16): kept here and not in registers, because one thread uses it
     alignas(8) unsigned long long mbar_steal;
     alignas(16) uint4 steal;                 // answer of the last request for another CTA's tiles
+    // Blocks of 64 draw from the counters as they are: the keys gain nothing there (2^24 elements, fp32: 1.00) and cost the modes that
+    // are read from the arguments 2 to 3 %.
+    static constexpr bool KEYS = G != 4;
     struct Walk {
         char* p;                             // tensor: its parameters, gradients, first block
         const char* g;
         int64_t jb0;
         uint64_t ctr0;                       // its place in the random stream
         uint32_t stream4, ctr_hi;
-        alignas(16) DrawKeys keys[2];        // for the high word of ctr0, and for the one after
+        alignas(16) DrawKeys keys[KEYS ? 2 : 1];     // for the high word of ctr0, and for the one after
         int tensor, t_lo, t_hi, full_tiles;  // tensor: tiles [t_lo, t_hi), the first full_tiles of them full
         int tile, tile_end;                  // last tile handed out; end of the tiles taken
         uint32_t phase;                      // parity of mbar_steal's next phase
@@ -174,8 +177,9 @@ struct Fast16Shared {
         const char* g;
         int64_t jb;
         int tile, valid;                     // valid 0: no tile left
-        uint32_t ctr;                        // low word of the stream position of its first element (element index / 8)
-        alignas(16) DrawKeys keys[2];        // [1]: of the elements behind a change of the high word
+        uint32_t ctr, ctr_hi;                // stream position of its first element (element index / 8)
+        uint32_t stream4;
+        alignas(16) DrawKeys keys[KEYS ? 2 : 1];     // [1]: of the elements behind a change of the high word
     };
     alignas(16) Desc desc[2];                 // written for the next tile between the two barriers of this one
 };
@@ -627,6 +631,7 @@ __device__ __forceinline__ int steal_answer(Shared& s, int* status) {
 // DRAWS: the step draws random numbers, so that the tile's Philox keys are wanted.
 template <int BM, int BV, bool PBF, int G, bool DRAWS>
 __device__ __forceinline__ void produce_tile16(const StepArgs& a, Fast16Shared<BM, BV, PBF, G>& s, typename Fast16Shared<BM, BV, PBF, G>::Desc& d) {
+    using Shared = Fast16Shared<BM, BV, PBF, G>;
     constexpr int NG = CTA16 / G, PSZ = PBF ? 2 : 4;
     typename Fast16Shared<BM, BV, PBF, G>::Walk& w = s.walk;
     int tile_end = w.tile_end, tile = w.gave_up ? tile_end : w.tile;
@@ -669,8 +674,10 @@ __device__ __forceinline__ void produce_tile16(const StepArgs& a, Fast16Shared<B
                 w.ctr0 = org.ctr0;
                 w.stream4 = org.stream * 4u;
                 w.ctr_hi = (uint32_t)(org.ctr0 >> 32);
-                w.keys[0] = draw_keys(a.rk, w.ctr_hi, a.step32, w.stream4);
-                w.keys[1] = draw_keys(a.rk, w.ctr_hi + 1u, a.step32, w.stream4);
+                if constexpr (Shared::KEYS) {
+                    w.keys[0] = draw_keys(a.rk, w.ctr_hi, a.step32, w.stream4);
+                    w.keys[1] = draw_keys(a.rk, w.ctr_hi + 1u, a.step32, w.stream4);
+                }
             }
         }
         if (tile - w.t_lo < w.full_tiles) break;
@@ -684,13 +691,18 @@ __device__ __forceinline__ void produce_tile16(const StepArgs& a, Fast16Shared<B
     if constexpr (DRAWS) {
         const uint64_t ctr = w.ctr0 + (uint64_t)(uint32_t)tin * (TILE / 8);
         d.ctr = (uint32_t)ctr;
-        if ((uint32_t)(ctr >> 32) != w.ctr_hi) {
-            w.ctr_hi = (uint32_t)(ctr >> 32);
-            w.keys[0] = draw_keys(a.rk, w.ctr_hi, a.step32, w.stream4);
-            w.keys[1] = draw_keys(a.rk, w.ctr_hi + 1u, a.step32, w.stream4);
+        if constexpr (Shared::KEYS) {
+            if ((uint32_t)(ctr >> 32) != w.ctr_hi) {
+                w.ctr_hi = (uint32_t)(ctr >> 32);
+                w.keys[0] = draw_keys(a.rk, w.ctr_hi, a.step32, w.stream4);
+                w.keys[1] = draw_keys(a.rk, w.ctr_hi + 1u, a.step32, w.stream4);
+            }
+            d.keys[0] = w.keys[0];
+            d.keys[1] = w.keys[1];
+        } else {
+            d.ctr_hi = (uint32_t)(ctr >> 32);
+            d.stream4 = w.stream4;
         }
-        d.keys[0] = w.keys[0];
-        d.keys[1] = w.keys[1];
     }
     d.tile = tile;
     d.valid = 1;
@@ -743,6 +755,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     // p-quantile, xi drawn), with Eq. 5 (MODES 3) or a baseline codebook (MODES 4) or without; the other
     // instantiations read these modes from the arguments, MODES 2 also Eq. 5 and the baseline codebooks
     constexpr bool PLAIN = MODES == 0 || MODES >= 3;
+    constexpr bool BRACKET = (MODES == 0 || MODES == 3) && (G == 8 || G == 128);    // see the update of bf16 parameters
     const bool l2 = !PLAIN && a.l2, belief = !PLAIN && a.belief;
     // baseline codebook for the second moment: levels s_yv, nearest level by the midpoints in s_nv
     const bool vtab = MODES == 4 || (MODES == 2 && a.tables_v != nullptr);
@@ -958,8 +971,12 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     // elements; a tensor starts at a multiple of eight of them, so that the thread's two share the high word.
     auto draw8 = [&](uint32_t half, uint32_t purpose, uint32_t (&out)[4]) {
         const uint32_t c0 = desc.ctr + 2u * (uint32_t)tid;
-        const DrawKeys k = desc.keys[c0 < desc.ctr ? 1 : 0];
-        philox_keys(c0 + half, k, purpose, a.rk, out);
+        if constexpr (Shared::KEYS) {
+            const DrawKeys k = desc.keys[c0 < desc.ctr ? 1 : 0];
+            philox_keys(c0 + half, k, purpose, a.rk, out);
+        } else {
+            philox_rk(c0 + half, desc.ctr_hi + (c0 < desc.ctr ? 1u : 0u), a.step32, desc.stream4 + purpose, a.rk, out);
+        }
     };
     if constexpr (!PBF) {
         // the thread's first eight elements (in its own order) at `sp[0]`, the others at `sp[1]`
@@ -988,83 +1005,151 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
         }
     } else {
         const uint4* const sp = reinterpret_cast<const uint4*>(st.p) + 2 * tid;
-        // The exact pairwise sequence where its scaling holds: v^ < 2^27, |m^| < 2^20 (a NaN compares false), usual
-        // hyper-parameters (this kernel runs with eps >= 1e-12 > 2^-40 only); the IEEE operations otherwise.  A quotient
-        // below 2^-126 is not rounded to the subnormal grid before it is multiplied, which shows in results below
-        // 2^-99 |step_size| <= 2^-80 only (in others it is lost against the parameter): a warp that gets one takes the IEEE
-        // operations instead, the parameters being in the stage still.  Two looks: exponent bit 6 is set in all results
-        // from 2^-63 to 2 (one operation per four of them), whatever lacks it is compared.  The two passes one after the other,
-        // and not two sides of a branch per half: LLaMA layer, 2/2 bit, 757 -> 716 us (one loop around both 747, and 2/2 bit with Eq. 5
-        // spilled: 659 -> 723 us on 2^27 elements, as it is 646).
-        bool exact = __all_sync(0xffffffffu, tmx_v < 0x4D000000u && mx_m_f < 0x1p20f && a.eps < 0x1p30f && a.inv_sqrt_bc2 < 0x1p30f &&
-                                                 fabsf(a.step_size) > 0x1p-40f && fabsf(a.step_size) < 0x1p19f);
-        auto load8 = [&](int h, float (&p)[8]) {
-            const uint4 pw = sp[(uint32_t)h ^ sw];
-            const uint32_t pin[4] = {pw.x, pw.y, pw.z, pw.w};
+        // An update by approximations is within 3.8 * 2^-23 of the IEEE operations' (the square root 2^-23, five roundings, a
+        // subnormal v^ that is taken as zero 2^-25).  Made smaller and larger by 5 * 2^-23 and rounded to bf16, both results are
+        // the same pattern but for one element in 65536 or fewer, whose result lies next to a rounding boundary; and then the IEEE
+        // update's too, every operation on the way being monotone.  A warp with an element of the other kind, and values or
+        // hyper-parameters out of these ranges, go the long way below.  (LLaMA layer, 2/2 bit: the long way for all 689 us, this 624.)
+        // Where updates are as large as the parameters one warp in ten has such an element.  Rounding to nearest, which costs less to
+        // begin with, then loses (3/3 bit, mixed gradients: up to 17 %), and so does a codebook that decodes small moments as zero:
+        // stochastic rounding with the logarithmic levels only.  Of blocks of 128 and 2048: where it is not taken its registers cost
+        // something all the same, rounded to nearest 2 to 8 % with blocks of 64, 1 to 4 % with 256, at most 1.5 % with 128.
+        // A quotient below 2^-126 is rounded otherwise than in the IEEE update, which shows in results below 2^-99 |step_size| <=
+        // 2^-80 only (in others it is lost against the parameter).
+        bool done = false;
+        if (BRACKET && a.param_sr) {
+            bool usual = tmx_v < 0x4D000000u && mx_m_f < 0x1p20f && a.eps < 0x1p30f && a.inv_sqrt_bc2 < 0x1p30f &&
+                         (a.step_size == 0.0f || fabsf(a.step_size) > 0x1p-100f) && fabsf(a.step_size) < 0x1p19f;
+            if (a.eps < a.inv_sqrt_bc2 * 0x1p-38f) {                  // (a subnormal v^ would show)
+                uint32_t least = 0xFFFFFFFFu;
 #pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                p[2 * k] = __uint_as_float(pin[k] << 16);
-                p[2 * k + 1] = __uint_as_float(pin[k] & 0xffff0000u);
+                for (int i = 0; i < EPT16; ++i) least = min(least, __float_as_uint(vh_at(i)) - 1u);
+                usual = usual && least >= 0x007FFFFFu;
             }
-        };
-        auto store8 = [&](int h, const float (&p)[8]) {             // returns the conjunction of the patterns
-            const uint32_t he = (uint32_t)h ^ sw;
-            uint32_t pp[4];
-            if (a.param_sr) {
-                uint32_t wp[4];
-                draw8(he, 2u, wp);
+            if (__all_sync(0xffffffffu, usual)) {
+                const F2 isb = F2::dup(a.inv_sqrt_bc2), eps = F2::dup(a.eps), decay = F2::dup(a.decay);
+                const F2 lr_lo = F2::dup(a.step_size * (1.0f - 0x1.4p-21f)), lr_hi = F2::dup(a.step_size * (1.0f + 0x1.4p-21f));
+                uint32_t differ = 0u, all = 0xFFFFFFFFu, some = 0u;
 #pragma unroll
-                for (int k = 0; k < 4; ++k)
-                    pp[k] = bf16_sr(p[2 * k], wp[k] & 0xFFFFu) | (bf16_sr(p[2 * k + 1], wp[k] >> 16) << 16);
-            } else {
+                for (int h = 0; h < 2; ++h) {
+                    const uint32_t he = (uint32_t)h ^ sw;
+                    const uint4 pw = sp[he];
+                    const uint32_t pin[4] = {pw.x, pw.y, pw.z, pw.w};
+                    uint32_t wp[4], pp[4];
+                    draw8(he, 2u, wp);
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const __nv_bfloat162 h2 = __floats2bfloat162_rn(p[2 * k], p[2 * k + 1]);
-                    pp[k] = *reinterpret_cast<const uint32_t*>(&h2);
+                    for (int k = 0; k < 4; ++k) {
+                        const F2 m = mh[4 * h + k], v = vh[4 * h + k];
+                        const F2 den = fma2(F2::pack(sqrt_approx(v.lo()), sqrt_approx(v.hi())), isb, eps);
+                        const F2 nrc = F2::pack(rcp_approx(-den.lo()), rcp_approx(-den.hi()));
+                        const F2 nq0 = mul2(m, nrc);
+                        const F2 nq1 = fma2(fma2(den, nq0, m), nrc, nq0);
+                        F2 pd = F2::pack(__uint_as_float(pin[k] << 16), __uint_as_float(pin[k] & 0xffff0000u));
+                        if (DECAY) pd = mul2(pd, decay);
+                        const F2 r1 = fma2(lr_lo, nq1, pd), r2 = fma2(lr_hi, nq1, pd);
+                        // (bf16_sr of what is no NaN)
+                        const uint32_t dl = wp[k] & 0xFFFFu, dh = wp[k] >> 16;
+                        pp[k] = __byte_perm(__float_as_uint(r1.lo()) + dl, __float_as_uint(r1.hi()) + dh, 0x7632u);
+                        const uint32_t o2 = __byte_perm(__float_as_uint(r2.lo()) + dl, __float_as_uint(r2.hi()) + dh, 0x7632u);
+                        differ |= pp[k] ^ o2;
+                    }
+                    all &= (pp[0] & pp[1]) & (pp[2] & pp[3]);
+                    some |= (pin[0] | pin[1]) | (pin[2] | pin[3]);
+                    __stcs(reinterpret_cast<uint4*>(pt) + 2 * tid + he, make_uint4(pp[0], pp[1], pp[2], pp[3]));
                 }
-            }
-            __stcs(reinterpret_cast<uint4*>(pt) + 2 * tid + he, make_uint4(pp[0], pp[1], pp[2], pp[3]));
-            return (pp[0] & pp[1]) & (pp[2] & pp[3]);
-        };
-        if (exact) {
-            uint32_t all = 0xFFFFFFFFu;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                float p[8];
-                load8(h, p);
-                const F2 nisb = F2::dup(-a.inv_sqrt_bc2 * 0x1p-50f), eps = F2::dup(a.eps), lr = F2::dup(a.step_size * 0x1p-64f);
-#pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    const int j = 4 * h + k;
-                    const F2 den = fma2(neg_sqrt2(mul2(vh[j], F2::dup(-0x1p100f))), nisb, eps);
-                    const F2 nq = neg_div2(mul2(mh[j], F2::dup(0x1p64f)), den);
-                    F2 pj = F2::pack(p[2 * k], p[2 * k + 1]);
-                    pj = fma2(lr, nq, DECAY ? mul2(pj, F2::dup(a.decay)) : pj);
-                    p[2 * k] = pj.lo();
-                    p[2 * k + 1] = pj.hi();
-                }
-                all &= store8(h, p);
-            }
-            if (__any_sync(0xffffffffu, (~all & 0x20002000u) != 0u)) {
-                uint32_t least = 0x7FFFu;                         // of the patterns stored, signs off
+                // Results below 2^-63 (exponent bit 6 is set from there to 2) and parameters from 2 up are looked at more closely: the
+                // former for subnormal quotients, the latter for NaN, which the short form of the stochastic rounding does not know.
+                done = !__any_sync(0xffffffffu, differ != 0u || (~all & 0x20002000u) != 0u || (some & 0x40004000u) != 0u);
+                if (!done) {
+                    bool redo = differ != 0u;
 #pragma unroll 1
-                for (int i = 0; i < EPT16; ++i)
-                    least = min(least, reinterpret_cast<const unsigned short*>(pt)[EPT16 * tid + i] & 0x7FFFu);
-                exact = !__any_sync(0xffffffffu, least < 0x1800u);        // 2^-79: no result below 2^-80 was rounded up to it
+                    for (int i = 0; i < EPT16; ++i) {
+                        redo |= (reinterpret_cast<const unsigned short*>(pt)[EPT16 * tid + i] & 0x7FFFu) < 0x1800u;
+                        redo |= (reinterpret_cast<const unsigned short*>(st.p)[EPT16 * tid + i] & 0x7FFFu) > 0x7F80u;
+                    }
+                    done = !__any_sync(0xffffffffu, redo);
+                }
             }
         }
-        if (!exact) {
+        if (!done) {
+            // The exact pairwise sequence where its scaling holds: v^ < 2^27, |m^| < 2^20 (a NaN compares false), usual
+            // hyper-parameters (this kernel runs with eps >= 1e-12 > 2^-40 only); the IEEE operations otherwise.  A quotient
+            // below 2^-126 is not rounded to the subnormal grid before it is multiplied, which shows in results below
+            // 2^-99 |step_size| <= 2^-80 only (in others it is lost against the parameter): a warp that gets one takes the IEEE
+            // operations instead, the parameters being in the stage still.  Two looks: exponent bit 6 is set in all results
+            // from 2^-63 to 2 (one operation per four of them), whatever lacks it is compared.  The two passes one after the other,
+            // and not two sides of a branch per half: LLaMA layer, 2/2 bit, 757 -> 716 us (one loop around both 747, and 2/2 bit with Eq. 5
+            // spilled: 659 -> 723 us on 2^27 elements, as it is 646).
+            bool exact = __all_sync(0xffffffffu, tmx_v < 0x4D000000u && mx_m_f < 0x1p20f && a.eps < 0x1p30f && a.inv_sqrt_bc2 < 0x1p30f &&
+                                                     fabsf(a.step_size) > 0x1p-40f && fabsf(a.step_size) < 0x1p19f);
+            auto load8 = [&](int h, float (&p)[8]) {
+                const uint4 pw = sp[(uint32_t)h ^ sw];
+                const uint32_t pin[4] = {pw.x, pw.y, pw.z, pw.w};
 #pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                float p[8];
-                load8(h, p);
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    const int i = 8 * h + k;
-                    const float den = __fmaf_rn(__fsqrt_rn(vh_at(i)), a.inv_sqrt_bc2, a.eps);
-                    p[k] = __fmaf_rn(-a.step_size, __fdiv_rn(mh_at(i), den), DECAY ? p[k] * a.decay : p[k]);
+                for (int k = 0; k < 4; ++k) {
+                    p[2 * k] = __uint_as_float(pin[k] << 16);
+                    p[2 * k + 1] = __uint_as_float(pin[k] & 0xffff0000u);
                 }
-                store8(h, p);
+            };
+            auto store8 = [&](int h, const float (&p)[8]) {             // returns the conjunction of the patterns
+                const uint32_t he = (uint32_t)h ^ sw;
+                uint32_t pp[4];
+                if (a.param_sr) {
+                    uint32_t wp[4];
+                    draw8(he, 2u, wp);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        pp[k] = bf16_sr(p[2 * k], wp[k] & 0xFFFFu) | (bf16_sr(p[2 * k + 1], wp[k] >> 16) << 16);
+                } else {
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const __nv_bfloat162 h2 = __floats2bfloat162_rn(p[2 * k], p[2 * k + 1]);
+                        pp[k] = *reinterpret_cast<const uint32_t*>(&h2);
+                    }
+                }
+                __stcs(reinterpret_cast<uint4*>(pt) + 2 * tid + he, make_uint4(pp[0], pp[1], pp[2], pp[3]));
+                return (pp[0] & pp[1]) & (pp[2] & pp[3]);
+            };
+            if (exact) {
+                uint32_t all = 0xFFFFFFFFu;
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    float p[8];
+                    load8(h, p);
+                    const F2 nisb = F2::dup(-a.inv_sqrt_bc2 * 0x1p-50f), eps = F2::dup(a.eps), lr = F2::dup(a.step_size * 0x1p-64f);
+#pragma unroll
+                    for (int k = 0; k < 4; ++k) {
+                        const int j = 4 * h + k;
+                        const F2 den = fma2(neg_sqrt2(mul2(vh[j], F2::dup(-0x1p100f))), nisb, eps);
+                        const F2 nq = neg_div2(mul2(mh[j], F2::dup(0x1p64f)), den);
+                        F2 pj = F2::pack(p[2 * k], p[2 * k + 1]);
+                        pj = fma2(lr, nq, DECAY ? mul2(pj, F2::dup(a.decay)) : pj);
+                        p[2 * k] = pj.lo();
+                        p[2 * k + 1] = pj.hi();
+                    }
+                    all &= store8(h, p);
+                }
+                if (__any_sync(0xffffffffu, (~all & 0x20002000u) != 0u)) {
+                    uint32_t least = 0x7FFFu;                         // of the patterns stored, signs off
+#pragma unroll 1
+                    for (int i = 0; i < EPT16; ++i)
+                        least = min(least, reinterpret_cast<const unsigned short*>(pt)[EPT16 * tid + i] & 0x7FFFu);
+                    exact = !__any_sync(0xffffffffu, least < 0x1800u);        // 2^-79: no result below 2^-80 was rounded up to it
+                }
+            }
+            if (!exact) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    float p[8];
+                    load8(h, p);
+#pragma unroll
+                    for (int k = 0; k < 8; ++k) {
+                        const int i = 8 * h + k;
+                        const float den = __fmaf_rn(__fsqrt_rn(vh_at(i)), a.inv_sqrt_bc2, a.eps);
+                        p[k] = __fmaf_rn(-a.step_size, __fdiv_rn(mh_at(i), den), DECAY ? p[k] * a.decay : p[k]);
+                    }
+                    store8(h, p);
+                }
             }
         }
     }

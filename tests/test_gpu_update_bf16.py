@@ -1,0 +1,52 @@
+"""bf16 parameters: the update that is taken by approximations and kept only where it rounds to the same pattern from both ends
+of its error, against the general kernel's IEEE operations, bit for bit: rates that put many results next to a rounding boundary,
+parameters of zero, from 2 up, infinite and NaN, subnormal second moments under a small eps, rates of zero and near the
+smallest number."""
+import pytest
+import torch
+
+pytestmark = pytest.mark.gpu
+
+
+def _params(kind, n, gen):
+    p = torch.randn(n, generator=gen) * 0.02
+    if kind == "zero":
+        p.zero_()
+    elif kind == "large":
+        p *= 200.0
+    elif kind == "special":
+        p[::7] = float("nan")
+        p[3::11] = float("inf")
+        p[5::13] = -float("inf")
+        p[1::17] = 3.0e38
+    elif kind == "tiny":
+        p *= 2.0 ** -100
+    return p.bfloat16()
+
+
+@pytest.mark.parametrize("sr", [0, 1])
+@pytest.mark.parametrize("lr,eps", [(2e-5, 1e-8), (1e-3, 1e-8), (0.3, 1e-8), (0.3, 1e-12), (0.0, 1e-8), (2.0 ** -120, 1e-8), (1e-3, 1.0)])
+@pytest.mark.parametrize("kind", ["normal", "zero", "large", "special", "tiny"])
+def test_patterns_are_the_ieee_updates(kind, lr, eps, sr):
+    from paper_2505_00347_b200 import binding as B
+    n = 2048 * 64
+    for bits_m, bits_v, block, scale in ((2, 2, 128, 1e-3), (8, 8, 2048, 1e-3), (4, 3, 64, 2.0 ** -64)):
+        gen = torch.Generator().manual_seed(21)
+        p0 = _params(kind, n, gen)
+        grads = [(torch.randn(n, generator=gen) * scale).bfloat16().cuda() for _ in range(3)]
+        h = B.hyper(lr=lr, beta1=0.5, eps=eps, weight_decay=0.01, seed=2, param_dtype=1, param_round=sr)
+        got = []
+        for policy in (1, 3):
+            p = p0.cuda()
+            state = B.State(n, bits_m, bits_v, block)
+            B.set_kernel_policy(policy)
+            try:
+                for t, g in enumerate(grads, 1):
+                    B.solo_step(p, g, state, h, t)
+            finally:
+                B.set_kernel_policy(0)
+            got.append(p.view(torch.int16).cpu())
+            state.destroy()
+        nan = [(x.int() & 0x7FFF) > 0x7F80 for x in got]
+        assert torch.equal(nan[0], nan[1])
+        assert torch.equal(got[0][~nan[0]], got[1][~nan[1]])
