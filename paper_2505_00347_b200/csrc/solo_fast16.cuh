@@ -1005,12 +1005,16 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
         }
     } else {
         const uint4* const sp = reinterpret_cast<const uint4*>(st.p) + 2 * tid;
-        // An update by approximations is within 3.8 * 2^-23 of the IEEE operations' (the square root 2^-23, five roundings, a
-        // subnormal v^ that is taken as zero 2^-25).  Made smaller and larger by 5 * 2^-23 and rounded to bf16, both results are
-        // the same pattern but for one element in 65536 or fewer, whose result lies next to a rounding boundary; and then the IEEE
-        // update's too, every operation on the way being monotone.  A warp with an element of the other kind, and values or
-        // hyper-parameters out of these ranges, go the long way below.  (LLaMA layer, 2/2 bit: the long way for all 689 us, this 624.)
-        // Where updates are as large as the parameters one warp in ten has such an element.  Rounding to nearest, which costs less to
+        // An update by approximations is within 5.25 * 2^-23 of the IEEE operations': the square root and the reciprocal 2^-23 each, the
+        // denominator's, the first quotient's and the last rounding 2^-24 each, the same of the IEEE square root, denominator and quotient,
+        // a subnormal v^ that is taken as zero 2^-25.  The residual step takes the reciprocal's error and the first quotient's out
+        // again (then 3.75), but not where the remainder is near the smallest subnormal number: |m^| below 2^-126.  Made smaller and larger
+        // by 6 * 2^-23 (5.5 are left after the factors' own roundings) and rounded to bf16, both results are the same pattern unless
+        // a rounding boundary lies between them; and then the IEEE update's too, every operation on the way being monotone.  A boundary lies
+        // there for 1.8e-4 to 3.7e-4 times |update / result| of the elements: one warp (512 elements) in some eight where updates are as large as the
+        // parameters, in some ten thousand where they are a thousandth of them.  Such a warp, and values or hyper-parameters out of
+        // these ranges, go the long way below.  (LLaMA layer, 2/2 bit: the long way for all 689 us, this 624.)
+        // Where updates are as large as the parameters, rounding to nearest, which costs less to
         // begin with, then loses (3/3 bit, mixed gradients: up to 17 %), and so does a codebook that decodes small moments as zero:
         // stochastic rounding with the logarithmic levels only.  Of blocks of 128 and 2048: where it is not taken its registers cost
         // something all the same, rounded to nearest 2 to 8 % with blocks of 64, 1 to 4 % with 256, at most 1.5 % with 128.
@@ -1028,7 +1032,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
             }
             if (__all_sync(0xffffffffu, usual)) {
                 const F2 isb = F2::dup(a.inv_sqrt_bc2), eps = F2::dup(a.eps), decay = F2::dup(a.decay);
-                const F2 lr_lo = F2::dup(a.step_size * (1.0f - 0x1.4p-21f)), lr_hi = F2::dup(a.step_size * (1.0f + 0x1.4p-21f));
+                const F2 lr_lo = F2::dup(a.step_size * (1.0f - 0x1.8p-21f)), lr_hi = F2::dup(a.step_size * (1.0f + 0x1.8p-21f));
                 uint32_t differ = 0u, all = 0xFFFFFFFFu, some = 0u;
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {

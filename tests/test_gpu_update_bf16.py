@@ -1,7 +1,7 @@
 """bf16 parameters: the update that is taken by approximations and kept only where it rounds to the same pattern from both ends
 of its error, against the general kernel's IEEE operations, bit for bit: rates that put many results next to a rounding boundary,
-parameters of zero, from 2 up, infinite and NaN, subnormal second moments under a small eps, rates of zero and near the
-smallest number."""
+parameters of zero, from 2 up, infinite and NaN, rates of zero and near the smallest number; then first and second moments near
+and below the smallest normal number under a small eps."""
 import pytest
 import torch
 
@@ -50,3 +50,34 @@ def test_patterns_are_the_ieee_updates(kind, lr, eps, sr):
         nan = [(x.int() & 0x7FFF) > 0x7F80 for x in got]
         assert torch.equal(nan[0], nan[1])
         assert torch.equal(got[0][~nan[0]], got[1][~nan[1]])
+
+
+@pytest.mark.parametrize("kind", ["normal", "zero", "tiny"])
+@pytest.mark.parametrize("lr", [1e-3, 0.3, 2.0 ** 18])
+@pytest.mark.parametrize("exponent", [-59, -64, -126])
+@pytest.mark.parametrize("bits_m,bits_v,block,round_m", [(2, 2, 128, 0), (8, 8, 2048, 0), (3, 3, 128, 1), (4, 2, 2048, 1)])
+def test_patterns_where_moments_are_subnormal(bits_m, bits_v, block, round_m, exponent, lr, kind):
+    """Blocks whose update is tried by approximations (128 and 2048; plain and Eq. 5).  Gradients of 2^-59: second moments around
+    2^-128, whose root times 31.6, the first step's bias correction, is 2^-19 of eps = 1e-12, far more than the bracket is wide.
+    2^-64: some 2^-138.  2^-126: first moments whose division leaves remainders below the smallest subnormal number; a rate of
+    2^18 lifts the quotients to where they are not looked at again."""
+    from paper_2505_00347_b200 import binding as B
+    n = 2048 * 64
+    gen = torch.Generator().manual_seed(22)
+    p0 = _params(kind, n, gen)
+    grads = [(torch.randn(n, generator=gen) * 2.0 ** exponent).bfloat16().cuda() for _ in range(3)]
+    h = B.hyper(lr=lr, beta1=0.5, eps=1e-12, weight_decay=0.0, seed=2, param_dtype=1, param_round=1, round_m=round_m)
+    got = []
+    for policy in (1, 3):
+        p = p0.cuda()
+        state = B.State(n, bits_m, bits_v, block)
+        B.set_kernel_policy(policy)
+        try:
+            for t, g in enumerate(grads, 1):
+                B.solo_step(p, g, state, h, t)
+        finally:
+            B.set_kernel_policy(0)
+        got.append([p.view(torch.int16).cpu()] + [state.raw_get(k) for k in ("codes_m", "codes_v", "scale_m", "scale_v", "alpha")])
+        state.destroy()
+    for a, b in zip(*got):
+        assert torch.equal(a, b)
