@@ -1020,7 +1020,12 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
         // something all the same, rounded to nearest 2 to 8 % with blocks of 64, 1 to 4 % with 256, at most 1.5 % with 128.
         // A quotient below 2^-126 is rounded otherwise than in the IEEE update, which shows in results below 2^-99 |step_size| <=
         // 2^-80 only (in others it is lost against the parameter).
-        bool done = false;
+        // A thread whose first moments are all zero has exact results on every way (quotients of zero, with the sign of the IEEE
+        // ones) and is not looked at for small ones: rows of zero weights and gradients take one pass, and a warp that has small results of another
+        // kind does not try the pairwise sequence, whose look they would fail as well.  (2^25 weights and gradients of zero, 2/2 bit,
+        // block 128: stochastic, in three passes 313 us, this 104; to nearest 206 and 100.)
+        const bool moves = mx_m_f != 0.0f;
+        bool done = false, small = false;
         if (BRACKET && a.param_sr) {
             bool usual = tmx_v < 0x4D000000u && mx_m_f < 0x1p20f && a.eps < 0x1p30f && a.inv_sqrt_bc2 < 0x1p30f &&
                          (a.step_size == 0.0f || fabsf(a.step_size) > 0x1p-100f) && fabsf(a.step_size) < 0x1p19f;
@@ -1063,15 +1068,16 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
                 }
                 // Results below 2^-63 (exponent bit 6 is set from there to 2) and parameters from 2 up are looked at more closely: the
                 // former for subnormal quotients, the latter for NaN, which the short form of the stochastic rounding does not know.
-                done = !__any_sync(0xffffffffu, differ != 0u || (~all & 0x20002000u) != 0u || (some & 0x40004000u) != 0u);
+                done = !__any_sync(0xffffffffu, differ != 0u || (moves && (~all & 0x20002000u) != 0u) || (some & 0x40004000u) != 0u);
                 if (!done) {
-                    bool redo = differ != 0u;
+                    bool redo = differ != 0u, tiny = false;
 #pragma unroll 1
                     for (int i = 0; i < EPT16; ++i) {
-                        redo |= (reinterpret_cast<const unsigned short*>(pt)[EPT16 * tid + i] & 0x7FFFu) < 0x1800u;
+                        tiny |= (reinterpret_cast<const unsigned short*>(pt)[EPT16 * tid + i] & 0x7FFFu) < 0x1800u;
                         redo |= (reinterpret_cast<const unsigned short*>(st.p)[EPT16 * tid + i] & 0x7FFFu) > 0x7F80u;
                     }
-                    done = !__any_sync(0xffffffffu, redo);
+                    small = __any_sync(0xffffffffu, moves && tiny);
+                    done = !small && !__any_sync(0xffffffffu, redo);
                 }
             }
         }
@@ -1084,7 +1090,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
             // from 2^-63 to 2 (one operation per four of them), whatever lacks it is compared.  The two passes one after the other,
             // and not two sides of a branch per half: LLaMA layer, 2/2 bit, 757 -> 716 us (one loop around both 747, and 2/2 bit with Eq. 5
             // spilled: 659 -> 723 us on 2^27 elements, as it is 646).
-            bool exact = __all_sync(0xffffffffu, tmx_v < 0x4D000000u && mx_m_f < 0x1p20f && a.eps < 0x1p30f && a.inv_sqrt_bc2 < 0x1p30f &&
+            bool exact = !small && __all_sync(0xffffffffu, tmx_v < 0x4D000000u && mx_m_f < 0x1p20f && a.eps < 0x1p30f && a.inv_sqrt_bc2 < 0x1p30f &&
                                                      fabsf(a.step_size) > 0x1p-40f && fabsf(a.step_size) < 0x1p19f);
             auto load8 = [&](int h, float (&p)[8]) {
                 const uint4 pw = sp[(uint32_t)h ^ sw];
@@ -1133,12 +1139,12 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
                     }
                     all &= store8(h, p);
                 }
-                if (__any_sync(0xffffffffu, (~all & 0x20002000u) != 0u)) {
+                if (__any_sync(0xffffffffu, moves && (~all & 0x20002000u) != 0u)) {
                     uint32_t least = 0x7FFFu;                         // of the patterns stored, signs off
 #pragma unroll 1
                     for (int i = 0; i < EPT16; ++i)
                         least = min(least, reinterpret_cast<const unsigned short*>(pt)[EPT16 * tid + i] & 0x7FFFu);
-                    exact = !__any_sync(0xffffffffu, least < 0x1800u);        // 2^-79: no result below 2^-80 was rounded up to it
+                    exact = !__any_sync(0xffffffffu, moves && least < 0x1800u);        // 2^-79: no result below 2^-80 was rounded up to it
                 }
             }
             if (!exact) {

@@ -81,3 +81,42 @@ def test_patterns_where_moments_are_subnormal(bits_m, bits_v, block, round_m, ex
         state.destroy()
     for a, b in zip(*got):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("sr", [0, 1])
+@pytest.mark.parametrize("lr", [1e-3, -0.3, 0.0])
+@pytest.mark.parametrize("bits_m,bits_v,block,hk", [(2, 2, 128, {}), (8, 8, 2048, {}), (3, 3, 128, dict(round_m=1)), (4, 2, 256, dict(belief=1)),
+                                                    (4, 3, 64, dict(v_codebook=3))])
+def test_zero_moments(bits_m, bits_v, block, hk, lr, sr):
+    """Rows without gradient (padding, masked weights): their results are not looked at for being small.  Zeros of both signs among the
+    gradients, the moments and the weights, weights of every size, whole warps of them, single threads and single elements."""
+    from paper_2505_00347_b200 import binding as B
+    n = 2048 * 32
+    gen = torch.Generator().manual_seed(23)
+    w = torch.randn(n, generator=gen) * torch.exp2(torch.randint(-148, 3, (n // 16,), generator=gen).float()).repeat_interleave(16)
+    w[torch.rand(n, generator=gen) < 0.3] = 0.0
+    w[2048 * 8:2048 * 16] = 0.0
+    w[torch.rand(n, generator=gen) < 0.3] *= -1.0
+    w[::4099] = float("inf")
+    p0 = w.bfloat16()
+    runs = torch.rand(n // 16, generator=gen).repeat_interleave(16) < torch.tensor([0.0, 0.5, 0.95, 0.0]).repeat_interleave(n // 4)
+    grads = []
+    for _ in range(3):
+        g = torch.randn(n, generator=gen) * 1e-3
+        g[~runs] = 0.0
+        g[torch.rand(n, generator=gen) < 0.1] = 0.0
+        grads.append(torch.where(torch.rand(n, generator=gen) < 0.5, g, -g).bfloat16().cuda())
+    h = B.hyper(lr=lr, beta1=0.5, weight_decay=0.01, seed=2, param_dtype=1, param_round=sr, **hk)
+    got = []
+    for policy in (1, 3):
+        p = p0.cuda()
+        state = B.State(n, bits_m, bits_v, block)
+        B.set_kernel_policy(policy)
+        try:
+            for t, g in enumerate(grads, 1):
+                B.solo_step(p, g, state, h, t)
+        finally:
+            B.set_kernel_policy(0)
+        got.append(p.view(torch.int16).cpu())
+        state.destroy()
+    assert torch.equal(*got)
