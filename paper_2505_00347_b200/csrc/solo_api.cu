@@ -278,7 +278,7 @@ int launch_step(solo_state* s, StepArgs& a, int64_t full, cudaStream_t stream) {
         large = full >= (w8 ? 1664 + 2 * rest : 2048 + 6 * rest);
     }
     if (fast_ok && ((policy == 0 && large) || policy == 3))
-        k16 = solo::fast16_kernel(s->bits_m, s->bits_v, s->block, a.param_bf16 != 0, modes);
+        k16 = solo::fast16_kernel(s->bits_m, s->bits_v, s->block, a.param_bf16 != 0, a.param_sr != 0, modes);
     if (k16) {
         // Three tiles per CTA once every resident CTA has some eight shares to take over in turn, fewer below: with
         // 8192 tiles one per CTA 55 us, three 59 us; with 395,000 (LLaMA layers) one 2172 us, three 2110 us, eight 2223 us.

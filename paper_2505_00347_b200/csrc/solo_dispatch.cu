@@ -40,13 +40,13 @@ StepKernel fast_tails_kernel(int bits_m, int bits_v, int block, bool param_bf16)
     }
 }
 
-StepKernel fast16_kernel(int bits_m, int bits_v, int block, bool param_bf16, int modes) {
-#define SOLO_PICK16(G, W8)                                                                    \
-    (modes == 0 ? fast16_kernel_g##G##_m0##W8(bits_m, bits_v, param_bf16)                     \
-     : modes == 1 ? fast16_kernel_g##G##_m1##W8(bits_m, bits_v, param_bf16)                   \
-     : modes == 2 ? fast16_kernel_g##G##_m2##W8(bits_m, bits_v, param_bf16)                   \
-     : modes == 3 ? fast16_kernel_g##G##_m3##W8(bits_m, bits_v, param_bf16)                   \
-                  : fast16_kernel_g##G##_m4##W8(bits_m, bits_v, param_bf16))
+StepKernel fast16_kernel(int bits_m, int bits_v, int block, bool param_bf16, bool param_sr, int modes) {
+#define SOLO_PICK16(G, W8)                                                            \
+    (modes == 0 ? fast16_kernel_g##G##_m0##W8(bits_m, bits_v, param_bf16, param_sr)   \
+     : modes == 1 ? fast16_kernel_g##G##_m1##W8(bits_m, bits_v, param_bf16, param_sr) \
+     : modes == 2 ? fast16_kernel_g##G##_m2##W8(bits_m, bits_v, param_bf16, param_sr) \
+     : modes == 3 ? fast16_kernel_g##G##_m3##W8(bits_m, bits_v, param_bf16, param_sr) \
+                  : fast16_kernel_g##G##_m4##W8(bits_m, bits_v, param_bf16, param_sr))
     const bool w8 = bits_m == 8 || bits_v == 8;
     switch (block) {
         case 64: return w8 ? SOLO_PICK16(4, _w8) : SOLO_PICK16(4, );

@@ -46,30 +46,33 @@ StepKernel fast_kernel(int bits_m, int bits_v, int block, bool param_bf16, bool 
 StepKernel fast_tails_kernel(int bits_m, int bits_v, int block, bool param_bf16);
 // Sixteen elements per thread: fp32 or bf16 parameters; `modes`: 0 as `plain` for
 // fast_kernel, 1 the modes fast_kernel reads at run time, 3 `plain` with Eq. 5 rounding, 4 `plain` with a baseline second-moment
-// codebook (StepArgs::tables_v set), 2 any of these together; full tiles
+// codebook (StepArgs::tables_v set), 2 any of these together; `param_sr`: bf16 parameters are rounded stochastically, which blocks
+// of 128 and 2048 have kernels of their own for with modes 0 and 3 (ROUNDING_INSTANCES); full tiles
 // of aligned tensors only (the rest is left to a launch of the streamlined or of the general kernel with
 // StepArgs::only_partial).  Launched with CTA16 = 128 threads.
 // Null / 0 for other block sizes.  One translation unit per block size, set of modes and group of widths.
 constexpr int CTA16 = 128;         // threads per CTA of that kernel
-#define SOLO_DECLARE16(G)                                                             \
-    StepKernel fast16_kernel_g##G##_m0(int bits_m, int bits_v, bool param_bf16);      \
-    StepKernel fast16_kernel_g##G##_m1(int bits_m, int bits_v, bool param_bf16);      \
-    StepKernel fast16_kernel_g##G##_m2(int bits_m, int bits_v, bool param_bf16);      \
-    StepKernel fast16_kernel_g##G##_m3(int bits_m, int bits_v, bool param_bf16);      \
-    StepKernel fast16_kernel_g##G##_m4(int bits_m, int bits_v, bool param_bf16);      \
-    StepKernel fast16_kernel_g##G##_m0_w8(int bits_m, int bits_v, bool param_bf16);   \
-    StepKernel fast16_kernel_g##G##_m1_w8(int bits_m, int bits_v, bool param_bf16);   \
-    StepKernel fast16_kernel_g##G##_m2_w8(int bits_m, int bits_v, bool param_bf16);   \
-    StepKernel fast16_kernel_g##G##_m3_w8(int bits_m, int bits_v, bool param_bf16);   \
-    StepKernel fast16_kernel_g##G##_m4_w8(int bits_m, int bits_v, bool param_bf16);   \
-    size_t fast16_smem_g##G(int bits_m, int bits_v, bool param_bf16);                 \
+template <int G, int MODES>        // G: lanes per block
+constexpr bool ROUNDING_INSTANCES = (MODES == 0 || MODES == 3) && (G == 8 || G == 128);
+#define SOLO_DECLARE16(G)                                                                          \
+    StepKernel fast16_kernel_g##G##_m0(int bits_m, int bits_v, bool param_bf16, bool param_sr);    \
+    StepKernel fast16_kernel_g##G##_m1(int bits_m, int bits_v, bool param_bf16, bool param_sr);    \
+    StepKernel fast16_kernel_g##G##_m2(int bits_m, int bits_v, bool param_bf16, bool param_sr);    \
+    StepKernel fast16_kernel_g##G##_m3(int bits_m, int bits_v, bool param_bf16, bool param_sr);    \
+    StepKernel fast16_kernel_g##G##_m4(int bits_m, int bits_v, bool param_bf16, bool param_sr);    \
+    StepKernel fast16_kernel_g##G##_m0_w8(int bits_m, int bits_v, bool param_bf16, bool param_sr); \
+    StepKernel fast16_kernel_g##G##_m1_w8(int bits_m, int bits_v, bool param_bf16, bool param_sr); \
+    StepKernel fast16_kernel_g##G##_m2_w8(int bits_m, int bits_v, bool param_bf16, bool param_sr); \
+    StepKernel fast16_kernel_g##G##_m3_w8(int bits_m, int bits_v, bool param_bf16, bool param_sr); \
+    StepKernel fast16_kernel_g##G##_m4_w8(int bits_m, int bits_v, bool param_bf16, bool param_sr); \
+    size_t fast16_smem_g##G(int bits_m, int bits_v, bool param_bf16);                              \
     size_t fast16_smem_g##G##_w8(int bits_m, int bits_v, bool param_bf16);
 SOLO_DECLARE16(4)
 SOLO_DECLARE16(8)
 SOLO_DECLARE16(16)
 SOLO_DECLARE16(128)
 #undef SOLO_DECLARE16
-StepKernel fast16_kernel(int bits_m, int bits_v, int block, bool param_bf16, int modes);
+StepKernel fast16_kernel(int bits_m, int bits_v, int block, bool param_bf16, bool param_sr, int modes);
 size_t fast16_kernel_smem(int bits_m, int bits_v, int block, bool param_bf16);
 // Dynamic shared memory the streamlined kernel for these widths is launched with.
 size_t fast_kernel_smem(int bits_m, int bits_v);

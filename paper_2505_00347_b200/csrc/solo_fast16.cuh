@@ -741,7 +741,7 @@ __device__ __forceinline__ void block_scalars16(const StepArgs& a, Shared& s, co
 // at a time; (C) the first moment's scale and codes (each thread divides for itself: the scale is
 // known to all eight lanes after the maximum); (D) the sorted lists and the selection rounds; (E) the
 // exchange with the first warp, the thread's two Philox blocks meanwhile, the second moment's codes, the stores.
-template <int BM, int BV, bool PBF, int G, bool DECAY, int MODES>
+template <int BM, int BV, bool PBF, int G, bool DECAY, int MODES, bool SR>
 __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, BV, PBF, G>& s, const float* s_y, const float* s_mid,
                                             const float4* s_mid4, const float* s_yv, const float4* s_nv,
                                             const float2* s_yg, const float4* s_br,
@@ -755,7 +755,9 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     // p-quantile, xi drawn), with Eq. 5 (MODES 3) or a baseline codebook (MODES 4) or without; the other
     // instantiations read these modes from the arguments, MODES 2 also Eq. 5 and the baseline codebooks
     constexpr bool PLAIN = MODES == 0 || MODES >= 3;
-    constexpr bool BRACKET = (MODES == 0 || MODES == 3) && (G == 8 || G == 128);    // see the update of bf16 parameters
+    // bf16 parameters: how they are rounded is a property of the instantiation where the update is tried by approximations (see there)
+    constexpr bool BY_ROUNDING = PBF && ROUNDING_INSTANCES<G, MODES>;
+    static_assert(BY_ROUNDING || !SR, "other instantiations read it from the arguments");
     const bool l2 = !PLAIN && a.l2, belief = !PLAIN && a.belief;
     // baseline codebook for the second moment: levels s_yv, nearest level by the midpoints in s_nv
     const bool vtab = MODES == 4 || (MODES == 2 && a.tables_v != nullptr);
@@ -1016,17 +1018,19 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
         // these ranges, go the long way below.  (LLaMA layer, 2/2 bit: the long way for all 689 us, this 624.)
         // Where updates are as large as the parameters, rounding to nearest, which costs less to
         // begin with, then loses (3/3 bit, mixed gradients: up to 17 %), and so does a codebook that decodes small moments as zero:
-        // stochastic rounding with the logarithmic levels only.  Of blocks of 128 and 2048: where it is not taken its registers cost
-        // something all the same, rounded to nearest 2 to 8 % with blocks of 64, 1 to 4 % with 256, at most 1.5 % with 128.
+        // stochastic rounding with the logarithmic levels only, and of blocks of 128 and 2048, which have a kernel per rounding: one kernel
+        // for both spilled 108 bytes a thread instead of 24 (nearest) and 48 (2/3 bit, block 128) and cost rounding to nearest up to 4 %
+        // (2^25 elements, 3/4 bit, block 128: 124.3 us; without the bracket 119.5, this 116.9).  Blocks of 64 and 256 have one kernel for both
+        // without the bracket, whose registers cost rounding to nearest 2 to 8 % and 1 to 4 % there.
         // A quotient below 2^-126 is rounded otherwise than in the IEEE update, which shows in results below 2^-99 |step_size| <=
         // 2^-80 only (in others it is lost against the parameter).
         // A thread whose first moments are all zero has exact results on every way (quotients of zero, with the sign of the IEEE
-        // ones) and is not looked at for small ones: rows of zero weights and gradients take one pass, and a warp that has small results of another
+        // ones) and is not looked at for small ones: rows of zero weights and gradients take one pass.  A warp that has small results of another
         // kind does not try the pairwise sequence, whose look they would fail as well.  (2^25 weights and gradients of zero, 2/2 bit,
         // block 128: stochastic, in three passes 313 us, this 104; to nearest 206 and 100.)
-        const bool moves = mx_m_f != 0.0f;
+        const bool moves = !BY_ROUNDING || mx_m_f != 0.0f;
         bool done = false, small = false;
-        if (BRACKET && a.param_sr) {
+        if (SR) {
             bool usual = tmx_v < 0x4D000000u && mx_m_f < 0x1p20f && a.eps < 0x1p30f && a.inv_sqrt_bc2 < 0x1p30f &&
                          (a.step_size == 0.0f || fabsf(a.step_size) > 0x1p-100f) && fabsf(a.step_size) < 0x1p19f;
             if (a.eps < a.inv_sqrt_bc2 * 0x1p-38f) {                  // (a subnormal v^ would show)
@@ -1104,7 +1108,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
             auto store8 = [&](int h, const float (&p)[8]) {             // returns the conjunction of the patterns
                 const uint32_t he = (uint32_t)h ^ sw;
                 uint32_t pp[4];
-                if (a.param_sr) {
+                if (BY_ROUNDING ? SR : a.param_sr) {
                     uint32_t wp[4];
                     draw8(he, 2u, wp);
 #pragma unroll
@@ -1595,7 +1599,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     store_codes16<BV>(a.codes_v + jb_tile * (2 * G * BV), s.cout[(BM == 3 && BV == 3) ? 1 : 0][BV == 3 ? warp : 0], tid, ov_e);
 }
 
-template <int BM, int BV, bool PBF, int G, int MODES>
+template <int BM, int BV, bool PBF, int G, int MODES, bool SR>
 __global__ void __launch_bounds__(CTA16, ctas16<BM, BV, G, MODES>()) solo_step_fast16_kernel(const __grid_constant__ StepArgs a) {
     constexpr int KM = 1 << BM;
     constexpr bool EXT = MODES >= 2, EQ5 = MODES == 2 || MODES == 3;
@@ -1714,9 +1718,9 @@ __global__ void __launch_bounds__(CTA16, ctas16<BM, BV, G, MODES>()) solo_step_f
     const bool decay = a.decay != 1.0f;
     for (; s.desc[fill & 1u].valid; ++fill) {
         if (decay)
-            fast16_tile<BM, BV, PBF, G, true, MODES>(a, s, s_y, s_mid, s_mid4, s_yv, s_nv, s_yg, s_br, fill, failed);
+            fast16_tile<BM, BV, PBF, G, true, MODES, SR>(a, s, s_y, s_mid, s_mid4, s_yv, s_nv, s_yg, s_br, fill, failed);
         else
-            fast16_tile<BM, BV, PBF, G, false, MODES>(a, s, s_y, s_mid, s_mid4, s_yv, s_nv, s_yg, s_br, fill, failed);
+            fast16_tile<BM, BV, PBF, G, false, MODES, SR>(a, s, s_y, s_mid, s_mid4, s_yv, s_nv, s_yg, s_br, fill, failed);
     }
     // A thread that gave up on a copy waits once more, again bounded, for the last one that was issued,
     // so that no copy is still writing to the stage when the CTA's shared memory is released; likewise for an answer.

@@ -22,8 +22,10 @@
 
 namespace solo {
 
-#define SOLO_K16(BM, BV) \
-    (param_bf16 ? solo_step_fast16_kernel<BM, BV, true, SOLO_G, SOLO_MODES> : solo_step_fast16_kernel<BM, BV, false, SOLO_G, SOLO_MODES>)
+#define SOLO_K16(BM, BV)                                                                                             \
+    (!param_bf16 ? solo_step_fast16_kernel<BM, BV, false, SOLO_G, SOLO_MODES, false>                                 \
+     : param_sr  ? solo_step_fast16_kernel<BM, BV, true, SOLO_G, SOLO_MODES, ROUNDING_INSTANCES<SOLO_G, SOLO_MODES>> \
+                 : solo_step_fast16_kernel<BM, BV, true, SOLO_G, SOLO_MODES, false>)
 #define SOLO_S16(BM, BV) \
     (param_bf16 ? sizeof(Fast16Shared<BM, BV, true, SOLO_G>) : sizeof(Fast16Shared<BM, BV, false, SOLO_G>))
 
@@ -35,7 +37,7 @@ namespace solo {
 #define SOLO_NAME(stem) stem
 #endif
 
-StepKernel SOLO_NAME(SOLO_CAT4(fast16_kernel_g, SOLO_G, _m, SOLO_MODES))(int bits_m, int bits_v, bool param_bf16) {
+StepKernel SOLO_NAME(SOLO_CAT4(fast16_kernel_g, SOLO_G, _m, SOLO_MODES))(int bits_m, int bits_v, bool param_bf16, bool param_sr) {
     switch (bits_m * 10 + bits_v) {
 #define SOLO_CASE(BM, BV) case BM * 10 + BV: return SOLO_K16(BM, BV);
         SOLO_WIDTHS(SOLO_CASE)
