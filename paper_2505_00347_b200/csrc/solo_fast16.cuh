@@ -63,7 +63,7 @@ constexpr int ctas16() { return BM == 8 || BV == 8 ? (MODES >= 2 ? 6 : 7) : BM =
 
 // What the first rounds of Philox4x32-10 leave of the counter's words that are the same for a whole tile: (position, high word,
 // step, 4 * stream) differ in the position's low word only, which reaches half of the second round and all of the third.
-// Computed per tensor by the thread that walks (draw_keys): a call is 16 wide multiplications instead of 20, and no thread looks up its
+// Computed per tensor by the thread that walks (draw_keys): a call is 18 wide multiplications instead of 20, and no thread looks up its
 // tensor's stream (2^26 elements: 2/3 bit 183.5 -> 181.7 us, bf16 parameters stochastically rounded 240 -> 236).
 struct DrawKeys {
     uint32_t k2, k3, k4, k6;
@@ -97,6 +97,15 @@ __device__ __forceinline__ void philox_keys(uint32_t c0, const DrawKeys& k, uint
     }
     out[0] = c0; out[1] = c1; out[2] = c2; out[3] = c3;
 }
+
+// Which kernels take a tile's keys from its description; the others draw from the counters as they are.  Blocks of 64: the keys
+// gain nothing there (2^24 elements, fp32: 1.00) and cost the modes that are read from the arguments 2 to 3 %.  Modes read from the
+// arguments with bf16 parameters, blocks of 128 and 256: the keys cost steps with a fixed base, which have little else to do, up to 4 %
+// (2^25 elements, block 128, 8/4 bit 105.2 us, without 100.1, 3/4 bit 108.0 and 103.6) and the other modes up to 3 % (AdaBelief, 2/2 bit
+// 117.0 and 113.5; 2/3 bit alone is faster with them, 120.0 and 122.1).  But with 4-bit first moments the kernel spills more without
+// (4/2 bit, fixed base, 99.6 and 104.3), and blocks of 2048 are 2 to 5 % slower without.
+template <int BM, bool PBF, int G, int MODES>
+constexpr bool DRAW_KEYS = G != 4 && !(PBF && MODES == 1 && BM != 4 && G <= 16);
 
 // G: lanes per block (4, 8, 16 or 128 for blocks of 64, 128, 256 or 2048 elements); NG = 128 / G blocks per tile.
 template <int BM, int BV, bool PBF, int G>
@@ -156,9 +165,7 @@ struct Fast16Shared {
     // The CTA's walk over the tiles (see produce_tile16): kept here and not in registers, because one thread uses it
     alignas(8) unsigned long long mbar_steal;
     alignas(16) uint4 steal;                 // answer of the last request for another CTA's tiles
-    // Blocks of 64 draw from the counters as they are: the keys gain nothing there (2^24 elements, fp32: 1.00) and cost the modes that
-    // are read from the arguments 2 to 3 %.
-    static constexpr bool KEYS = G != 4;
+    static constexpr bool KEYS = G != 4;     // some kernel with this layout has DRAW_KEYS
     struct Walk {
         char* p;                             // tensor: its parameters, gradients, first block
         const char* g;
@@ -177,8 +184,8 @@ struct Fast16Shared {
         const char* g;
         int64_t jb;
         int tile, valid;                     // valid 0: no tile left
-        uint32_t ctr, ctr_hi;                // stream position of its first element (element index / 8)
-        uint32_t stream4;
+        uint32_t ctr, ctr_hi;                // stream position of its first element (element index / 8); ctr_hi and
+        uint32_t stream4;                    // stream4 are left out with DRAW_KEYS
         alignas(16) DrawKeys keys[KEYS ? 2 : 1];     // [1]: of the elements behind a change of the high word
     };
     alignas(16) Desc desc[2];                 // written for the next tile between the two barriers of this one
@@ -628,11 +635,11 @@ __device__ __forceinline__ int steal_answer(Shared& s, int* status) {
 // A CTA that waited in vain for a copy ends here: it takes in the answer to its last request, so that nothing writes to its
 // shared memory any more, and asks for no other.  What it then leaves unstepped (and has reported in the status word) is
 // the rest of its share and at most the one that answer brought, however many CTAs have not started yet.
-// DRAWS: the step draws random numbers, so that the tile's Philox keys are wanted.
-template <int BM, int BV, bool PBF, int G, bool DRAWS>
+template <int BM, int BV, bool PBF, int G, int MODES>
 __device__ __forceinline__ void produce_tile16(const StepArgs& a, Fast16Shared<BM, BV, PBF, G>& s, typename Fast16Shared<BM, BV, PBF, G>::Desc& d) {
     using Shared = Fast16Shared<BM, BV, PBF, G>;
     constexpr int NG = CTA16 / G, PSZ = PBF ? 2 : 4;
+    constexpr bool DRAWS = MODES != 4 || PBF, KEYS = DRAW_KEYS<BM, PBF, G, MODES>;
     typename Fast16Shared<BM, BV, PBF, G>::Walk& w = s.walk;
     int tile_end = w.tile_end, tile = w.gave_up ? tile_end : w.tile;
     for (;;) {
@@ -674,7 +681,7 @@ __device__ __forceinline__ void produce_tile16(const StepArgs& a, Fast16Shared<B
                 w.ctr0 = org.ctr0;
                 w.stream4 = org.stream * 4u;
                 w.ctr_hi = (uint32_t)(org.ctr0 >> 32);
-                if constexpr (Shared::KEYS) {
+                if constexpr (KEYS) {
                     w.keys[0] = draw_keys(a.rk, w.ctr_hi, a.step32, w.stream4);
                     w.keys[1] = draw_keys(a.rk, w.ctr_hi + 1u, a.step32, w.stream4);
                 }
@@ -691,7 +698,7 @@ __device__ __forceinline__ void produce_tile16(const StepArgs& a, Fast16Shared<B
     if constexpr (DRAWS) {
         const uint64_t ctr = w.ctr0 + (uint64_t)(uint32_t)tin * (TILE / 8);
         d.ctr = (uint32_t)ctr;
-        if constexpr (Shared::KEYS) {
+        if constexpr (KEYS) {
             if ((uint32_t)(ctr >> 32) != w.ctr_hi) {
                 w.ctr_hi = (uint32_t)(ctr >> 32);
                 w.keys[0] = draw_keys(a.rk, w.ctr_hi, a.step32, w.stream4);
@@ -785,7 +792,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     if (G != 128 && gave_up) {
         if (gl == 0) s.xin[grp] = make_uint4(0u, 0u, 0u, 1u);
         bar_sync16(1);
-        if (tid == 32) produce_tile16<BM, BV, PBF, G, MODES != 4 || PBF>(a, s, s.desc[(fill + 1u) & 1u]);
+        if (tid == 32) produce_tile16<BM, BV, PBF, G, MODES>(a, s, s.desc[(fill + 1u) & 1u]);
         if (tid < NG) block_scalars16<KV>(a, s, jb_tile, tid, fixed_base, vtab);
         bar_sync16(2);
         return;
@@ -957,7 +964,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
         const uint4 m4 = *reinterpret_cast<const uint4*>(c.m), v4 = *reinterpret_cast<const uint4*>(c.v);
         const uint4 l4 = *reinterpret_cast<const uint4*>(c.lo), f4 = *reinterpret_cast<const uint4*>(c.failed);
         if (f4.x | f4.y | f4.z | f4.w) {
-            if (tid == 32) produce_tile16<BM, BV, PBF, G, MODES != 4 || PBF>(a, s, s.desc[(fill + 1u) & 1u]);
+            if (tid == 32) produce_tile16<BM, BV, PBF, G, MODES>(a, s, s.desc[(fill + 1u) & 1u]);
             bar_sync16(2);
             return;
         }
@@ -973,7 +980,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     // elements; a tensor starts at a multiple of eight of them, so that the thread's two share the high word.
     auto draw8 = [&](uint32_t half, uint32_t purpose, uint32_t (&out)[4]) {
         const uint32_t c0 = desc.ctr + 2u * (uint32_t)tid;
-        if constexpr (Shared::KEYS) {
+        if constexpr (DRAW_KEYS<BM, PBF, G, MODES>) {
             const DrawKeys k = desc.keys[c0 < desc.ctr ? 1 : 0];
             philox_keys(c0 + half, k, purpose, a.rk, out);
         } else {
@@ -1441,7 +1448,7 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
     if (gl == 0) s.xin[grp] = make_uint4(mx_m, mx_v, x_p, 0u);
     bar_sync16(1);
     // every thread has read what it needs from the stage
-    if (tid == 32) produce_tile16<BM, BV, PBF, G, MODES != 4 || PBF>(a, s, s.desc[(fill + 1u) & 1u]);
+    if (tid == 32) produce_tile16<BM, BV, PBF, G, MODES>(a, s, s.desc[(fill + 1u) & 1u]);
     if (tid < NG) block_scalars16<KV>(a, s, jb_tile, tid, fixed_base, vtab);
     // meanwhile every thread draws: Philox4x32-10 on the counters of its two groups of eight elements,
     // (ctr, step, 4 * stream) and (ctr + 1, ...), in its own order.  (Between the selection's rounds, where the draws
@@ -1709,7 +1716,7 @@ __global__ void __launch_bounds__(CTA16, ctas16<BM, BV, G, MODES>()) solo_step_f
         s.walk.tile_end = (int)min((int64_t)s.walk.tile + 1 + a.share, a.total_tiles);
         s.walk.tensor = (a.num_tensors > 1 ? find_tensor(a.tile_start, a.num_tensors, s.walk.tile + 1) : 0) - 1;
         steal_request(s);
-        produce_tile16<BM, BV, PBF, G, MODES != 4 || PBF>(a, s, s.desc[0]);
+        produce_tile16<BM, BV, PBF, G, MODES>(a, s, s.desc[0]);
     }
     __syncthreads();
 

@@ -1,7 +1,8 @@
 """A tile whose elements lie on both sides of a change of the stream position's high word (element 2^35 of a tensor, reached by a
 shard of a larger tensor), directly before and behind it.  Blocks of 128 and 256: the sixteen-per-thread kernel computes what the
 counters have in common once per tile, for the high word and for the one after; blocks of 2048 too, but a tile of theirs begins at
-a multiple of its size and so never lies on both sides.  Blocks of 64: every counter as it is, like the general kernel's."""
+a multiple of its size and so never lies on both sides.  Blocks of 64, and bf16 parameters with modes that are read from the
+arguments: every counter as it is, like the general kernel's."""
 import pytest
 import torch
 
@@ -10,7 +11,8 @@ pytestmark = pytest.mark.gpu
 KEYS = ("codes_m", "codes_v", "scale_m", "scale_v", "alpha")
 
 
-@pytest.mark.parametrize("hk", [dict(round_m=1), dict(param_dtype=1, param_round=1), dict(v_codebook=1, param_dtype=1, param_round=1)])
+@pytest.mark.parametrize("hk", [dict(round_m=1), dict(param_dtype=1, param_round=1), dict(v_codebook=1, param_dtype=1, param_round=1),
+                                dict(fixed_alpha=0.5, param_dtype=1, param_round=1), dict(belief=1)])
 @pytest.mark.parametrize("bits_m,bits_v,block,before",       # `before`: elements before element 2^35
                          [(2, 3, 64, b) for b in (0, 64, 1024, 2048 + 192, 4096)] + [(8, 8, 64, b) for b in (0, 64, 1024, 2048 + 192, 4096)] +
                          [(2, 3, 128, b) for b in (0, 128, 1024, 2048 + 256, 4096)] + [(8, 8, 128, b) for b in (128, 4096 + 1920)] +
