@@ -286,6 +286,7 @@ int launch_step(solo_state* s, StepArgs& a, int64_t full, cudaStream_t stream) {
                                  solo::kernel_occupancy(k16, solo::fast16_kernel_smem(s->bits_m, s->bits_v, s->block, a.param_bf16 != 0), solo::CTA16);
         if (resident <= 0) return SOLO_ECUDA;
         a.share = (int32_t)std::min<int64_t>(3, std::max<int64_t>(1, (a.total_tiles - a.tile_first) / (resident * 8)));
+        a.only_partial = 0;       // its selections add this zero to keys (list_drop)
         // full tiles by the sixteen-per-thread kernel, whatever it leaves (tails, tensors that are
         // not 16-byte aligned) by the streamlined kernel, or by the general one where that has no path
         int rc = launch_kernel(k16, a, s->device, solo::CTA16, solo::fast16_kernel_smem(s->bits_m, s->bits_v, s->block, a.param_bf16 != 0), stream);

@@ -42,7 +42,8 @@ struct StepArgs {
     int64_t tile_first;
     int32_t tensor_first, tensor_end;  // those tiles belong to tensors [tensor_first, tensor_end): no other entry of a list is read
     int32_t share;                     // sixteen-per-thread kernel: tiles of one CTA
-    int32_t only_partial;              // streamlined and general kernel: skip full tiles of aligned tensors (another launch did them)
+    int32_t only_partial;              // streamlined and general kernel: skip full tiles of aligned tensors (another launch did them).
+                                       // Sixteen-per-thread kernel: 0, as its compiler does not know; list_drop adds it to keys
     int64_t debug_stall_tile_p1;       // test hook of the staged kernels: 1 + the number of the tile whose input copy
                                        // announces 16 bytes more than it brings (the wait for it runs out); 0: none
     // state

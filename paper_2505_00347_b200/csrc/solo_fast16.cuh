@@ -362,7 +362,7 @@ __device__ __forceinline__ uint32_t lanes_rank(uint32_t x, int rank, int lane) {
 }
 
 // Drops the head of a sorted list if it is at most t and n < rem (`p`, `go`: the same as predicates).  Groups of eight: the entries
-// move up by predicated additions of `zero`, which the compiler does not know: an addition goes to any of the integer pipes at
+// move up by predicated additions of `zero` (StepArgs::only_partial), which the compiler does not know: an addition goes to any of the integer pipes at
 // one warp a cycle, a selection to one that takes a warp every other cycle (2^26 elements, 2/3 bit 186.7 -> 183.5 us, 3/3 bit 204.3 ->
 // 201; bf16 parameters, 2/2 bit, 249 -> 240).  Groups of sixteen and the CTA's selections are faster (4/4 bit 220 us against 232).
 template <int G>
@@ -370,8 +370,8 @@ __device__ __forceinline__ void list_drop(uint32_t (&l)[4], const bool p, const 
                                           const uint32_t zero) {
     if constexpr (G == 8) {
         asm("{\n\t.reg .pred g, p;\n\tsetp.lt.s32 g, %4, %5;\n\tsetp.le.and.u32 p, %0, %6, g;\n\t@p add.u32 %0, %1, %7;\n\t@p add.u32 %1, %2, %7;\n\t"
-            "@p add.u32 %2, %3, %7;\n\t@p add.u32 %3, %7, 0x7FFFFFFF;\n\t}"
-            : "+r"(l[0]), "+r"(l[1]), "+r"(l[2]), "+r"(l[3]) : "r"(n), "r"(rem), "r"(t), "r"(zero));
+            "@p add.u32 %2, %3, %7;\n\t@p add.u32 %3, %7, %8;\n\t}"
+            : "+r"(l[0]), "+r"(l[1]), "+r"(l[2]), "+r"(l[3]) : "r"(n), "r"(rem), "r"(t), "r"(zero), "n"(KEY_MAX));
     } else if (p && go) {
         l[0] = l[1]; l[1] = l[2]; l[2] = l[3]; l[3] = KEY_MAX;
     }
