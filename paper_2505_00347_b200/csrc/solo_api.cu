@@ -257,9 +257,13 @@ int launch_step(solo_state* s, StepArgs& a, int64_t full, cudaStream_t stream) {
     } else if (!streamlined) {
         // Lists, and tensors with a tail, need a second launch: 6 to 10 us after the first.  Here the whole set decides and not the
         // chunk of a host-buffer call, because the general kernel's fp32 parameters differ in the last bits.  Us in one launch of the
-        // general kernel / in two (4/2 bit Eq. 5): full tiles only 256 13.3 / 13.0, 768 24.7 / 18.7; with a tail 512 19.2 / 21.8, 768
-        // 22.6 / 23.7, 1024 29.9 / 25.4 (8-bit dynamic exponent 512 18.0 / 19.3, 768 25.6 / 20.4); blocks of 2048: full tiles
-        // only 768 23.5 / 21.9, with a tail 1536 41.0 / 41.5, 2048 50.9 / 43.1.
+        // general kernel / in two, 4/2 bit Eq. 5, full tiles only: 256 13.2 / 12.5, 320 13.3 / 16.6, 448 20.4 / 16.9; with a tail 640 22.6 / 25.3,
+        // 832 22.9 / 25.6, 896 28.0 / 25.6; 4/4 bit linear without zero 448 12.7 / 12.8, with a tail 832 13.8 / 17.9, 1024 17.5 / 18.3.  8/8 bit
+        // Eq. 5 256 13.6 / 15.0, 320 23.1 / 17.6, with a tail 512 23.3 / 27.2, 640 31.6 / 27.4; dynamic exponent 256 11.2 / 11.8, 320 18.3 / 13.7,
+        // with a tail 512 18.1 / 20.3, 640 25.0 / 20.5.  The general kernel's times go up by the wave: the lines are those of 8-bit
+        // states, 2- to 4-bit ones would have theirs at 448 and 896.  Blocks of 2048, 4/2 bit Eq. 5 (8/8 bit): full tiles only 640
+        // 23.1 / 19.4 (27.5 / 21.2), 768 23.4 / 19.6 (27.9 / 21.3); with a tail 1280 31.9 / 36.2 (38.4 / 41.4), 1536 41.7 / 37.5 (50.2 / 42.1),
+        // 1792 43.0 / 38.0 (51.9 / 46.4).
         const bool others = s->tiles_total != s->full_tiles;
         large = s->full_tiles >= (cta_group ? (others ? 1664 : 768) : (others ? 640 : 320));
     } else if (cta_group) {

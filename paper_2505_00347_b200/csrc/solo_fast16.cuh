@@ -57,7 +57,7 @@ static_assert(CTA16 * EPT16 == TILE, "same tile as the other kernels");
 // and for blocks of 256, which spill more at 64 (2^27 elements: 2/3 bit at block 128 380 us at seven, 367 us at
 // eight; 4/4 bit 422 and 421 us; 4/4 bit at block 256 432 and 434 us).  8-bit states, whose tables fill the shared
 // memory: seven, six where the modes' tables come on top (8/8 bit five 516, six 498, seven 496 us; Eq. 5 four 830, five
-// 799, six 763 us).
+// 799, six 763 us, read from the arguments; Eq. 5 alone and a codebook alone have the same number and were not timed with others).
 template <int BM, int BV, int G, int MODES>
 constexpr int ctas16() { return BM == 8 || BV == 8 ? (MODES >= 2 ? 6 : 7) : BM == 4 || G >= 16 ? 7 : 8; }
 
@@ -1019,9 +1019,9 @@ __device__ __forceinline__ void fast16_tile(const StepArgs& a, Fast16Shared<BM, 
         // a subnormal v^ that is taken as zero 2^-25.  The residual step takes the reciprocal's error and the first quotient's out
         // again (then 3.75), but not where the remainder is near the smallest subnormal number: |m^| below 2^-126.  Made smaller and larger
         // by 6 * 2^-23 (5.5 are left after the factors' own roundings) and rounded to bf16, both results are the same pattern unless
-        // a rounding boundary lies between them; and then the IEEE update's too, every operation on the way being monotone.  A boundary lies
-        // there for 1.8e-4 to 3.7e-4 times |update / result| of the elements: one warp (512 elements) in some eight where updates are as large as the
-        // parameters, in some ten thousand where they are a thousandth of them.  Such a warp, and values or hyper-parameters out of
+        // a rounding boundary lies between them; and then the IEEE update's too, every operation on the way being monotone.  A
+        // boundary lies there for 1.8e-4 to 3.7e-4 times |update / result| of the elements: one warp (512 elements) in some eight where
+        // updates are as large as the parameters, in some ten thousand where they are a thousandth of them.  Such a warp, and values or hyper-parameters out of
         // these ranges, go the long way below.  (LLaMA layer, 2/2 bit: the long way for all 689 us, this 624.)
         // Where updates are as large as the parameters, rounding to nearest, which costs less to
         // begin with, then loses (3/3 bit, mixed gradients: up to 17 %), and so does a codebook that decodes small moments as zero:
